@@ -199,6 +199,15 @@ BATCH_KERNEL_NAMES = {
                      "up to 16 lattices in one launch)",
 }
 TMA_GROUP_MAX = 16      # lattices per shared TMA-fed launch
+# the kernel that runs of steps use where the library reports it (Lattice.two_step)
+TWO_STEP_NAME = "trt::k_step_pair (two fused stream-collide steps per launch{}; single steps at the ends of a run)"
+
+
+def two_step_launches(steps: int, odd: bool) -> int:
+    """Launches of a run of `steps` steps of lattices that advance two steps at a
+    time from odd levels: a single step to an odd level, and one for an odd rest."""
+    first = 0 if odd or steps == 0 else 1
+    return first + (steps - first) // 2 + (steps - first) % 2
 
 
 def kernel_label(mode: str, kinds) -> str:
@@ -636,6 +645,7 @@ def main():
     # the timed region: exactly K steps, back to back (the working set is far
     # larger than L2, so each step's reads come from HBM and the write-back of
     # the previous step's dirty lines is paid inside the region)
+    level = lats[0].t
     local_ms = timed(args.steps)
     barrier()
     # beside it, not part of the value: a steady-state sample of at least 1000
@@ -653,13 +663,17 @@ def main():
     # roofline of the step kernel: algorithmic bytes per launch / mean launch time
     kinds = [lat.step_kernel() for lat in lats]
     per_step_launches = step_launches(args.mode, kinds)
-    launches = args.steps * per_step_launches
+    # lattices that advance two steps per launch share the launches as the single
+    # steps do, and a launch moves the bytes of one state for two steps
+    two = all(lat.two_step() for lat in lats)
+    per_launch = 2 if two else 1
+    launches = per_step_launches * (two_step_launches(args.steps, bool(level & 1)) if two else args.steps)
     launch_s = local_ms / 1e3 / launches
     masked = any(p.mask is not None for p in problems)
     per_launch_bytes = bytes_per_node(storage, args.g_mode, masked) * nodes / per_step_launches
     achieved = per_launch_bytes / launch_s / 1e9
     peak, peak_kind = hbm_peak()
-    steady_gbs = per_launch_bytes * per_step_launches * steady_n / (steady_ms / 1e3) / 1e9
+    steady_gbs = per_launch_bytes * per_step_launches * steady_n / per_launch / (steady_ms / 1e3) / 1e9
     flushed_gbs = per_launch_bytes * per_step_launches * flushed_n / (flushed_ms / 1e3) / 1e9
     traffic = recorded_traffic(f"{args.workload}/{storage}/{args.g_mode}") if args.mode == "batch" else None
 
@@ -706,7 +720,7 @@ def main():
                                  + (" (autotuned)" if args.kernel == "tuned" else ""),
                        "tuning": tuner.measured if args.kernel == "tuned" else None,
                        "parallelism": f"replicas x{world}",
-                       "launch": (f"{per_step_launches} step-kernel launch(es) per time step, "
+                       "launch": (f"{per_step_launches} step-kernel launch(es) per {'two time steps' if two else 'time step'}, "
                                   + ("batched" if args.mode == "batch" else "one lattice each")),
                        "working_set_bytes": working_set,
                        "l2": ("inputs larger than L2: the timed steps run back to back, no flush "
@@ -731,7 +745,8 @@ def main():
             "clocks": clk,
             "fp64_fma_tflops": fp64_tflops,
         }
-        line["roofline"]["kernel"] = kernel_label(args.mode, kinds)
+        line["roofline"]["kernel"] = (TWO_STEP_NAME.format(", all lattices in one launch" if args.mode == "batch" else "")
+                                      if two else kernel_label(args.mode, kinds))
         line["roofline"]["launch_ms"] = launch_s * 1e3
         line["roofline"]["hbm_gbs"] = achieved        # algorithmic bytes / time, every format
         line["roofline"]["frac_of_nominal_hbm"] = achieved / HBM_NOMINAL_GBS

@@ -20,6 +20,7 @@ namespace {
 
 constexpr int kGraphSteps = 32;  // steps per captured graph (even: parity and Phi
                                  // buffers return to their start after a replay)
+constexpr size_t kMaxGraphs = 4;
 
 }  // namespace
 
@@ -29,8 +30,9 @@ struct trtrlb_batch {
     cudaStream_t copy_out = nullptr;   // moments, of trtrlb_batch_solve (created on
     cudaStream_t aux = nullptr;        // its first call)
     std::vector<trtrlb_t> lats;
-    cudaGraphExec_t graph = nullptr;
-    std::vector<int> graph_sig;   // (parity, cur) of every member when captured
+    // runs of kGraphSteps steps, captured once per start (parity, Phi buffer and
+    // population buffer of every member), at most kMaxGraphs of them
+    std::map<std::vector<int>, cudaGraphExec_t> graphs;
     char err[256] = "";
 };
 
@@ -46,18 +48,18 @@ int cuda_fail(trtrlb_batch* b, cudaError_t e, const char* where) {
     return TRTRLB_ECUDA;
 }
 
-void drop_graph(trtrlb_batch* b) {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-    b->graph_sig.clear();
+void drop_graphs(trtrlb_batch* b) {
+    for (const auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
+    b->graphs.clear();
 }
 
-std::vector<int> signature(const trtrlb_batch* b) {
+std::vector<int> signature(const trtrlb_batch* b, const std::vector<trt::State>& sim) {
     std::vector<int> sig;
-    for (const trtrlb_lattice* h : b->lats) {
-        sig.push_back(h->s.parity);
-        sig.push_back(h->s.cur);
-        sig.push_back(h->s.f == h->f ? 0 : 1);   // two-buffer lattices alternate buffers
+    for (size_t i = 0; i < sim.size(); ++i) {
+        sig.push_back(sim[i].parity);
+        sig.push_back(sim[i].cur);
+        sig.push_back(sim[i].f == b->lats[i]->f ? 0 : 1);   // two-buffer lattices alternate buffers
+        sig.push_back(sim[i].pair ? 1 : 0);
     }
     return sig;
 }
@@ -79,77 +81,116 @@ int log2i(int v) {
         }                                                                             \
     }()
 
-// Launches n steps of every member, starting from the members' current
-// states; step q sees parity ^ (q & 1) and, for lagged G, cur ^ (q & 1).
-cudaError_t launch_steps(trtrlb_batch* b, int64_t n) {
+// Launches n steps of every member from the states `sim` (one per member),
+// which it advances.  A member whose lattice the two-step kernel runs takes
+// single steps to an odd level and for a last odd one, and two at a time
+// between; members at different points share the launches they can.  closed: n
+// is kGraphSteps and every member must end at the parity and on the buffers it
+// began with, so that the launches can be replayed: every count of flips must
+// be even, which 16 launches of two steps from an odd level are, and, from an
+// even one, a single step, 14 launches of two and three single steps.
+cudaError_t launch_steps(trtrlb_batch* b, std::vector<trt::State>& sim, int64_t n, bool closed = false) {
     using Key = std::tuple<int, int, int, int>;  // storage, flavour, g_mode, odd
+    std::vector<int64_t> done(sim.size(), 0);
+    std::vector<int64_t> last(sim.size(), n);    // no launch of two steps ends after it
+    for (size_t i = 0; i < sim.size(); ++i)
+        if (closed && sim[i].parity == 0) last[i] = n - 3;
     for (int64_t q = 0; q < n; ++q) {
-        const int flip = (int)(q & 1);
         std::map<Key, std::vector<int>> groups;
-        for (int i = 0; i < (int)b->lats.size(); ++i) {
+        std::map<std::tuple<int, int>, std::vector<int>> pairs;   // storage, g_mode
+        std::vector<int> tma, alone;
+        for (int i = 0; i < (int)sim.size(); ++i) {
+            if (done[i] != q) continue;
             const trtrlb_lattice* h = b->lats[i];
-            if (h->s.g_mode == TRTRLB_G_CURRENT) continue;   // two-buffer kernel, below
-            const int flav = h->s.general ? trt::FLAV_GENERAL : (h->s.vec ? trt::FLAV_VECTOR : trt::FLAV_PERIODIC);
-            groups[Key{h->p.storage, flav, h->s.g_mode, h->s.parity ^ flip}].push_back(i);
+            const trt::State& s = sim[i];
+            if (s.g_mode == TRTRLB_G_CURRENT) {
+                // two-buffer members: the small TMA-fed ones share launches, the
+                // others run one launch each
+                (shares_tma_launch(h) ? tma : alone).push_back(i);
+                done[i] += 1;
+            } else if (s.pair && s.parity == 1 && q + 2 <= last[i]) {
+                pairs[{h->p.storage, s.g_mode}].push_back(i);
+                done[i] += 2;
+            } else {
+                const int flav = s.general ? trt::FLAV_GENERAL : (s.vec ? trt::FLAV_VECTOR : trt::FLAV_PERIODIC);
+                groups[Key{h->p.storage, flav, s.g_mode, s.parity}].push_back(i);
+                done[i] += 1;
+            }
+        }
+        for (const auto& kv : pairs) {
+            std::vector<const trt::State*> m;
+            for (int i : kv.second) m.push_back(&sim[i]);
+            const cudaError_t e = TRT_DISPATCH_S(std::get<0>(kv.first), step_pair(m.data(), (int)m.size(), b->stream));
+            if (e != cudaSuccess) return e;
+            for (int i : kv.second) trt::after_pair(sim[i]);
         }
         for (const auto& kv : groups) {
             const Key& k = kv.first;
             std::vector<const trt::State*> m;
             std::vector<int> cur, l2;
             for (int i : kv.second) {
-                const trtrlb_lattice* h = b->lats[i];
-                m.push_back(&h->s);
-                cur.push_back(h->s.g_mode == TRTRLB_G_LAGGED ? (h->s.cur ^ flip) : h->s.cur);
-                l2.push_back(log2i(h->tile_w));
+                m.push_back(&sim[i]);
+                cur.push_back(sim[i].cur);
+                l2.push_back(log2i(b->lats[i]->tile_w));
             }
-            const cudaError_t e = TRT_DISPATCH_S(
+            cudaError_t e = TRT_DISPATCH_S(
                 std::get<0>(k), step_group(m.data(), cur.data(), l2.data(), (int)m.size(),
                                            std::get<3>(k) != 0, std::get<1>(k),
                                            std::get<2>(k), b->stream));
-            if (e != cudaSuccess) return e;
-        }
-        // two-buffer (G_CURRENT) members: the small TMA-fed ones share
-        // launches, the others run one launch each
-        std::vector<const trt::State*> tma;
-        for (trtrlb_lattice* h : b->lats)
-            if (shares_tma_launch(h)) tma.push_back(&h->s);
-        if (!tma.empty()) {
-            const cudaError_t e = trt::Ops<float>::step_ab_group(tma.data(), (int)tma.size(), flip, b->stream);
-            if (e != cudaSuccess) return e;
-        }
-        for (trtrlb_lattice* h : b->lats) {
-            if (h->s.g_mode == TRTRLB_G_CURRENT) {
-                if (shares_tma_launch(h)) continue;
-                const cudaError_t e = TRT_DISPATCH_S(h->p.storage, step_ab(h->s, flip, b->stream));
-                if (e != cudaSuccess) return e;
-                continue;
+            for (int i : kv.second) {
+                if (e == cudaSuccess && sim[i].nghost > 0)
+                    e = TRT_DISPATCH_S(std::get<0>(k), ghost_pass(sim[i], 0, b->stream));
+                sim[i].parity ^= 1;
+                if (sim[i].g_mode == TRTRLB_G_LAGGED) sim[i].cur ^= 1;
             }
-            if (h->s.nghost == 0) continue;
-            const cudaError_t e = TRT_DISPATCH_S(h->p.storage, ghost_pass(h->s, flip, b->stream));
             if (e != cudaSuccess) return e;
+        }
+        std::vector<const trt::State*> m;
+        for (int i : tma) m.push_back(&sim[i]);
+        if (!m.empty()) {
+            const cudaError_t e = trt::Ops<float>::step_ab_group(m.data(), (int)m.size(), 0, b->stream);
+            if (e != cudaSuccess) return e;
+        }
+        for (int i : alone) {
+            const cudaError_t e = TRT_DISPATCH_S(b->lats[i]->p.storage, step_ab(sim[i], 0, b->stream));
+            if (e != cudaSuccess) return e;
+            tma.push_back(i);
+        }
+        for (int i : tma) {
+            void* t = sim[i].f;
+            sim[i].f = sim[i].f2;
+            sim[i].f2 = t;
         }
     }
     return cudaSuccess;
 }
 
-int capture(trtrlb_batch* b) {
+// The graph of kGraphSteps steps from `sim`, captured if it is not there yet.
+int graph_from(trtrlb_batch* b, const std::vector<trt::State>& sim, cudaGraphExec_t* out) {
+    const std::vector<int> sig = signature(b, sim);
+    const auto it = b->graphs.find(sig);
+    if (it != b->graphs.end()) {
+        *out = it->second;
+        return TRTRLB_OK;
+    }
+    if (b->graphs.size() >= kMaxGraphs) drop_graphs(b);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(b, e, "graph capture");
-    const cudaError_t le = launch_steps(b, kGraphSteps);
+    std::vector<trt::State> copy = sim;
+    const cudaError_t le = launch_steps(b, copy, kGraphSteps, true);
     e = cudaStreamEndCapture(b->stream, &g);
     if (le != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
         return cuda_fail(b, le, "graph capture launch");
     }
     if (e != cudaSuccess) return cuda_fail(b, e, "graph capture end");
-    e = cudaGraphInstantiate(&b->graph, g, 0);
+    cudaGraphExec_t x = nullptr;
+    e = cudaGraphInstantiate(&x, g, 0);
     cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        b->graph = nullptr;
-        return cuda_fail(b, e, "graph instantiate");
-    }
-    b->graph_sig = signature(b);
+    if (e != cudaSuccess) return cuda_fail(b, e, "graph instantiate");
+    b->graphs[sig] = x;
+    *out = x;
     return TRTRLB_OK;
 }
 
@@ -169,7 +210,7 @@ int trtrlb_batch_create(void* stream, trtrlb_batch_t* out) {
 int trtrlb_batch_destroy(trtrlb_batch_t b) {
     if (!b) return TRTRLB_OK;
     cudaStreamSynchronize(b->stream);
-    drop_graph(b);
+    drop_graphs(b);
     if (b->copy_in) cudaStreamDestroy(b->copy_in);
     if (b->copy_out) cudaStreamDestroy(b->copy_out);
     if (b->aux) cudaStreamDestroy(b->aux);
@@ -187,7 +228,7 @@ int trtrlb_batch_set(trtrlb_batch_t b, const trtrlb_t* lattices, int count) {
         for (int r = 0; r < q; ++r)
             if (l[r] == l[q]) return fail(b, TRTRLB_EINVAL, "a lattice appears twice");
     }
-    drop_graph(b);
+    drop_graphs(b);
     b->lats.swap(l);
     return TRTRLB_OK;
 }
@@ -217,31 +258,34 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
     b->err[0] = 0;
     if (nsteps < 0) return fail(b, TRTRLB_EINVAL, "nsteps must be >= 0");
     if (nsteps == 0 || b->lats.empty()) return TRTRLB_OK;
+    std::vector<trt::State> sim;
+    for (trtrlb_lattice* h : b->lats) {
+        trt::keep_spare(h);   // graphs name it
+        sim.push_back(h->s);
+    }
     int64_t done = 0;
+    cudaError_t e = cudaSuccess;
     if (b->stream != nullptr && nsteps >= kGraphSteps) {
-        if (b->graph && b->graph_sig != signature(b)) drop_graph(b);
-        if (!b->graph) {
-            if (int rc = capture(b)) return rc;
+        // to odd levels, where the runs of two start, if that is a step for all
+        bool odd_pair = false, even_pair = false;
+        for (const trt::State& x : sim) (x.parity ? odd_pair : even_pair) |= x.pair;
+        if (even_pair && !odd_pair && nsteps > kGraphSteps) {
+            e = launch_steps(b, sim, 1);
+            done = 1;
+            if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
         }
+        cudaGraphExec_t graph = nullptr;
+        if (int rc = graph_from(b, sim, &graph)) return rc;
         for (; done + kGraphSteps <= nsteps; done += kGraphSteps) {
-            const cudaError_t e = cudaGraphLaunch(b->graph, b->stream);
+            e = cudaGraphLaunch(graph, b->stream);
             if (e != cudaSuccess) return cuda_fail(b, e, "graph launch");
         }
     }
-    const cudaError_t e = launch_steps(b, nsteps - done);
+    e = launch_steps(b, sim, nsteps - done);
     if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
-    for (trtrlb_lattice* h : b->lats) {
-        if (h->s.g_mode == TRTRLB_G_CURRENT) {
-            if (nsteps & 1) {
-                void* t = h->s.f;
-                h->s.f = h->s.f2;
-                h->s.f2 = t;
-            }
-        } else {
-            h->s.parity ^= (int)(nsteps & 1);
-            if (h->s.g_mode == TRTRLB_G_LAGGED) h->s.cur ^= (int)(nsteps & 1);
-        }
-        h->t += nsteps;
+    for (size_t i = 0; i < sim.size(); ++i) {
+        b->lats[i]->s = sim[i];
+        b->lats[i]->t += nsteps;
     }
     return TRTRLB_OK;
 }

@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(AB_TX * AB_TY, 4) k_step_ab(Args<typename Fmt<
         dpy = C(0.5) * (sy[ty + 2][tx] - sy[ty][tx]);
     }
     C o[9], phx, phy;
-    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.rho0, o, phx, phy);
+    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
     if (!GENERAL) {
         const int xm = ab_wrap(x - 1, a.nx), xp = ab_wrap(x + 1, a.nx);
         const long long rm = (long long)ab_wrap(y - 1, a.ny) * a.pitch;

@@ -81,18 +81,18 @@ __global__ void __launch_bounds__(COL_WARPS * 32, col_min_blocks<S>())
         const int k = y * a.pitch + cw;
 #pragma unroll
         for (int i = 0; i < 9; ++i) d[i] = Fmt<S>::ld(F[(long long)i * a.plane + k]);
-        return node_moments<C>(d, a.gx, a.gy, a.rho0);
+        return node_moments<C>(d, a.hgx, a.hgy, a.rho0);
     };
     NodeMom<C> m_prev = row_moments(y0 == 0 ? a.ny - 1 : y0 - 1);
-    C phy_prev = m_prev.rho * m_prev.uy * m_prev.uy * m_prev.uy;
+    C phy_prev = phi_of(m_prev.rho, m_prev.uy);
     NodeMom<C> m_cur = row_moments(y0);
-    C phx_cur = m_cur.rho * m_cur.ux * m_cur.ux * m_cur.ux;
-    C phy_cur = m_cur.rho * m_cur.uy * m_cur.uy * m_cur.uy;
+    C phx_cur = phi_of(m_cur.rho, m_cur.ux);
+    C phy_cur = phi_of(m_cur.rho, m_cur.uy);
     for (int y = y0; y < y1; ++y) {
         const int yn = y + 1 == a.ny ? 0 : y + 1;
         const NodeMom<C> m_next = row_moments(yn);
-        const C phx_next = m_next.rho * m_next.ux * m_next.ux * m_next.ux;
-        const C phy_next = m_next.rho * m_next.uy * m_next.uy * m_next.uy;
+        const C phx_next = phi_of(m_next.rho, m_next.ux);
+        const C phy_next = phi_of(m_next.rho, m_next.uy);
         const C left = __shfl_up_sync(0xffffffffu, phx_cur, 1);
         const C right = __shfl_down_sync(0xffffffffu, phx_cur, 1);
         if (inner) {

@@ -213,11 +213,11 @@ __global__ void __launch_bounds__(AB_TX * AB_TY, TMA_R == 1 ? 5 : 3)
             float d[9];
 #pragma unroll
             for (int i = 0; i < 9; ++i) d[i] = st.v[i][ry + 1][tx + TMA_XOFF];
-            m[r] = node_moments<float>(d, a.gx, a.gy, a.rho0);
+            m[r] = node_moments<float>(d, a.hgx, a.hgy, a.rho0);
             float px = 0.f, py = 0.f;
             if (x < a.nx && y < a.ny) {
-                px = m[r].rho * m[r].ux * m[r].ux * m[r].ux;
-                py = m[r].rho * m[r].uy * m[r].uy * m[r].uy;
+                px = phi_of(m[r].rho, m[r].ux);
+                py = phi_of(m[r].rho, m[r].uy);
             } else if ((x == a.nx && y < a.ny) || (y == a.ny && x < a.nx)) {
                 tma_phi_global(a, F, ab_wrap(x, a.nx), ab_wrap(y, a.ny), px, py);
             }

@@ -82,6 +82,7 @@ template <typename C> struct Args {
     C k1, k1lo, k2, k2lo; // 1 - 1/tau as a hi + lo pair (lo = 0 for FP64)
     C kf;                 // 1 - 1/(2 tau1)
     C gx, gy, rho0;
+    C hgx, hgy;           // g / 2
     C corr[9];            // moving-wall term 2 w_i rho_w (e_i.u_w) / c_s^2
     C phin_x, phin_y;     // Phi of moving-wall (inlet) nodes, rho_w u_w^3
     C zh_dr;              // rho0 - outlet_rho of the Zou-He pressure outlet
@@ -278,38 +279,57 @@ __device__ __forceinline__ void collide_dw(const df64 (&d)[9], df64 dpx, df64 dp
     phy = ruyy * uy;
 }
 
+// Single-rounding operations.  Every kernel writes the collision with these, so
+// that where a product and a sum share one rounding (ffma) is fixed here and
+// not chosen by the compiler per kernel: the one-step, two-step, batched and
+// two-buffer kernels give the same bits for the same node.
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float rrcp(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
+
 // Raw moments of one node's shifted populations and its eq11 velocity: the
 // first half of the collision, which the two-buffer TMA kernel also uses for
-// Phi before its halo barrier.
+// Phi before its halo barrier.  hgx, hgy: g/2.
 template <typename C> struct NodeMom {
     C drho, s13, s24, sd, pxy, qxxy, qxyy, jx, jy;   // sums of d weighted by e
     C rho, ux, uy;
 };
 
 template <typename C>
-__device__ __forceinline__ NodeMom<C> node_moments(const C (&d)[9], const C gx, const C gy,
+__device__ __forceinline__ NodeMom<C> node_moments(const C (&d)[9], const C hgx, const C hgy,
                                                    const C rho0) {
     NodeMom<C> m;
-    m.s13 = d[1] + d[3];
-    const C m13 = d[1] - d[3];
-    m.s24 = d[2] + d[4];
-    const C m24 = d[2] - d[4];
-    const C a57 = d[5] + d[7], m57 = d[5] - d[7];
-    const C a68 = d[6] + d[8], m68 = d[6] - d[8];
-    m.sd = a57 + a68;      // sum of the four diagonal populations
-    m.pxy = a57 - a68;     // sum e_x e_y d
-    m.qxxy = m57 + m68;    // sum e_x^2 e_y d
-    m.qxyy = m57 - m68;    // sum e_x e_y^2 d
-    m.jx = m13 + m.qxyy;   // sum e_x d
-    m.jy = m24 + m.qxxy;   // sum e_y d
-    m.drho = (d[0] + m.sd) + (m.s13 + m.s24);
+    m.s13 = radd(d[1], d[3]);
+    const C m13 = rsub(d[1], d[3]);
+    m.s24 = radd(d[2], d[4]);
+    const C m24 = rsub(d[2], d[4]);
+    const C a57 = radd(d[5], d[7]), m57 = rsub(d[5], d[7]);
+    const C a68 = radd(d[6], d[8]), m68 = rsub(d[6], d[8]);
+    m.sd = radd(a57, a68);      // sum of the four diagonal populations
+    m.pxy = rsub(a57, a68);     // sum e_x e_y d
+    m.qxxy = radd(m57, m68);    // sum e_x^2 e_y d
+    m.qxyy = rsub(m57, m68);    // sum e_x e_y^2 d
+    m.jx = radd(m13, m.qxyy);   // sum e_x d
+    m.jy = radd(m24, m.qxxy);   // sum e_y d
+    m.drho = radd(radd(d[0], m.sd), radd(m.s13, m.s24));
     // eq11: rho = sum f, u = (sum e f)/rho + g/2
-    m.rho = rho0 + m.drho;
-    const C inv = C(1) / m.rho;
-    m.ux = m.jx * inv + C(0.5) * gx;
-    m.uy = m.jy * inv + C(0.5) * gy;
+    m.rho = radd(rho0, m.drho);
+    const C inv = rrcp(m.rho);
+    m.ux = rfma(m.jx, inv, hgx);
+    m.uy = rfma(m.jy, inv, hgy);
     return m;
 }
+
+// Phi_xxx = rho u_x^3 (eq_Gi), rounded as the collision rounds it.
+template <typename C>
+__device__ __forceinline__ C phi_of(const C rho, const C u) { return rmul(rmul(rmul(rho, u), u), u); }
 
 // The rest of the collision (eq2 with eq9, eq_Gi and eq6) from the moments.
 template <typename C>
@@ -318,71 +338,80 @@ __device__ __forceinline__ void collide_from(const NodeMom<C>& m, C dpx, C dpy, 
                                              const C gx, const C gy, C (&o)[9], C& phx, C& phy) {
     const C third = C(1.0 / 3.0);
     const C drho = m.drho, rho = m.rho, ux = m.ux, uy = m.uy, jx = m.jx, jy = m.jy;
-    const C Fx = rho * gx, Fy = rho * gy;
-    const C rux = rho * ux, ruy = rho * uy;
-    const C ruxx = rux * ux, ruyy = ruy * uy, ruxy = rux * uy;
-    const C rxxy = ruxx * uy, rxyy = ruyy * ux;
+    const C rux = rmul(rho, ux), ruy = rmul(rho, uy);
+    const C ruxx = rmul(rux, ux), ruyy = rmul(ruy, uy), ruxy = rmul(rux, uy);
+    const C rxxy = rmul(ruxx, uy), rxyy = rmul(ruyy, ux);
     // Hermite moments sum H f: second order (H_xx = e_x^2 - 1/3, ...) and the
     // surviving third-order components; minus the equilibrium moments of
     // eq9_2 they are the non-equilibrium projections A of eq9 (A_x = -F_x/2
     // is folded into a1)
-    const C drho3 = third * drho;
-    const C Pxx = (m.s13 + m.sd) - drho3, Pyy = (m.s24 + m.sd) - drho3;
-    const C Qxxy = m.qxxy - third * jy, Qxyy = m.qxyy - third * jx;
-    const C Axx = Pxx - ruxx, Ayy = Pyy - ruyy, Axy = m.pxy - ruxy;
-    const C Axxy = Qxxy - rxxy, Axyy = Qxyy - rxyy;
+    const C Axx = rsub(rfma(-third, drho, radd(m.s13, m.sd)), ruxx);
+    const C Ayy = rsub(rfma(-third, drho, radd(m.s24, m.sd)), ruyy);
+    const C Axy = rsub(m.pxy, ruxy);
+    const C Axxy = rsub(rfma(-third, jy, m.qxxy), rxxy);
+    const C Axyy = rsub(rfma(-third, jx, m.qxyy), rxyy);
     // relaxation: (1 - 1/tau) A with 1 - 1/tau carried as hi + lo, so the rate
     // 1/tau stays exact to ~2^-48 even when tau is large (FP32 alone would
     // round 1 - 1/tau to 2^-24 absolute, i.e. 1/tau to 2^-24 tau relative)
     // (FP64 needs no low part: its rounding of 1 - 1/tau is below 1e-11 of the
     // rate for any tau this library accepts in practice)
     constexpr bool split = sizeof(C) < 8;
-    const C a1x = jx + Fx, a1y = jy + Fy;
-    C r2xx = ruxx + k1 * Axx, r2yy = ruyy + k1 * Ayy, r2xy = ruxy + k1 * Axy;
-    C a3xxy = rxxy + k2 * Axxy, a3xyy = rxyy + k2 * Axyy;
+    C r2xx = rfma(k1, Axx, ruxx), r2yy = rfma(k1, Ayy, ruyy), r2xy = rfma(k1, Axy, ruxy);
+    C a3xxy = rfma(k2, Axxy, rxxy), a3xyy = rfma(k2, Axyy, rxyy);
     if (split) {
-        r2xx += k1lo * Axx;
-        r2yy += k1lo * Ayy;
-        r2xy += k1lo * Axy;
-        a3xxy += k2lo * Axxy;
-        a3xyy += k2lo * Axyy;
+        r2xx = rfma(k1lo, Axx, r2xx);
+        r2yy = rfma(k1lo, Ayy, r2yy);
+        r2xy = rfma(k1lo, Axy, r2xy);
+        a3xxy = rfma(k2lo, Axxy, a3xxy);
+        a3xyy = rfma(k2lo, Axyy, a3xyy);
     }
-    const C a2xx = r2xx + kf * (C(2) * Fx * ux - dpx);
-    const C a2yy = r2yy + kf * (C(2) * Fy * uy - dpy);
-    const C a2xy = r2xy + kf * (Fx * uy + ux * Fy);
+    // body force; FP64, whose pipe bounds the step, skips its terms (exact zeros)
+    // without one (a uniform branch)
+    C a1x = jx, a1y = jy, a2xx, a2yy, a2xy = r2xy;
+    if (sizeof(C) < 8 || gx != C(0) || gy != C(0)) {
+        const C Fx = rmul(rho, gx), Fy = rmul(rho, gy);
+        a1x = radd(jx, Fx);
+        a1y = radd(jy, Fy);
+        a2xx = rfma(kf, rfma(radd(Fx, Fx), ux, -dpx), r2xx);
+        a2yy = rfma(kf, rfma(radd(Fy, Fy), uy, -dpy), r2yy);
+        a2xy = rfma(kf, rfma(Fx, uy, rmul(ux, Fy)), r2xy);
+    } else {
+        a2xx = rfma(-kf, dpx, r2xx);
+        a2yy = rfma(-kf, dpy, r2yy);
+    }
     // reconstruction, w_i folded in: w0 = 4/9, w1..4 = 1/9, w5..8 = 1/36
-    const C t = a2xx + a2yy;
-    o[0] = C(4.0 / 9.0) * drho - C(2.0 / 3.0) * t;
-    const C b9 = C(1.0 / 9.0) * drho;
-    const C c13 = b9 + C(1.0 / 3.0) * a2xx - C(1.0 / 6.0) * a2yy;
-    const C o13 = C(1.0 / 3.0) * a1x - C(0.5) * a3xyy;
-    const C c24 = b9 - C(1.0 / 6.0) * a2xx + C(1.0 / 3.0) * a2yy;
-    const C o24 = C(1.0 / 3.0) * a1y - C(0.5) * a3xxy;
-    o[1] = c13 + o13;
-    o[3] = c13 - o13;
-    o[2] = c24 + o24;
-    o[4] = c24 - o24;
-    const C cd = C(1.0 / 36.0) * drho + C(1.0 / 12.0) * t;
-    const C q = C(0.25) * a2xy;
-    const C c57 = cd + q, c68 = cd - q;
-    const C o57 = C(1.0 / 12.0) * (a1x + a1y) + C(0.25) * (a3xxy + a3xyy);
-    const C o68 = C(1.0 / 12.0) * (a1y - a1x) + C(0.25) * (a3xxy - a3xyy);
-    o[5] = c57 + o57;
-    o[7] = c57 - o57;
-    o[6] = c68 + o68;
-    o[8] = c68 - o68;
-    phx = ruxx * ux;
-    phy = ruyy * uy;
+    const C t = radd(a2xx, a2yy);
+    o[0] = rfma(C(4.0 / 9.0), drho, rmul(C(-2.0 / 3.0), t));
+    const C b9 = rmul(C(1.0 / 9.0), drho);
+    const C c13 = rfma(C(-1.0 / 6.0), a2yy, rfma(C(1.0 / 3.0), a2xx, b9));
+    const C o13 = rfma(C(1.0 / 3.0), a1x, rmul(C(-0.5), a3xyy));
+    const C c24 = rfma(C(-1.0 / 6.0), a2xx, rfma(C(1.0 / 3.0), a2yy, b9));
+    const C o24 = rfma(C(1.0 / 3.0), a1y, rmul(C(-0.5), a3xxy));
+    o[1] = radd(c13, o13);
+    o[3] = rsub(c13, o13);
+    o[2] = radd(c24, o24);
+    o[4] = rsub(c24, o24);
+    const C cd = rfma(C(1.0 / 12.0), t, rmul(C(1.0 / 36.0), drho));
+    const C c57 = rfma(C(0.25), a2xy, cd), c68 = rfma(C(-0.25), a2xy, cd);
+    const C o57 = rfma(C(1.0 / 12.0), radd(a1x, a1y), rmul(C(0.25), radd(a3xxy, a3xyy)));
+    const C o68 = rfma(C(1.0 / 12.0), rsub(a1y, a1x), rmul(C(0.25), rsub(a3xxy, a3xyy)));
+    o[5] = radd(c57, o57);
+    o[7] = rsub(c57, o57);
+    o[6] = radd(c68, o68);
+    o[8] = rsub(c68, o68);
+    phx = rmul(ruxx, ux);
+    phy = rmul(ruyy, uy);
 }
 
 template <typename C>
 __device__ __forceinline__ void collide(const C (&d)[9], C dpx, C dpy, const C k1, const C k1lo,
                                         const C k2, const C k2lo, const C kf, const C gx,
-                                        const C gy, const C rho0, C (&o)[9], C& phx, C& phy) {
+                                        const C gy, const C hgx, const C hgy, const C rho0, C (&o)[9],
+                                        C& phx, C& phy) {
     if constexpr (std::is_same<C, df64>::value) {
         collide_dw(d, dpx, dpy, k1, k2, kf, gx, gy, rho0, o, phx, phy);
     } else {
-        collide_from<C>(node_moments<C>(d, gx, gy, rho0), dpx, dpy, k1, k1lo, k2, k2lo, kf, gx, gy, o,
+        collide_from<C>(node_moments<C>(d, hgx, hgy, rho0), dpx, dpy, k1, k1lo, k2, k2lo, kf, gx, gy, o,
                         phx, phy);
     }
 }
@@ -475,7 +504,7 @@ __device__ __forceinline__ void periodic_finish(const Args<typename Fmt<S>::C>& 
     const int cyp = y == a.ny - 1 ? -pl : 0, cym = y == 0 ? pl : 0;
     S* __restrict__ F = static_cast<S*>(a.f);
     C o[9], phx, phy;
-    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.rho0, o, phx, phy);
+    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
     if (GMODE == G_LAGGED) {
         a.phi_out[own] = phx;
         a.phi_out[a.plane + own] = phy;
@@ -531,7 +560,7 @@ __device__ __forceinline__ void node_step_periodic(const Args<typename Fmt<S>::C
         dpy = C(0.5) * (Py[pt + cyp] - Py[-pt + cym]);
     }
     C o[9], phx, phy;
-    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.rho0, o, phx, phy);
+    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
     if (GMODE == G_LAGGED) {
         a.phi_out[own] = phx;
         a.phi_out[a.plane + own] = phy;
@@ -609,7 +638,7 @@ __device__ __forceinline__ void node_step(const Args<typename Fmt<S>::C>& a, int
         dpy = C(0.5) * (pyp - pym);
     }
     C o[9], phx, phy;
-    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.rho0, o, phx, phy);
+    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
     if (GMODE == G_LAGGED) {
         a.phi_out[own] = phx;
         a.phi_out[a.plane + own] = phy;

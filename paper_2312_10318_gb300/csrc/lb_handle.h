@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "lb_ops.cuh"
 #include "trtrlb.h"
 
@@ -12,7 +14,7 @@ struct trtrlb_lattice {
     cudaStream_t stream;
     int64_t t;           // steps since init / set_f
     void* f;             // device allocations owned by the handle
-    void* f2;            // second population buffer (G_CURRENT only)
+    void* f2;            // second population buffer (G_CURRENT; the two-step kernel's), or null
     void* phi;           // both Phi buffers in one allocation
     uint8_t* mask;
     uint8_t* seg;        // interior row segments of a general lattice (State::seg), or null
@@ -28,6 +30,8 @@ struct trtrlb_lattice {
     int* kerr;           // device flag set when a kernel's bounded wait ran out, or null
     int tma_grid;        // persistent grid of the TMA kernel on this device (0: none)
     int sms;             // multiprocessors of the handle's device
+    std::mutex spare_mu; // held while launches that use f2 of a lagged lattice are queued
+    bool spare_kept;     // f2 is named by a captured graph: not given back before the handle
     char err[256];
 };
 
@@ -43,6 +47,22 @@ inline bool shares_tma_launch(const trtrlb_lattice* h) {
 }
 
 namespace trt {
+// Keeps the two-step kernel's second buffer of h for the handle's lifetime
+// (launches that use it are captured, or queued outside advance()).
+void keep_spare(trtrlb_lattice* h);
+
+// Advances h by n time steps on st: two at a time from odd levels where the
+// two-step kernel runs the lattice.
+cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st);
+
+// The effect of one launch of the two-step kernel on a lattice's state.
+inline void after_pair(State& s) {
+    void* t = s.f;
+    s.f = s.f2;
+    s.f2 = t;
+    if (s.g_mode == TRTRLB_G_LAGGED) s.cur ^= 1;
+}
+
 // Body of trtrlb_batch_solve over the members m[0 .. count): see trtrlb.h.
 // st runs the members' steps, aux their initial states and moments; cin and
 // cout their uploads and downloads.

@@ -31,9 +31,15 @@ constexpr int TMA_BX = 40, TMA_BY = TMA_TH + 2, TMA_XOFF = 4;
 // for a tile copy; the limit only bounds a wait that would never end).
 constexpr long long kDefaultWaitLimit = 1ll << 22;
 
+// Two-step kernel (lb_pair.cuh): nodes of a row a warp updates, warps per CTA.
+constexpr int PAIR_W = 60, PAIR_WARPS = 4;
+
 struct State {
     void* f;              // populations, S[9][ny][pitch]
-    void* f2;             // second buffer of the two-buffer G_CURRENT kernel (else null)
+    void* f2;             // second buffer: of the two-buffer G_CURRENT kernel, or of
+                          // the two-step kernel (else null)
+    bool pair;            // the two-step kernel advances this lattice from odd levels
+    int sms;              // multiprocessors of the device
     void* phi[2];         // Phi buffers, C[2][ny][pitch]
     int cur;              // phi[cur] holds the previous level
     const uint8_t* mask;  // device [ny][pitch] or nullptr
@@ -67,6 +73,10 @@ struct State {
 template <typename S> struct Ops {
     // One time step (plus the outlet-ghost pass); flips parity and Phi buffers.
     static cudaError_t step(State& s, cudaStream_t st);
+    // Two time steps of n lattices (State::pair, at an odd level, same flavour
+    // and G mode) in one launch per 64; the caller swaps f and f2, and with Phi
+    // lagged the Phi buffers.
+    static cudaError_t step_pair(const State* const* members, int n, cudaStream_t st);
     static cudaError_t phi_static(State& s, cudaStream_t st);
     static cudaError_t init(State& s, const double* rho, const double* ux, const double* uy,
                             cudaStream_t st);

@@ -8,6 +8,7 @@
 #include "lb_aux.cuh"
 #include "lb_batch.cuh"
 #include "lb_ops.cuh"
+#include "lb_pair.cuh"
 
 namespace trt {
 
@@ -30,6 +31,7 @@ static Args<C> make_args(const State& s, bool swap_phi = false) {
     a.k2lo = (C)(k2 - (double)a.k2);
     a.kf = (C)(1.0 - 1.0 / (2.0 * s.tau1));
     a.gx = (C)s.gx; a.gy = (C)s.gy; a.rho0 = (C)s.rho0;
+    a.hgx = (C)(0.5 * s.gx); a.hgy = (C)(0.5 * s.gy);
     for (int i = 0; i < 9; ++i) {
         // 2 w_i rho_w (e_i.u_w) / c_s^2, subtracted from f*_i when e_i points
         // into a moving wall (Ladd's correction)
@@ -375,6 +377,47 @@ cudaError_t Ops<S>::step_group(const State* const* m, const int* cur, const int*
     if (flavour == FLAV_GENERAL) return launch_group_g<S, false, FLAV_GENERAL>(m, cur, l2tw, n, g_mode, st);
     if (flavour == FLAV_VECTOR) return launch_group_g<S, false, FLAV_VECTOR>(m, cur, l2tw, n, g_mode, st);
     return launch_group_g<S, false, FLAV_PERIODIC>(m, cur, l2tw, n, g_mode, st);
+}
+
+template <typename S, int GMODE, int MAXL>
+static cudaError_t launch_pair(const State* const* m, int n, cudaStream_t st) {
+    PairParams<MAXL> p;
+    p.n = n;
+    const int band = pair_band_rows(m, n, (long long)m[0]->sms * PAIR_BLOCKS * PAIR_WARPS);
+    int tiles = 0;
+    for (int q = 0; q < n; ++q) {
+        const State& s = *m[q];
+        p.a[q] = make_args<float>(s);
+        p.out[q] = s.f2;
+        p.tile_begin[q] = tiles;
+        p.strips[q] = pair_strips(s.nx);
+        p.inv_d[q] = 1.0f / (float)p.strips[q];
+        p.band[q] = band;
+        const long long warps = (long long)p.strips[q] * ((s.ny + band - 1) / band);
+        tiles += (int)((warps + PAIR_WARPS - 1) / PAIR_WARPS);
+    }
+    p.tile_begin[n] = tiles;
+    k_step_pair<S, GMODE, MAXL><<<tiles, PAIR_WARPS * 32, 0, st>>>(p);
+    return cudaGetLastError();
+}
+
+template <typename S>
+cudaError_t Ops<S>::step_pair(const State* const* m, int n, cudaStream_t st) {
+    if constexpr (sizeof(S) <= 4) {
+        for (int q0 = 0; q0 < n; q0 += 64) {
+            const int c = n - q0 < 64 ? n - q0 : 64;
+            cudaError_t e;
+            if (m[q0]->g_mode == G_OFF)
+                e = c <= 4 ? launch_pair<S, G_OFF, 4>(m + q0, c, st) : launch_pair<S, G_OFF, 64>(m + q0, c, st);
+            else
+                e = c <= 4 ? launch_pair<S, G_LAGGED, 4>(m + q0, c, st) : launch_pair<S, G_LAGGED, 64>(m + q0, c, st);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    } else {
+        (void)m; (void)n; (void)st;
+        return cudaErrorInvalidValue;
+    }
 }
 
 template <typename S>

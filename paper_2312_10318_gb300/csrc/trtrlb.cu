@@ -10,7 +10,9 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "lb_ab_col.cuh"
@@ -73,8 +75,73 @@ bool on_device(const void* p) {
         }                                                                        \
     }()
 
+// Handles whose two-step kernel has a second population buffer.
+std::mutex g_spares_mu;
+std::vector<trtrlb_lattice*> g_spares;
+size_t g_spares_bytes = 0;
+
+// Removes h (g_spares_mu held).
+void forget_spare(trtrlb_lattice* h) {
+    for (size_t i = 0; i < g_spares.size(); ++i)
+        if (g_spares[i] == h) {
+            g_spares[i] = g_spares.back();
+            g_spares.pop_back();
+            g_spares_bytes -= elem_size(h->p.storage) * 9 * (size_t)h->s.plane;
+            return;
+        }
+}
+
+// Whether another second buffer of `bytes` may be allocated: while they take up
+// no more than kSparesFree in all, or leave half of the device's memory free
+// (the query costs a small lattice's create a tenth).
+constexpr size_t kSparesFree = (size_t)4 << 30;
+bool spare_fits(size_t bytes) {
+    {
+        std::lock_guard<std::mutex> lk(g_spares_mu);
+        if (g_spares_bytes + bytes <= kSparesFree) return true;
+    }
+    size_t free_b = 0, total_b = 0;
+    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b > bytes && free_b - bytes >= total_b / 2;
+}
+
+// Gives back the second buffers that no queued or captured launch will name
+// (cudaFree waits for the queued ones); the lattices go on with single steps.
+// Called when an allocation fails, so that the buffers never cost a caller a
+// lattice that would have fit without them.
+void reclaim_spares() {
+    std::lock_guard<std::mutex> lk(g_spares_mu);
+    for (size_t i = 0; i < g_spares.size();) {
+        trtrlb_lattice* h = g_spares[i];
+        std::unique_lock<std::mutex> hl(h->spare_mu, std::try_to_lock);
+        if (!hl.owns_lock() || h->spare_kept) {
+            ++i;
+            continue;
+        }
+        if (h->s.f == h->f2) std::swap(h->f, h->f2);
+        cudaFree(h->f2);
+        h->bytes -= (int64_t)(elem_size(h->p.storage) * 9 * (size_t)h->s.plane);
+        h->f2 = nullptr;
+        h->s.f2 = nullptr;
+        h->s.pair = false;
+        forget_spare(h);
+    }
+}
+
+// cudaMalloc; if the device is full, once more without the second buffers.
+cudaError_t device_alloc(void** ptr, size_t bytes) {
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    reclaim_spares();
+    return cudaMalloc(ptr, bytes);
+}
+
 void release(trtrlb_lattice* h) {
     if (!h) return;
+    {
+        std::lock_guard<std::mutex> lk(g_spares_mu);
+        forget_spare(h);
+    }
     if (h->f) cudaFree(h->f);
     if (h->f2) cudaFree(h->f2);
     if (h->phi) cudaFree(h->phi);
@@ -114,6 +181,11 @@ bool vector_applies(const trtrlb_lattice* h) {
 bool auto_vector(const trtrlb_lattice* h) {
     const int st = h->p.storage;
     return vector_applies(h) && st != TRTRLB_F64 && st != TRTRLB_F64_DW;
+}
+
+// Lattices the two-step kernel advances (lb_pair.cuh).
+bool pair_applies(const trtrlb_params& p) {
+    return p.g_mode != TRTRLB_G_CURRENT && elem_size(p.storage) <= 4 && p.nx >= 32;
 }
 
 // Default two-buffer kernel of a G_CURRENT lattice that is periodic without a
@@ -174,7 +246,7 @@ cudaError_t ensure_stage(trtrlb_lattice* h, int fields) {
         h->stage_fields = 0;
     }
     const size_t bytes = sizeof(double) * fields * n;
-    const cudaError_t e = cudaMalloc((void**)&h->stage, bytes);
+    const cudaError_t e = device_alloc((void**)&h->stage, bytes);
     if (e == cudaSuccess) {
         h->bytes += (int64_t)bytes;
         h->stage_fields = fields;
@@ -318,13 +390,21 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
         return cuda_fail(err, e, "device query");
     }
     auto alloc = [&](void** ptr, size_t bytes) {
-        e = cudaMalloc(ptr, bytes);
+        e = device_alloc(ptr, bytes);
         if (e == cudaSuccess) h->bytes += (int64_t)bytes;
         return e == cudaSuccess;
     };
     bool ok = alloc(&h->f, es * 9 * plane) && alloc(&h->phi, ps * 4 * plane) &&
               alloc((void**)&h->dout, sizeof(double) * kResultDoubles);
     if (ok && p.g_mode == TRTRLB_G_CURRENT) ok = alloc(&h->f2, es * 9 * plane);
+    if (ok && !mask && p.periodic_x && p.periodic_y && pair_applies(p)) {
+        // the two-step kernel's second buffer, never a reason to fail
+        if (spare_fits(es * 9 * plane) && cudaMalloc(&h->f2, es * 9 * plane) == cudaSuccess)
+            h->bytes += (int64_t)(es * 9 * plane);
+        else
+            h->f2 = nullptr;
+        cudaGetLastError();
+    }
     if (ok && mask) ok = alloc((void**)&h->mask, (size_t)plane);
     if (ok && !ghosts.empty()) ok = alloc((void**)&h->ghosts, sizeof(int) * ghosts.size());
     trt::State& s = h->s;
@@ -370,7 +450,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     }
     if (s.general) {
         const std::vector<uint8_t> seg = interior_segments(mask, p.nx, p.ny, p.periodic_x, p.periodic_y);
-        e = cudaMalloc((void**)&h->seg, seg.size());
+        e = device_alloc((void**)&h->seg, seg.size());
         if (e == cudaSuccess) {
             h->bytes += (int64_t)seg.size();
             e = cudaMemcpy(h->seg, seg.data(), seg.size(), cudaMemcpyHostToDevice);
@@ -384,7 +464,8 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
         s.segs = (p.nx + 31) / 32;
     }
     e = cudaMemsetAsync(h->f, 0, es * 9 * plane, h->stream);
-    if (e == cudaSuccess && h->f2) e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
+    if (e == cudaSuccess && h->f2 && p.g_mode == TRTRLB_G_CURRENT)   // the two-step kernel writes before it reads
+        e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
     if (e == cudaSuccess) e = TRT_DISPATCH(p.storage, phi_static(h->s, h->stream));
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
@@ -397,6 +478,8 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     s.tile_w = h->tile_w;
     h->variant = TRTRLB_KERNEL_AUTO;
     s.vec = auto_vector(h);
+    s.sms = h->sms;
+    s.pair = p.g_mode != TRTRLB_G_CURRENT && h->f2;
     s.col_h = auto_column(h);
     if (p.g_mode == TRTRLB_G_CURRENT && p.storage == TRTRLB_F32 && !s.general) {
         // the TMA-fed two-buffer kernel; without a descriptor the plain one runs
@@ -421,6 +504,11 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
             h->kerr = nullptr;
             cudaGetLastError();
         }
+    }
+    if (s.pair) {
+        std::lock_guard<std::mutex> lk(g_spares_mu);
+        g_spares.push_back(h);
+        g_spares_bytes += es * 9 * (size_t)plane;
     }
     *out = h;
     return TRTRLB_OK;
@@ -468,12 +556,8 @@ int trtrlb_step(trtrlb_t h, int64_t nsteps) {
     if (!h) return TRTRLB_EINVAL;
     h->err[0] = 0;
     if (nsteps < 0) return fail(h->err, TRTRLB_EINVAL, "nsteps must be >= 0");
-    for (int64_t k = 0; k < nsteps; ++k) {
-        const cudaError_t e = TRT_DISPATCH(h->p.storage, step(h->s, h->stream));
-        if (e != cudaSuccess) return cuda_fail(h->err, e, "step");
-        ++h->t;
-    }
-    return TRTRLB_OK;
+    const cudaError_t e = trt::advance(h, nsteps, h->stream);
+    return e == cudaSuccess ? TRTRLB_OK : cuda_fail(h->err, e, "step");
 }
 
 int trtrlb_moments(trtrlb_t h, double* rho, double* ux, double* uy) {
@@ -736,6 +820,7 @@ int trtrlb_set_kernel(trtrlb_t h, int32_t variant, int32_t tile_w) {
     }
     h->variant = variant;
     h->s.vec = vec;
+    h->s.pair = variant == TRTRLB_KERNEL_AUTO && h->p.g_mode != TRTRLB_G_CURRENT && h->f2;
     if (variant == TRTRLB_KERNEL_COLUMN) {
         // the tallest band that still fills the device, else the shortest
         const int es = (int)elem_size(h->p.storage);
@@ -763,6 +848,12 @@ int trtrlb_get_kernel(trtrlb_t h, int32_t* vector, int32_t* tile_w) {
     if (!h) return TRTRLB_EINVAL;
     if (vector) *vector = h->s.vec ? 1 : 0;
     if (tile_w) *tile_w = h->tile_w;
+    return TRTRLB_OK;
+}
+
+int trtrlb_two_step(trtrlb_t h, int32_t* on) {
+    if (!h || !on) return TRTRLB_EINVAL;
+    *on = h->s.pair ? 1 : 0;
     return TRTRLB_OK;
 }
 
@@ -802,6 +893,37 @@ namespace trt {
 template <typename T>
 static T* at(T* const* a, int k) {
     return a ? a[k] : nullptr;
+}
+
+void keep_spare(trtrlb_lattice* h) {
+    std::lock_guard<std::mutex> lk(h->spare_mu);
+    h->spare_kept = true;
+}
+
+cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st) {
+    std::lock_guard<std::mutex> lk(h->spare_mu);
+    if (h->s.pair && !h->spare_kept) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+        if (e != cudaSuccess) return e;
+        h->spare_kept = cs != cudaStreamCaptureStatusNone;
+    }
+    while (n > 0) {
+        cudaError_t e;
+        int k = 1;
+        if (h->s.pair && h->s.parity == 1 && n >= 2) {
+            const State* one = &h->s;
+            e = TRT_DISPATCH(h->p.storage, step_pair(&one, 1, st));
+            if (e == cudaSuccess) after_pair(h->s);
+            k = 2;
+        } else {
+            e = TRT_DISPATCH(h->p.storage, step(h->s, st));
+        }
+        if (e != cudaSuccess) return e;
+        h->t += k;
+        n -= k;
+    }
+    return cudaSuccess;
 }
 
 // End-to-end solve of several lattices with the copies beside the steps (the
@@ -872,10 +994,7 @@ int solve_members(trtrlb_lattice* const* m, int count, cudaStream_t st, cudaStre
         trtrlb_lattice* h = m[k];
         const size_t n = (size_t)h->p.nx * h->p.ny;
         e = cudaStreamWaitEvent(st, ev_init[k], 0);
-        for (int64_t q = 0; q < nsteps && e == cudaSuccess; ++q) {
-            e = TRT_DISPATCH(h->p.storage, step(h->s, st));
-            ++h->t;
-        }
+        if (e == cudaSuccess) e = advance(h, nsteps, st);
         if (e == cudaSuccess) e = cudaEventRecord(ev_step[k], st);
         double* dst[3] = {at(rho_out, k), at(ux_out, k), at(uy_out, k)};
         double* dev[3] = {nullptr, nullptr, nullptr};

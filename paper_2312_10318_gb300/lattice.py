@@ -177,6 +177,12 @@ class Lattice:
         self._chk(self._lib.trtrlb_get_kernel(self._h, C.byref(vec), C.byref(tw)))
         return bool(vec.value), tw.value
 
+    def two_step(self) -> bool:
+        """Whether runs of steps advance two at a time (one launch for two steps)."""
+        k = C.c_int32()
+        self._chk(self._lib.trtrlb_two_step(self._h, C.byref(k)))
+        return bool(k.value)
+
     def step_kernel(self) -> str:
         """The step kernel the current settings select: 'aa' | 'aa_vector' (fused
         AA stream-collide), 'ab' | 'ab_tma' | 'ab_tma_shared' | 'ab_column'

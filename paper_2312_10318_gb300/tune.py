@@ -4,8 +4,10 @@ For each (storage format, boundary flavour, G mode, lattice-size bucket) it
 times the candidate kernels on a scratch lattice of that shape through the
 batched, graph-replayed path that the benchmark and the server use, and keeps
 the fastest.  With Phi lagged (the fused AA step) the candidates are the
-scalar kernel with 256-thread tiles of width 32, 64, 128 or 256 nodes and the
-vector kernel (V nodes per thread) where it applies; with Phi at the current
+scalar kernel with 256-thread tiles of width 32, 64, 128 or 256 nodes, the
+vector kernel (V nodes per thread) where it applies and, for FP32 and 16-bit
+storage on a periodic lattice, the two-step kernel (variant 'auto'); with Phi at
+the current
 level (the two-buffer step) on a periodic lattice without a mask they are the
 plain kernel, the column-walking kernel and, for FP32, the TMA-fed one.
 Results are cached in a JSON file keyed by the bucket, so a shape is measured
@@ -79,6 +81,8 @@ class Tuner:
         out = [("scalar", tw) for tw in TILE_WIDTHS if tw <= max(32, 2 * nx)]
         if flavour(periodic, has_mask) == "periodic" and nx % VEC_WIDTH[storage] == 0:
             out.append(("vector", 0))
+        if flavour(periodic, has_mask) == "periodic" and storage in ("f32", "f16", "bf16"):
+            out.append(("auto", 0))            # two steps per launch
         return out
 
     def measure(self, storage: str, nx: int, ny: int, periodic=(True, True),
@@ -128,7 +132,9 @@ class Tuner:
         if len(cands) == 1:
             return cands[0]
         k = key(storage, nx, ny, periodic, has_mask, g_mode)
-        if k not in self.table:
+        # measured already, and with every candidate there is now
+        known = self.table.get(k, {}).get("candidates", {})
+        if any(f"{v}:{tw}" not in known for v, tw in cands):
             bx, by = bucket(nx), bucket(ny)
             per = (True, True) if flavour(periodic, has_mask) == "periodic" else (True, False)
             times = self.measure(storage, bx, by, per, g_mode=g_mode, **kw)

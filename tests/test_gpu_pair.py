@@ -1,0 +1,88 @@
+"""The two-step kernel against single steps: the same bits, for every format and
+G mode it runs, at the edges of its strips (60 nodes) and lattices narrower than
+one, even and odd widths (paired and elementwise rows at the wrap), heights of
+one band and less, and step counts of every split; alone and in batches (direct
+launches and replayed runs from both parities), and after its second buffer has
+been given back."""
+import numpy as np
+import pytest
+
+from paper_2312_10318_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [(32, 1), (33, 2), (59, 3), (60, 5), (61, 130), (62, 4), (121, 9), (122, 257), (250, 246)]
+
+
+def _lattices(nx, ny, storage, g_mode, seed, n=2, **kw):
+    from paper_2312_10318_gb300 import Lattice
+    rho, ux, uy = W.random_fields(nx, ny, seed=seed, u_amp=0.05, rho_amp=0.01)
+    return [Lattice(nx, ny, 0.7, tau_s2=0.9, g=(2e-5, -1e-5), storage=storage, g_mode=g_mode, **kw)
+            .init(ux, uy, rho) for _ in range(n)]
+
+
+def _same(a, b):
+    (fa, pa), (fb, pb) = a.get_f(with_phi=True), b.get_f(with_phi=True)
+    return np.array_equal(fa, fb) and np.array_equal(pa, pb) and \
+        all(np.array_equal(x, y) for x, y in zip(a.moments(), b.moments()))
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("g_mode", ["lagged", "off"])
+def test_two_steps_equal_single_steps(gpu_lib, storage, g_mode):
+    for k, (nx, ny) in enumerate(SIZES):
+        a, b = _lattices(nx, ny, storage, g_mode, k)
+        a.set_kernel("scalar")
+        assert b.two_step() and not a.two_step()
+        for n in (1, 2, 3, 6, 7):
+            a.step(n)
+            b.step(n)
+            assert a.t == b.t and _same(a, b), (nx, ny, n)
+
+
+def test_two_steps_in_batches(gpu_lib):
+    import torch
+    from paper_2312_10318_gb300.lattice import Batch
+    stream = torch.cuda.Stream()
+    alone, members = [], []
+    for q, (st, nx, ny) in enumerate([("f32", 130, 70), ("f32", 64, 33), ("f16", 61, 40), ("f64", 40, 20),
+                                      ("bf16", 300, 9), ("f32", 200, 65)]):
+        a, b = _lattices(nx, ny, st, "lagged", q, stream=stream)
+        a.set_kernel("scalar")
+        for lat in (a, b):
+            lat.step(q % 2)                    # members at both parities
+        alone.append(a)
+        members.append(b)
+    for group in ([0, 2, 4], [0, 1, 2, 3, 4, 5]):      # all even, then mixed
+        batch = Batch(stream).set([members[k] for k in group])
+        for n in (3, 32, 33, 70, 64, 1, 65):
+            batch.step(n)
+            for k in group:
+                alone[k].step(n)
+        torch.cuda.synchronize()
+        for k in group:
+            assert _same(alone[k], members[k]), (group, k)
+
+
+def test_second_buffer_is_given_back_when_memory_runs_out(gpu_lib):
+    import torch
+    from paper_2312_10318_gb300 import Lattice
+    a, b = _lattices(4096, 2048, "f32", "lagged", 3)
+    assert a.two_step() and b.two_step()
+    held = b.device_bytes()
+    z = torch.zeros((2048, 4096), dtype=torch.float64, device="cuda")
+    for lat in (a, b):
+        lat.init(z + 0.03, z)
+        lat.step(4)                             # odd-level launches: the state may sit in either buffer
+    b.step(2)
+    a.set_kernel("scalar").step(2)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    filler = torch.empty(free - (200 << 20), dtype=torch.uint8, device="cuda")
+    c = Lattice(4096, 2048, 0.7, magic=0.25, storage="f32")    # 436 MB, of which 236 are missing
+    assert not b.two_step() and b.device_bytes() < held and not c.two_step()
+    del filler
+    torch.cuda.empty_cache()
+    for lat in (a, b):
+        lat.step(3)
+    assert _same(a, b)
