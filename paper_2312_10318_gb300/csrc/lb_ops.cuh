@@ -87,25 +87,22 @@ template <typename S> struct Ops {
     // Deterministic FP64 diagnostics; part holds diag_blocks() * 8 doubles.
     static cudaError_t diagnostics(const State& s, double* part, double* out, cudaStream_t st);
     // One batched step of n lattices that share the kernel flavour (FLAV_*),
-    // G mode and the parity of their current level (odd); cur[q] is the Phi
-    // buffer holding member q's previous level, log2_tw[q] its tile width
-    // (scalar flavours).  Launches ceil(n / 64) kernels.
-    static cudaError_t step_group(const State* const* members, const int* cur, const int* log2_tw,
-                                  int n, bool odd, int flavour, int g_mode, cudaStream_t st);
-    // Outlet-ghost pass after step index k of a sequence that started at the
-    // state's current parity and Phi buffer.
-    static cudaError_t ghost_pass(const State& s, int k, cudaStream_t st);
-    // Two-buffer G_CURRENT step q of a sequence starting from s.f (the buffers
-    // alternate with q); the caller swaps s.f / s.f2 after an odd count.
-    static cudaError_t step_ab(const State& s, int q, cudaStream_t st);
+    // G mode and the parity of their current level (odd).
+    static cudaError_t step_group(const State* const* members, int n, bool odd, int flavour, int g_mode,
+                                  cudaStream_t st);
+    // Outlet-ghost pass after a step from the state s (its parity and Phi
+    // buffer before that step).
+    static cudaError_t ghost_pass(const State& s, cudaStream_t st);
+    // Two-buffer G_CURRENT step from s.f to s.f2; the caller swaps them.
+    static cudaError_t step_ab(const State& s, cudaStream_t st);
     // Persistent grid (resident CTAs per SM x SMs) of the TMA-fed two-buffer
     // kernel on the current device; 0 for formats that do not have it.
     static int tma_grid();
     // Whether the TMA-fed two-buffer kernel advances this lattice (FP32,
     // periodic without a mask, G_CURRENT, descriptors present).
     static bool tma_eligible(const State& s);
-    // Two-buffer step q of n such lattices, up to 16 per launch.
-    static cudaError_t step_ab_group(const State* const* members, int n, int q, cudaStream_t st);
+    // Two-buffer step of n such lattices, up to 16 per launch.
+    static cudaError_t step_ab_group(const State* const* members, int n, cudaStream_t st);
 };
 
 int diag_blocks(const State& s);

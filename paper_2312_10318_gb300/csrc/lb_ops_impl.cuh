@@ -48,17 +48,66 @@ static inline dim3 grid2d(const State& s, dim3 b) {
     return dim3((s.nx + b.x - 1) / b.x, (s.ny + b.y - 1) / b.y);
 }
 
+// Launches a step kernel (one that begins with chain_begin()) so that its set-up
+// overlaps the end of the previous kernel of the stream.  Dependent launches of
+// an empty kernel: 2.1 to 3.9 us apart without, 1.45 to 1.9 with (the host's
+// rate).  Us per step without / with: FP64 64^2 6.17 / 4.13, FP32 250 x 246 3.09 /
+// 2.22, 512^2 5.15 / 3.59, 1024^2 10.2 / 8.7, 4096^2 within noise.  Captured
+// launches keep full edges: a replay's dependent kernels start 0.6 to 0.8 us
+// apart, and 0.7 to 1.7 with programmatic ones.
+template <typename P, typename... A>
+static cudaError_t launch_chained(void (*kernel)(P, A...), dim3 g, dim3 b, cudaStream_t st, const P& p, A... rest) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = g;
+    c.blockDim = b;
+    c.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &cs);
+    c.attrs = at;
+    c.numAttrs = cs == cudaStreamCaptureStatusNone ? 1 : 0;
+    void* args[] = {const_cast<P*>(&p), &rest...};
+    return cudaLaunchKernelExC(&c, reinterpret_cast<const void*>(kernel), args);
+}
+
+// Scalar kernels: threads per CTA of a launch over n lattices, and the tile width
+// (a power of two) of one of them.  A lattice narrower than its tile takes the
+// next power of two of its width, so that a warp spans rows instead of idling
+// lanes (8-wide channels ran on a quarter of theirs, and FP64's pipe is busy for
+// all 32).  A launch that would leave SMs without a CTA halves its CTAs, down to
+// a warp: FP64 64^2 in 16 CTAs used 16 SMs' FP64 pipes.
+static inline int scalar_tile(const State& s, int threads) {
+    int tw = s.tile_w > 0 ? s.tile_w : 128;
+    while (tw > threads || (tw > 1 && tw / 2 >= s.nx)) tw /= 2;
+    return tw;
+}
+static inline int scalar_threads(const State* const* m, int n) {
+    int t = 256;
+    for (; t > 32; t /= 2) {
+        long long tiles = 0;
+        for (int q = 0; q < n; ++q) {
+            const int tw = scalar_tile(*m[q], t), th = t / tw;
+            tiles += (long long)((m[q]->nx + tw - 1) / tw) * ((m[q]->ny + th - 1) / th);
+        }
+        if (tiles >= 2 * m[0]->sms) break;
+    }
+    return t;
+}
+
 template <typename S, bool ODD>
 static void launch_step(const State& s, const Args<typename Fmt<S>::C>& a, cudaStream_t st) {
-    const int tw = s.tile_w > 0 ? s.tile_w : 128;
-    const dim3 b(tw, 256 / tw);
+    const State* one = &s;
+    const int t = scalar_threads(&one, 1), tw = scalar_tile(s, t);
+    const dim3 b(tw, t / tw);
     const dim3 g = grid2d(s, b);
     if (s.general) {
-        if (s.g_mode == G_OFF) k_step<S, ODD, true, G_OFF><<<g, b, 0, st>>>(a);
-        else k_step<S, ODD, true, G_LAGGED><<<g, b, 0, st>>>(a);
+        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, true, G_OFF>, g, b, st, a);
+        else launch_chained(k_step<S, ODD, true, G_LAGGED>, g, b, st, a);
     } else {
-        if (s.g_mode == G_OFF) k_step<S, ODD, false, G_OFF><<<g, b, 0, st>>>(a);
-        else k_step<S, ODD, false, G_LAGGED><<<g, b, 0, st>>>(a);
+        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, false, G_OFF>, g, b, st, a);
+        else launch_chained(k_step<S, ODD, false, G_LAGGED>, g, b, st, a);
     }
 }
 
@@ -68,37 +117,32 @@ static void launch_step_vec(const State& s, const Args<typename Fmt<S>::C>& a, c
     const int spr = (s.nx + 32 * V - 1) / (32 * V);
     const long long nseg = (long long)spr * s.ny;
     const int blocks = (int)((nseg + 7) / 8);
-    if (s.g_mode == G_OFF) k_step_vec<S, ODD, G_OFF><<<blocks, 256, 0, st>>>(a, spr);
-    else k_step_vec<S, ODD, G_LAGGED><<<blocks, 256, 0, st>>>(a, spr);
+    if (s.g_mode == G_OFF) launch_chained(k_step_vec<S, ODD, G_OFF>, blocks, 256, st, a, spr);
+    else launch_chained(k_step_vec<S, ODD, G_LAGGED>, blocks, 256, st, a, spr);
 }
 
 template <typename S>
-cudaError_t Ops<S>::step_ab(const State& s, int q, cudaStream_t st) {
+cudaError_t Ops<S>::step_ab(const State& s, cudaStream_t st) {
     using C = typename Fmt<S>::C;
-    State v = s;
-    if (q & 1) {            // odd step of a sequence: the buffers have swapped
-        v.f = s.f2;
-        v.f2 = s.f;
-    }
     if constexpr (std::is_same<S, float>::value) {
         if (tma_eligible(s)) {
             const State* one = &s;
-            return step_ab_group(&one, 1, q, st);
+            return step_ab_group(&one, 1, st);
         }
     }
-    const Args<C> a = make_args<C>(v);
+    const Args<C> a = make_args<C>(s);
     if constexpr (!std::is_same<S, f64dw>::value) {
         if (s.col_h > 0 && !s.general) {
             const int gx = (s.nx + COL_W - 1) / COL_W, bands = (s.ny + s.col_h - 1) / s.col_h;
             const long long warps = (long long)gx * bands;
             const int blocks = (int)((warps + COL_WARPS - 1) / COL_WARPS);
-            k_step_ab_col<S><<<blocks, COL_WARPS * 32, 0, st>>>(a, static_cast<S*>(v.f2), gx, bands, s.col_h);
+            k_step_ab_col<S><<<blocks, COL_WARPS * 32, 0, st>>>(a, static_cast<S*>(s.f2), gx, bands, s.col_h);
             return cudaGetLastError();
         }
     }
     const dim3 g((s.nx + AB_TX - 1) / AB_TX, (s.ny + AB_TY - 1) / AB_TY);
-    if (s.general) k_step_ab<S, true><<<g, AB_TX * AB_TY, 0, st>>>(a, static_cast<S*>(v.f2), 0);
-    else k_step_ab<S, false><<<g, AB_TX * AB_TY, 0, st>>>(a, static_cast<S*>(v.f2), 0);
+    if (s.general) k_step_ab<S, true><<<g, AB_TX * AB_TY, 0, st>>>(a, static_cast<S*>(s.f2), 0);
+    else k_step_ab<S, false><<<g, AB_TX * AB_TY, 0, st>>>(a, static_cast<S*>(s.f2), 0);
     return cudaGetLastError();
 }
 
@@ -125,33 +169,27 @@ bool Ops<S>::tma_eligible(const State& s) {
            s.kerr != nullptr;
 }
 
-// Member k of a TMA launch: lattice s at step q of a sequence (the buffers
-// alternate with q, as in step_ab); returns its tile count.
+// Member k of a TMA launch; returns its tile count.
 template <int MAXL>
-static int tma_member(TmaGroup<MAXL>& g, int k, const State& s, int q) {
-    State v = s;
-    if (q & 1) {
-        v.f = s.f2;
-        v.f2 = s.f;
-    }
-    const int buf = v.f == s.tma_buf[0] ? 0 : 1;
+static int tma_member(TmaGroup<MAXL>& g, int k, const State& s) {
+    const int buf = s.f == s.tma_buf[0] ? 0 : 1;
     g.map[k] = *static_cast<const CUtensorMap*>(s.tma_map[buf]);
-    g.a[k] = make_args<float>(v);
-    g.dst[k] = static_cast<float*>(v.f2);
+    g.a[k] = make_args<float>(s);
+    g.dst[k] = static_cast<float*>(s.f2);
     g.err[k] = s.kerr;
     g.tiles_x[k] = (s.nx + AB_TX - 1) / AB_TX;
     return g.tiles_x[k] * ((s.ny + TMA_TH - 1) / TMA_TH);
 }
 
 template <int MAXL>
-static cudaError_t launch_tma(const State* const* m, int n, int q, cudaStream_t st) {
+static cudaError_t launch_tma(const State* const* m, int n, cudaStream_t st) {
     TmaGroup<MAXL> g;
     g.n = n;
     g.tile_begin[0] = 0;
     int grid = 0;
     long long wait = 0;
     for (int k = 0; k < n; ++k) {
-        g.tile_begin[k + 1] = g.tile_begin[k] + tma_member(g, k, *m[k], q);
+        g.tile_begin[k + 1] = g.tile_begin[k] + tma_member(g, k, *m[k]);
         grid = k == 0 || m[k]->tma_grid < grid ? m[k]->tma_grid : grid;
         wait = k == 0 || m[k]->wait_limit < wait ? m[k]->wait_limit : wait;
     }
@@ -162,19 +200,19 @@ static cudaError_t launch_tma(const State* const* m, int n, int q, cudaStream_t 
 }
 
 template <typename S>
-cudaError_t Ops<S>::step_ab_group(const State* const* members, int n, int q, cudaStream_t st) {
+cudaError_t Ops<S>::step_ab_group(const State* const* members, int n, cudaStream_t st) {
     if constexpr (std::is_same<S, float>::value) {
         for (int k = 0; k < n; ++k)
             if (!tma_eligible(*members[k])) return cudaErrorInvalidValue;
-        if (n == 1) return launch_tma<1>(members, 1, q, st);
+        if (n == 1) return launch_tma<1>(members, 1, st);
         for (int k0 = 0; k0 < n; k0 += TMA_GROUP_MAX) {
             const int c = n - k0 < TMA_GROUP_MAX ? n - k0 : TMA_GROUP_MAX;
-            const cudaError_t e = launch_tma<TMA_GROUP_MAX>(members + k0, c, q, st);
+            const cudaError_t e = launch_tma<TMA_GROUP_MAX>(members + k0, c, st);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
     } else {
-        (void)members; (void)n; (void)q; (void)st;
+        (void)members; (void)n; (void)st;
         return cudaErrorInvalidValue;
     }
 }
@@ -198,7 +236,7 @@ template <typename S>
 cudaError_t Ops<S>::step(State& s, cudaStream_t st) {
     using C = typename Fmt<S>::C;
     if (s.g_mode == G_CURRENT) {
-        const cudaError_t e = step_ab(s, 0, st);
+        const cudaError_t e = step_ab(s, st);
         void* t = s.f;
         s.f = s.f2;
         s.f2 = t;
@@ -215,8 +253,8 @@ cudaError_t Ops<S>::step(State& s, cudaStream_t st) {
     }
     if (s.nghost > 0) {
         const int t = 128, g = (s.nghost + t - 1) / t;
-        if (s.parity == 0) k_ghosts<S, true><<<g, t, 0, st>>>(a, s.ghosts, s.nghost);
-        else k_ghosts<S, false><<<g, t, 0, st>>>(a, s.ghosts, s.nghost);
+        if (s.parity == 0) launch_chained(k_ghosts<S, true>, g, t, st, a, s.ghosts, s.nghost);
+        else launch_chained(k_ghosts<S, false>, g, t, st, a, s.ghosts, s.nghost);
     }
     s.parity ^= 1;
     if (s.g_mode == G_LAGGED) s.cur ^= 1;
@@ -310,16 +348,17 @@ cudaError_t Ops<S>::diagnostics(const State& s, double* part, double* out, cudaS
 
 // FLAV: FLAV_GENERAL, FLAV_PERIODIC (scalar kernels) or FLAV_VECTOR.
 template <typename S, bool ODD, int FLAV, int GMODE, int MAXL>
-static cudaError_t launch_group(const State* const* m, const int* cur, const int* l2tw, int n,
-                                cudaStream_t st) {
+static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     using C = typename Fmt<S>::C;
     constexpr int V = Pk<S>::V;
     GroupParams<C, MAXL> p;
     p.n = n;
     int tiles = 0;
+    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n);
+    p.log2_threads = 0;
+    while ((1 << p.log2_threads) < threads) ++p.log2_threads;
     for (int q = 0; q < n; ++q) {
-        State v = *m[q];
-        v.cur = cur[q];
+        const State& v = *m[q];
         p.a[q] = make_args<C>(v);
         p.tile_begin[q] = tiles;
         if (FLAV == FLAV_VECTOR) {
@@ -329,8 +368,9 @@ static cudaError_t launch_group(const State* const* m, const int* cur, const int
             p.log2_tw[q] = 0;
             tiles += (int)(((long long)p.segs[q] * v.ny + 7) / 8);
         } else {
-            const int tw = 1 << l2tw[q], th = BATCH_THREADS / tw;
-            p.log2_tw[q] = l2tw[q];
+            const int tw = scalar_tile(v, threads), th = threads / tw;
+            p.log2_tw[q] = 0;
+            while ((1 << p.log2_tw[q]) < tw) ++p.log2_tw[q];
             p.segs[q] = 0;
             p.tiles_x[q] = (v.nx + tw - 1) / tw;
             p.inv_d[q] = 1.0f / (float)p.tiles_x[q];
@@ -339,44 +379,39 @@ static cudaError_t launch_group(const State* const* m, const int* cur, const int
     }
     p.tile_begin[n] = tiles;
     if (FLAV == FLAV_VECTOR)
-        k_step_group_vec<S, ODD, GMODE, MAXL><<<tiles, BATCH_THREADS, 0, st>>>(p);
+        return launch_chained(k_step_group_vec<S, ODD, GMODE, MAXL>, tiles, BATCH_THREADS, st, p);
     else
-        k_step_group<S, ODD, FLAV == FLAV_GENERAL, GMODE, MAXL><<<tiles, BATCH_THREADS, 0, st>>>(p);
-    return cudaGetLastError();
+        return launch_chained(k_step_group<S, ODD, FLAV == FLAV_GENERAL, GMODE, MAXL>, tiles, threads, st, p);
 }
 
 template <typename S, bool ODD, int FLAV, int GMODE>
-static cudaError_t launch_group_sized(const State* const* m, const int* cur, const int* l2tw,
-                                      int n, cudaStream_t st) {
-    for (int q0 = 0; q0 < n; q0 += 64) {
-        const int c = n - q0 < 64 ? n - q0 : 64;
-        const cudaError_t e = c <= 4
-            ? launch_group<S, ODD, FLAV, GMODE, 4>(m + q0, cur + q0, l2tw + q0, c, st)
-            : launch_group<S, ODD, FLAV, GMODE, 64>(m + q0, cur + q0, l2tw + q0, c, st);
+static cudaError_t launch_group_sized(const State* const* m, int n, cudaStream_t st) {
+    for (int q0 = 0; q0 < n; q0 += GROUP_MAX) {
+        const int c = n - q0 < GROUP_MAX ? n - q0 : GROUP_MAX;
+        const cudaError_t e = c <= 4 ? launch_group<S, ODD, FLAV, GMODE, 4>(m + q0, c, st)
+                                     : launch_group<S, ODD, FLAV, GMODE, GROUP_MAX>(m + q0, c, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
 template <typename S, bool ODD, int FLAV>
-static cudaError_t launch_group_g(const State* const* m, const int* cur, const int* l2tw, int n,
-                                  int g_mode, cudaStream_t st) {
-    return g_mode == G_OFF ? launch_group_sized<S, ODD, FLAV, G_OFF>(m, cur, l2tw, n, st)
-                           : launch_group_sized<S, ODD, FLAV, G_LAGGED>(m, cur, l2tw, n, st);
+static cudaError_t launch_group_g(const State* const* m, int n, int g_mode, cudaStream_t st) {
+    return g_mode == G_OFF ? launch_group_sized<S, ODD, FLAV, G_OFF>(m, n, st)
+                           : launch_group_sized<S, ODD, FLAV, G_LAGGED>(m, n, st);
 }
 
 template <typename S>
-cudaError_t Ops<S>::step_group(const State* const* m, const int* cur, const int* l2tw, int n,
-                               bool odd, int flavour, int g_mode, cudaStream_t st) {
+cudaError_t Ops<S>::step_group(const State* const* m, int n, bool odd, int flavour, int g_mode, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     if (odd) {
-        if (flavour == FLAV_GENERAL) return launch_group_g<S, true, FLAV_GENERAL>(m, cur, l2tw, n, g_mode, st);
-        if (flavour == FLAV_VECTOR) return launch_group_g<S, true, FLAV_VECTOR>(m, cur, l2tw, n, g_mode, st);
-        return launch_group_g<S, true, FLAV_PERIODIC>(m, cur, l2tw, n, g_mode, st);
+        if (flavour == FLAV_GENERAL) return launch_group_g<S, true, FLAV_GENERAL>(m, n, g_mode, st);
+        if (flavour == FLAV_VECTOR) return launch_group_g<S, true, FLAV_VECTOR>(m, n, g_mode, st);
+        return launch_group_g<S, true, FLAV_PERIODIC>(m, n, g_mode, st);
     }
-    if (flavour == FLAV_GENERAL) return launch_group_g<S, false, FLAV_GENERAL>(m, cur, l2tw, n, g_mode, st);
-    if (flavour == FLAV_VECTOR) return launch_group_g<S, false, FLAV_VECTOR>(m, cur, l2tw, n, g_mode, st);
-    return launch_group_g<S, false, FLAV_PERIODIC>(m, cur, l2tw, n, g_mode, st);
+    if (flavour == FLAV_GENERAL) return launch_group_g<S, false, FLAV_GENERAL>(m, n, g_mode, st);
+    if (flavour == FLAV_VECTOR) return launch_group_g<S, false, FLAV_VECTOR>(m, n, g_mode, st);
+    return launch_group_g<S, false, FLAV_PERIODIC>(m, n, g_mode, st);
 }
 
 template <typename S, int GMODE, int MAXL>
@@ -397,20 +432,19 @@ static cudaError_t launch_pair(const State* const* m, int n, cudaStream_t st) {
         tiles += (int)((warps + PAIR_WARPS - 1) / PAIR_WARPS);
     }
     p.tile_begin[n] = tiles;
-    k_step_pair<S, GMODE, MAXL><<<tiles, PAIR_WARPS * 32, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_chained(k_step_pair<S, GMODE, MAXL>, tiles, PAIR_WARPS * 32, st, p);
 }
 
 template <typename S>
 cudaError_t Ops<S>::step_pair(const State* const* m, int n, cudaStream_t st) {
     if constexpr (sizeof(S) <= 4) {
-        for (int q0 = 0; q0 < n; q0 += 64) {
-            const int c = n - q0 < 64 ? n - q0 : 64;
+        for (int q0 = 0; q0 < n; q0 += GROUP_MAX) {
+            const int c = n - q0 < GROUP_MAX ? n - q0 : GROUP_MAX;
             cudaError_t e;
             if (m[q0]->g_mode == G_OFF)
-                e = c <= 4 ? launch_pair<S, G_OFF, 4>(m + q0, c, st) : launch_pair<S, G_OFF, 64>(m + q0, c, st);
+                e = c <= 4 ? launch_pair<S, G_OFF, 4>(m + q0, c, st) : launch_pair<S, G_OFF, GROUP_MAX>(m + q0, c, st);
             else
-                e = c <= 4 ? launch_pair<S, G_LAGGED, 4>(m + q0, c, st) : launch_pair<S, G_LAGGED, 64>(m + q0, c, st);
+                e = c <= 4 ? launch_pair<S, G_LAGGED, 4>(m + q0, c, st) : launch_pair<S, G_LAGGED, GROUP_MAX>(m + q0, c, st);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -421,16 +455,13 @@ cudaError_t Ops<S>::step_pair(const State* const* m, int n, cudaStream_t st) {
 }
 
 template <typename S>
-cudaError_t Ops<S>::ghost_pass(const State& s, int k, cudaStream_t st) {
+cudaError_t Ops<S>::ghost_pass(const State& s, cudaStream_t st) {
     if (s.nghost <= 0) return cudaSuccess;
     using C = typename Fmt<S>::C;
-    State v = s;
-    v.parity = s.parity ^ (k & 1);
-    if (s.g_mode == G_LAGGED) v.cur = s.cur ^ (k & 1);
-    const Args<C> a = make_args<C>(v);
+    const Args<C> a = make_args<C>(s);
     const int t = 128, g = (s.nghost + t - 1) / t;
-    if (v.parity == 0) k_ghosts<S, true><<<g, t, 0, st>>>(a, s.ghosts, s.nghost);
-    else k_ghosts<S, false><<<g, t, 0, st>>>(a, s.ghosts, s.nghost);
+    if (s.parity == 0) launch_chained(k_ghosts<S, true>, g, t, st, a, s.ghosts, s.nghost);
+    else launch_chained(k_ghosts<S, false>, g, t, st, a, s.ghosts, s.nghost);
     return cudaGetLastError();
 }
 

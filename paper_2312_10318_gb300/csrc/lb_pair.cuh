@@ -117,6 +117,7 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_BLOCKS)
     k_step_pair(const __grid_constant__ PairParams<MAXL> p) {
     using K = Pr<S>;
     using P = typename K::P;
+    chain_begin();
     const int b = (int)blockIdx.x;
     int lo = 0, hi = p.n - 1;
     while (lo < hi) {

@@ -388,6 +388,7 @@ __device__ __forceinline__ void seg_step(const Args<typename Fmt<S>::C>& a, int 
 // owns segment s = 8 b + w of the (row, segment) list.
 template <typename S, bool ODD, int GMODE>
 __global__ void __launch_bounds__(256, sizeof(S) == 2 ? 4 : 3) k_step_vec(Args<typename Fmt<S>::C> a, int segs_per_row) {
+    chain_begin();
     constexpr int V = Pk<S>::V;
     const int lane = (int)threadIdx.x & 31;
     const long long s = (long long)blockIdx.x * 8 + ((int)threadIdx.x >> 5);
