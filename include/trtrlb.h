@@ -323,8 +323,9 @@ int trtrlb_get_kernel(trtrlb_t h, int32_t* vector, int32_t* tile_w);
 int trtrlb_step_kernel(trtrlb_t h, int32_t* kind);
 
 /* Whether runs of steps advance this lattice two steps per launch (*on = 1): G
- * lagged or off, FP32, FP16 or BF16 storage, periodic in both directions without
- * a mask, nx >= 32, TRTRLB_KERNEL_AUTO, and a second population buffer, which
+ * lagged or off, FP32, FP16 or BF16 storage, nx >= 32, no node of the halo classes
+ * and no outlet ghost with a colliding node at x + 1 (any row of the three),
+ * TRTRLB_KERNEL_AUTO, and a second population buffer, which
  * trtrlb_create allocates while such buffers take no more than 4 GiB or leave
  * half of the device's memory free, and which goes back when a later allocation of the library would fail.  The
  * two steps start at an odd level: a run from an even one begins with a single

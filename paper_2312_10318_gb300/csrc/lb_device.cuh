@@ -96,6 +96,24 @@ template <typename C> struct Args {
     C zh_dr;              // rho0 - outlet_rho of the Zou-He pressure outlet
 };
 
+// Single-rounding operations.  Every kernel writes the collision with these, so
+// that where a product and a sum share one rounding (ffma) is fixed here and
+// not chosen by the compiler per kernel: the one-step, two-step, batched and
+// two-buffer kernels give the same bits for the same node.
+__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float rrcp(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
+__device__ __forceinline__ df64 radd(const df64& a, const df64& b) { return a + b; }
+__device__ __forceinline__ df64 rsub(const df64& a, const df64& b) { return a - b; }
+__device__ __forceinline__ df64 rmul(const df64& a, const df64& b) { return a * b; }
+
 // Zou-He constant-pressure outlet (Sec. III D) on the shifted populations
 // d_i = f_i - w_i rho0 of a node on the last column of a lattice open in x:
 // the three populations entering across the edge (e_x = -1) are rebuilt so
@@ -107,12 +125,12 @@ template <typename C> struct Args {
 //   d_7 = d_5 + (d_2 - d_4)/2 - j/6.
 template <typename C>
 __device__ __forceinline__ void zh_fill(C (&d)[9], C zh_dr) {
-    const C j = (d[0] + d[2] + d[4]) + C(2) * (d[1] + d[5] + d[8]) + zh_dr;
-    const C t = C(0.5) * (d[2] - d[4]);
-    const C j6 = j * C(1.0 / 6.0);
-    d[3] = d[1] - C(4) * j6;
-    d[6] = d[8] - t - j6;
-    d[7] = d[5] + t - j6;
+    const C j = radd(radd(radd(radd(d[0], d[2]), d[4]), rmul(C(2), radd(radd(d[1], d[5]), d[8]))), zh_dr);
+    const C t = rmul(C(0.5), rsub(d[2], d[4]));
+    const C j6 = rmul(j, C(1.0 / 6.0));
+    d[3] = rsub(d[1], rmul(C(4), j6));
+    d[6] = rsub(rsub(d[8], t), j6);
+    d[7] = rsub(radd(d[5], t), j6);
 }
 
 // Neighbourhood of node (x, y): wrapped coordinates and out-of-domain flags.
@@ -286,21 +304,6 @@ __device__ __forceinline__ void collide_dw(const df64 (&d)[9], df64 dpx, df64 dp
     phx = ruxx * ux;
     phy = ruyy * uy;
 }
-
-// Single-rounding operations.  Every kernel writes the collision with these, so
-// that where a product and a sum share one rounding (ffma) is fixed here and
-// not chosen by the compiler per kernel: the one-step, two-step, batched and
-// two-buffer kernels give the same bits for the same node.
-__device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
-__device__ __forceinline__ float rmul(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ float rfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ float rrcp(float a) { return __frcp_rn(a); }
-__device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
-__device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
-__device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
 
 // Raw moments of one node's shifted populations and its eq11 velocity: the
 // first half of the collision, which the two-buffer TMA kernel also uses for

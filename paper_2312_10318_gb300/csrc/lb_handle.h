@@ -18,6 +18,7 @@ struct trtrlb_lattice {
     void* phi;           // both Phi buffers in one allocation
     uint8_t* mask;
     uint8_t* seg;        // interior row segments of a general lattice (State::seg), or null
+    unsigned* pair_map;  // State::pinfo and State::pspecial of a general lattice, or null
     int* ghosts;
     double* stage;       // FP64 staging for host transfers and comparisons
     int stage_fields;    // its size in fields of nx * ny doubles (3, 4 or 11)

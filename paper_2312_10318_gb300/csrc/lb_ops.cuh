@@ -33,12 +33,15 @@ constexpr long long kDefaultWaitLimit = 1ll << 22;
 
 // Two-step kernel (lb_pair.cuh): nodes of a row a warp updates, warps per CTA.
 constexpr int PAIR_W = 60, PAIR_WARPS = 4;
+inline int pair_strips(int nx) { return (nx + PAIR_W - 1) / PAIR_W; }
 
 struct State {
     void* f;              // populations, S[9][ny][pitch]
     void* f2;             // second buffer: of the two-buffer G_CURRENT kernel, or of
                           // the two-step kernel (else null)
     bool pair;            // the two-step kernel advances this lattice from odd levels
+    const unsigned* pinfo;     // its maps of a general lattice (lb_pair.cuh): a word per node,
+    const unsigned* pspecial;  // [ny][pitch], and a bit per strip and row, [strips][(ny + 31) / 32]
     int sms;              // multiprocessors of the device
     void* phi[2];         // Phi buffers, C[2][ny][pitch]
     int cur;              // phi[cur] holds the previous level
@@ -77,6 +80,8 @@ template <typename S> struct Ops {
     // and G mode) in one launch per 64; the caller swaps f and f2, and with Phi
     // lagged the Phi buffers.
     static cudaError_t step_pair(const State* const* members, int n, cudaStream_t st);
+    // Fills a general lattice's maps of the two-step kernel.
+    static cudaError_t pair_maps(const State& s, unsigned* info, unsigned* special, cudaStream_t st);
     static cudaError_t phi_static(State& s, cudaStream_t st);
     static cudaError_t init(State& s, const double* rho, const double* ux, const double* uy,
                             cudaStream_t st);

@@ -414,25 +414,56 @@ cudaError_t Ops<S>::step_group(const State* const* m, int n, bool odd, int flavo
     return launch_group_g<S, false, FLAV_PERIODIC>(m, n, g_mode, st);
 }
 
-template <typename S, int GMODE, int MAXL>
+template <typename S, bool GENERAL, int GMODE, int MAXL>
 static cudaError_t launch_pair(const State* const* m, int n, cudaStream_t st) {
     PairParams<MAXL> p;
     p.n = n;
-    const int band = pair_band_rows(m, n, (long long)m[0]->sms * PAIR_BLOCKS * PAIR_WARPS);
+    // general lattices leave a sixteenth of the slots to the parts of split tiles
+    const long long slots = (long long)m[0]->sms * PAIR_BLOCKS * PAIR_WARPS;
+    const int band = pair_band_rows(m, n, GENERAL ? slots - slots / 16 : slots);
+    p.split = GENERAL ? pair_split(band) : 1;
     int tiles = 0;
     for (int q = 0; q < n; ++q) {
         const State& s = *m[q];
         p.a[q] = make_args<float>(s);
         p.out[q] = s.f2;
+        p.info[q] = s.pinfo;
+        p.special[q] = s.pspecial;
         p.tile_begin[q] = tiles;
         p.strips[q] = pair_strips(s.nx);
         p.inv_d[q] = 1.0f / (float)p.strips[q];
         p.band[q] = band;
         const long long warps = (long long)p.strips[q] * ((s.ny + band - 1) / band);
-        tiles += (int)((warps + PAIR_WARPS - 1) / PAIR_WARPS);
+        tiles += p.split * (int)((warps + PAIR_WARPS - 1) / PAIR_WARPS);
     }
     p.tile_begin[n] = tiles;
-    return launch_chained(k_step_pair<S, GMODE, MAXL>, tiles, PAIR_WARPS * 32, st, p);
+    return launch_chained(k_step_pair<S, GENERAL, GMODE, MAXL>, tiles, PAIR_WARPS * 32, st, p);
+}
+
+template <typename S, bool GENERAL>
+static cudaError_t launch_pair_g(const State* const* m, int n, cudaStream_t st) {
+    if (m[0]->g_mode == G_OFF)
+        return n <= 4 ? launch_pair<S, GENERAL, G_OFF, 4>(m, n, st) : launch_pair<S, GENERAL, G_OFF, GROUP_MAX>(m, n, st);
+    return n <= 4 ? launch_pair<S, GENERAL, G_LAGGED, 4>(m, n, st)
+                  : launch_pair<S, GENERAL, G_LAGGED, GROUP_MAX>(m, n, st);
+}
+
+template <typename S>
+cudaError_t Ops<S>::pair_maps(const State& s, unsigned* info, unsigned* special, cudaStream_t st) {
+    if constexpr (sizeof(S) <= 4) {
+        const Args<float> a = make_args<float>(s);
+        const int strips = pair_strips(s.nx), words = (s.ny + 31) / 32;
+        const cudaError_t e = cudaMemsetAsync(special, 0, sizeof(unsigned) * (size_t)strips * words, st);
+        if (e != cudaSuccess) return e;
+        const dim3 b(32, 8);
+        k_pair_info<<<grid2d(s, b), b, 0, st>>>(a, info);
+        const long long warps = (long long)strips * s.ny;
+        k_pair_special<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(a, info, special, strips, words);
+        return cudaGetLastError();
+    } else {
+        (void)s; (void)info; (void)special; (void)st;
+        return cudaErrorInvalidValue;
+    }
 }
 
 template <typename S>
@@ -440,11 +471,8 @@ cudaError_t Ops<S>::step_pair(const State* const* m, int n, cudaStream_t st) {
     if constexpr (sizeof(S) <= 4) {
         for (int q0 = 0; q0 < n; q0 += GROUP_MAX) {
             const int c = n - q0 < GROUP_MAX ? n - q0 : GROUP_MAX;
-            cudaError_t e;
-            if (m[q0]->g_mode == G_OFF)
-                e = c <= 4 ? launch_pair<S, G_OFF, 4>(m + q0, c, st) : launch_pair<S, G_OFF, GROUP_MAX>(m + q0, c, st);
-            else
-                e = c <= 4 ? launch_pair<S, G_LAGGED, 4>(m + q0, c, st) : launch_pair<S, G_LAGGED, GROUP_MAX>(m + q0, c, st);
+            const cudaError_t e = m[q0]->general ? launch_pair_g<S, true>(m + q0, c, st)
+                                                 : launch_pair_g<S, false>(m + q0, c, st);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;

@@ -1,5 +1,4 @@
-// Two time steps in one launch, for lattices periodic in x and y without a mask
-// (lagged Phi or no G; FP32 and 16-bit storage).
+// Two time steps in one launch (lagged Phi or no G; FP32 and 16-bit storage).
 //
 // A step on its own is bound by HBM (FP32, 88 B per node) or by its launch and
 // tail (lattices in L2); two steps together read and write the state once.  The
@@ -20,6 +19,10 @@
 // rows per band are collided once more than they are stored.  The next row's
 // loads are issued before the two collisions that hide them.
 //
+// On a lattice with walls, a mask or open edges, tiles (a strip's band) whose
+// nodes and links are all plain take the same walk (pair_walk); the others
+// pair_walk_general, which looks at one word per node.
+//
 // The same arithmetic in the same order as two single steps, each population
 // rounded to the storage type between them: the same bits.
 //
@@ -31,7 +34,9 @@
 // the rest is bound by issue (FP16 77 % of the slots, 187 instructions per node
 // and step) and, below 1024^2, by the walk of the band.  4 resident CTAs of 4
 // warps (128 registers, no spills); 5 for the 16-bit formats (102 registers)
-// were slower (4096^2 108.8, 1024^2 11.3).
+// were slower (4096^2 108.8, 1024^2 11.3).  With walls and masks, whole solves:
+// creeping flow 4096 x 2048 FP32, 50 steps, 7.3 ms in single steps, 4.4 here;
+// channel 2048 x 1024 FP16, 200 steps, 4.4 and 3.5.
 #pragma once
 #include "lb_batch.cuh"
 #include "lb_device.cuh"
@@ -40,7 +45,6 @@
 namespace trt {
 
 constexpr int PAIR_ROWS = 128, PAIR_ROWS_MIN = 2;   // rows of a band
-inline int pair_strips(int nx) { return (nx + PAIR_W - 1) / PAIR_W; }
 
 // ---- two consecutive nodes of one population ----------------------------------
 // up(p): [x - 1, x] of the pair at [x, x + 1]; down(p): [x + 1, x + 2].
@@ -102,39 +106,35 @@ inline int pair_band_rows(const State* const* m, int n, long long slots) {
     return lo;
 }
 
+// Parts of a tile of a general lattice that is not plain.  Its rows take longer
+// (walls on the way in and out, elementwise loads), and in one wave the longest
+// walk is the launch's length: such a tile is walked by up to 8 warps of at least
+// 8 rows each.  They come first; where the tile is plain they leave at once.
+// Whole solves, ms, 1 / 2 / 8 parts at most: creeping flow 4096 x 2048 FP32 6.2 /
+// 5.4 / 4.4, channel 2048 x 1024 FP16 (bands of 16 rows) 4.2 / 3.5 / 3.5; parts of
+// 4 rows and more, channel 3.6.
+inline int pair_split(int band) { return band < 16 ? 1 : (band >= 64 ? 8 : band / 8); }
+
 template <int MAXL> struct PairParams {
     int n;                       // lattices in this launch
+    int split;                   // parts of a tile that is not plain (general lattices)
     int tile_begin[MAXL + 1];    // prefix sums of CTAs
     int strips[MAXL];            // column strips of PAIR_W nodes
     int band[MAXL];              // rows per band
     float inv_d[MAXL];           // 1 / strips, rounded
     void* out[MAXL];             // the other population buffer
+    const unsigned* info[MAXL];     // general lattices: State::pinfo, State::pspecial
+    const unsigned* special[MAXL];
     Args<float> a[MAXL];
 };
 
-template <typename S, int GMODE, int MAXL>
-__global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_BLOCKS)
-    k_step_pair(const __grid_constant__ PairParams<MAXL> p) {
+// The walk of one warp down rows y0 .. y1 - 1 of a strip whose rows y0 - 1 .. y1
+// hold plain fluid nodes only, none of them linked to anything else.
+template <typename S, int GMODE>
+__device__ __forceinline__ void pair_walk(const Args<float>& a, S* __restrict__ O, int strip, int y0, int y1, int lane) {
     using K = Pr<S>;
     using P = typename K::P;
-    chain_begin();
-    const int b = (int)blockIdx.x;
-    int lo = 0, hi = p.n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (p.tile_begin[mid] <= b) lo = mid;
-        else hi = mid - 1;
-    }
-    const Args<float>& a = p.a[lo];
     const int nx = a.nx, ny = a.ny, pitch = a.pitch;
-    const int strips = p.strips[lo], band_h = p.band[lo];
-    const int lane = (int)threadIdx.x & 31;
-    const int w = (b - p.tile_begin[lo]) * PAIR_WARPS + ((int)threadIdx.x >> 5);
-    int band, strip;
-    tile_divmod(w, strips, p.inv_d[lo], band, strip);
-    const int y0 = band * band_h;
-    if (y0 >= ny) return;   // the whole warp leaves together
-    const int y1 = y0 + band_h < ny ? y0 + band_h : ny;
 
     // this lane's two columns c, c + 1 and where they lie in the lattice
     const int c = strip * PAIR_W - 2 + 2 * lane;
@@ -147,7 +147,6 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_BLOCKS)
     const bool st_a = inner && c < nx, st_b = inner && c + 1 < nx;
 
     const S* __restrict__ F = static_cast<const S*>(a.f);
-    S* __restrict__ O = static_cast<S*>(p.out[lo]);
     const long long plane = a.plane;
 
     // the row that is loaded next, and the offsets of it and its two neighbours
@@ -276,6 +275,304 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_BLOCKS)
         hym = hyc;
         hyc = hy;
     }
+}
+
+// ---- walls, masks and open edges -----------------------------------------------
+// What a node's two steps need of its surroundings, one word per node of a
+// general lattice: bit i - 1: f_i arrives from a wall (x - e_i is solid, a moving
+// wall or outside), so it is the node's own f*_ibar of the step before; bit
+// 7 + i: f*_i leaves into a moving wall (Ladd's correction); bits 16 ..: class.
+enum : unsigned { PI_CLASS_SHIFT = 16, PI_OUTSIDE = 0xffu | ((unsigned)SOLID << PI_CLASS_SHIFT) };
+
+static __global__ void k_pair_info(Args<float> a, unsigned* info) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= a.nx || y >= a.ny) return;
+    int nb[9], kind[9];
+    links<true>(a, x, y, nb, kind);
+    unsigned v = (unsigned)(a.mask ? a.mask[nb[0]] : FLUID) << PI_CLASS_SHIFT;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+        if (kind[opp(i)] != K_STREAM) v |= 1u << (i - 1);
+        if (kind[i] == K_MOVING) v |= 1u << (7 + i);
+    }
+    info[nb[0]] = v;
+}
+
+// Bit y % 32 of special[strip][y / 32]: a node of the strip's 64 columns in row y
+// is not plain fluid or has a link that is not.  One warp per strip and row.
+static __global__ void k_pair_special(Args<float> a, const unsigned* __restrict__ info, unsigned* special, int strips,
+                                      int words) {
+    const int lane = (int)threadIdx.x & 31;
+    const long long w = (long long)blockIdx.x * (blockDim.x / 32) + ((int)threadIdx.x >> 5);
+    if (w >= (long long)strips * a.ny) return;   // the whole warp leaves together
+    const int strip = (int)(w / a.ny), y = (int)(w % a.ny);
+    bool any = false;
+    for (int k = 0; k < 2; ++k) {
+        const int c = strip * PAIR_W - 2 + 2 * lane + k;
+        const bool in = (unsigned)c < (unsigned)a.nx;
+        const int x = (c % a.nx + a.nx) % a.nx;
+        any = any || (!in && !a.px) || info[(long long)y * a.pitch + x] != (unsigned)FLUID << PI_CLASS_SHIFT;
+    }
+    if (__any_sync(0xffffffffu, any) && lane == 0) atomicOr(&special[(long long)strip * words + (y >> 5)], 1u << (y & 31));
+}
+
+// The same walk over any nodes.  The first step reads each population of a node
+// straight from the slot that holds it (an odd level's rule, pop_loc), so that it
+// is valid on all 64 columns and the second on 62: an outlet ghost in the first
+// column stored takes what its inward neighbour, one column before, emits.
+template <typename S, int GMODE>
+__device__ __forceinline__ void pair_walk_general(const Args<float>& a, S* __restrict__ O,
+                                               const unsigned* __restrict__ info, int strip, int y0, int y1, int lane) {
+    using K = Pr<S>;
+    using P = typename K::P;
+    const int nx = a.nx, ny = a.ny, pitch = a.pitch;
+    const long long plane = a.plane;
+    const S* __restrict__ F = static_cast<const S*>(a.f);
+    const int c = strip * PAIR_W - 2 + 2 * lane;
+    // columns c - 1 .. c + 2: wrapped, or, past an open edge, the nearest one (never
+    // read as a neighbour there: those links are walls)
+    int col[4];
+    bool out[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int x = c - 1 + k;
+        out[k] = !a.px && (unsigned)x >= (unsigned)nx;
+        col[k] = a.px ? (x % nx + nx) % nx : (x < 0 ? 0 : (x >= nx ? nx - 1 : x));
+    }
+    const bool inner = lane >= 1 && lane <= 30;
+    // rows: wrapped, or past an open edge the nearest one, and whether they lie there
+    auto row_out = [&](int y) { return !a.py && (unsigned)y >= (unsigned)ny; };
+    auto row_of = [&](int y) {
+        return (unsigned)((a.py ? ((y % ny) + ny) % ny : (y < 0 ? 0 : (y >= ny ? ny - 1 : y))) * pitch);
+    };
+    auto load_info = [&](unsigned row, bool ro) {
+        uint2 v;
+        v.x = ro || out[1] ? (unsigned)PI_OUTSIDE : info[row + (unsigned)col[1]];
+        v.y = ro || out[2] ? (unsigned)PI_OUTSIDE : info[row + (unsigned)col[2]];
+        return v;
+    };
+    auto cls = [](unsigned v) { return (int)(v >> PI_CLASS_SHIFT); };
+    auto phi_row = [&](int comp, unsigned row, bool o) {   // Phi of the level before at this lane's two nodes
+        const float* q = a.phi_in + comp * plane + row;
+        return make_float2(o || out[1] ? 0.f : q[col[1]], o || out[2] ? 0.f : q[col[2]]);
+    };
+    // one node's collision with its corrections into moving walls
+    auto collide_node = [&](float (&d)[9], unsigned v, float dpx, float dpy, float (&o)[9], float& hx, float& hy) {
+        if (cls(v) == PRESSURE) zh_fill<float>(d, a.zh_dr);
+        collide<float>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, hx, hy);
+        if (v & 0xff00u) {
+#pragma unroll
+            for (int i = 1; i < 9; ++i)
+                if (v >> (7 + i) & 1u) o[i] -= a.corr[i];
+        }
+    };
+
+    P C[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) C[i] = K::make(0.f, 0.f);
+    P B2 = C[2], B5 = C[5], B6 = C[6];
+    const float2 z2 = make_float2(0.f, 0.f);
+    float2 hxc = z2, hym = z2, hyc = z2, pym = z2, pyc = z2;
+    if (GMODE == G_LAGGED) {
+        pym = phi_row(1, row_of(y0 - 2), row_out(y0 - 2));
+        pyc = phi_row(1, row_of(y0 - 1), row_out(y0 - 1));
+    }
+    // the row loaded next, r, with r - 1 and r + 1; info is read a row ahead of that,
+    // because it decides where the row's populations are
+    unsigned rm = row_of(y0 - 2), r0 = row_of(y0 - 1), rp = row_of(y0);
+    int yp = (int)(rp / (unsigned)pitch);
+    uint2 vq = make_uint2(PI_OUTSIDE, PI_OUTSIDE), v = load_info(r0, row_out(y0 - 1)), vn = load_info(rp, row_out(y0));
+    float l0 = 0.f, l3 = 0.f;          // Phi_xxx beside the strip (lanes 0 and 31)
+    S la[9], lb[9];
+    float2 lpx = z2, lpy = z2;
+    // whether a row has a node that is not plain (all bits of a plain fluid node's
+    // word are 0); the others skip what walls, ghosts and outlets need
+    auto special = [](uint2 w) { return __any_sync(0xffffffffu, (w.x | w.y) != 0u) != 0; };
+    auto load_row = [&](int r, uint2 w) {
+        if (special(w)) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const unsigned row = ey(i) > 0 ? rm : (ey(i) < 0 ? rp : r0);
+                const bool wa = i > 0 && (w.x >> (i > 0 ? i - 1 : 0) & 1u), wb = i > 0 && (w.y >> (i > 0 ? i - 1 : 0) & 1u);
+                la[i] = F[(wa ? i : opp(i)) * plane + (wa ? r0 + (unsigned)col[1] : row + (unsigned)col[1 - ex(i)])];
+                lb[i] = F[(wb ? i : opp(i)) * plane + (wb ? r0 + (unsigned)col[2] : row + (unsigned)col[2 - ex(i)])];
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const S* q = F + opp(i) * plane + (ey(i) > 0 ? rm : (ey(i) < 0 ? rp : r0));
+                la[i] = q[col[1 - ex(i)]];
+                lb[i] = q[col[2 - ex(i)]];
+            }
+        }
+        if (GMODE == G_LAGGED) {
+            const bool ro = row_out(r);
+            lpx = phi_row(0, r0, ro);
+            lpy = phi_row(1, rp, row_out(r + 1));
+            if (lane == 0) l0 = ro || out[0] ? 0.f : a.phi_in[r0 + (unsigned)col[0]];
+            if (lane == 31) l3 = ro || out[3] ? 0.f : a.phi_in[r0 + (unsigned)col[3]];
+        }
+        rm = r0;
+        r0 = rp;
+        yp = yp == ny - 1 ? (a.py ? 0 : yp) : yp + 1;
+        rp = (unsigned)(yp * pitch);
+    };
+    load_row(y0 - 1, v);
+    bool above = true;                 // special(vq)
+    for (int r = y0 - 1; r <= y1; ++r) {
+        float d[9], e[9], oa[9], ob[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            d[i] = Fmt<S>::ld(la[i]);
+            e[i] = Fmt<S>::ld(lb[i]);
+        }
+        const float2 px = lpx, own_y = pyc;
+        float2 dpx = z2, dpy = z2;
+        if (GMODE == G_LAGGED) {
+            float l = shfl_up1(px.y), rr = shfl_down1(px.x);
+            if (lane == 0) l = l0;
+            if (lane == 31) rr = l3;
+            dpx.x = 0.5f * ((cls(v.x) == PRESSURE ? px.x : px.y) - l);
+            dpx.y = 0.5f * ((cls(v.y) == PRESSURE ? px.y : rr) - px.x);
+            dpy = make_float2(0.5f * (lpy.x - pym.x), 0.5f * (lpy.y - pym.y));
+            pym = pyc;
+            pyc = lpy;
+        }
+        uint2 v2 = vn;
+        if (r < y1) {
+            v2 = load_info(rp, row_out(r + 2));
+            load_row(r + 1, vn);
+        }
+        float2 hx, hy;
+        collide_node(d, v.x, dpx.x, dpy.x, oa, hx.x, hy.x);
+        collide_node(e, v.y, dpx.y, dpy.y, ob, hx.y, hy.y);
+        P N[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) N[i] = K::make(oa[i], ob[i]);
+        // outlet ghosts emit what their inward neighbour, one column before, does;
+        // Phi of solid and moving-wall nodes does not change
+        auto settle = [&](uint2 w, P (&n)[9], float2& gx, float2& gy, float2 keep_x, float2 keep_y) {
+            const bool ga = cls(w.x) == OUTLET, gb = cls(w.y) == OUTLET;
+            if (__any_sync(0xffffffffu, ga || gb)) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    const P u = K::up(n[i]);
+                    n[i] = K::join(ga ? K::first(u) : K::first(n[i]), gb ? K::second(u) : K::second(n[i]));
+                }
+                const float ux = shfl_up1(gx.y), uy = shfl_up1(gy.y);
+                if (gb) gx.y = gx.x, gy.y = gy.x;
+                if (ga) gx.x = ux, gy.x = uy;
+            }
+            if (!collides(cls(w.x)) && !ga) gx.x = keep_x.x, gy.x = keep_y.x;
+            if (!collides(cls(w.y)) && !gb) gx.y = keep_x.y, gy.y = keep_y.y;
+        };
+        const bool here = special(v);
+        if (here) settle(v, N, hx, hy, px, own_y);
+        if (r > y0) {
+            const P E[9] = {C[0], K::up(C[1]), B2, K::down(C[3]), N[4],
+                            K::up(B5), K::down(B6), K::down(N[7]), K::up(N[8])};
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                d[i] = K::lo(E[i]);
+                e[i] = K::hi(E[i]);
+            }
+            if (above) {
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    if (vq.x >> (i - 1) & 1u) d[i] = K::lo(C[opp(i)]);
+                    if (vq.y >> (i - 1) & 1u) e[i] = K::hi(C[opp(i)]);
+                }
+            }
+            float2 qx = z2, qy = z2, kx, ky;
+            if (GMODE == G_LAGGED) {
+                const float l = shfl_up1(hxc.y), rr = shfl_down1(hxc.x);
+                qx.x = 0.5f * ((cls(vq.x) == PRESSURE ? hxc.x : hxc.y) - l);
+                qx.y = 0.5f * ((cls(vq.y) == PRESSURE ? hxc.y : rr) - hxc.x);
+                qy = make_float2(0.5f * (hy.x - hym.x), 0.5f * (hy.y - hym.y));
+            }
+            collide_node(d, vq.x, qx.x, qy.x, oa, kx.x, ky.x);
+            collide_node(e, vq.y, qx.y, qy.y, ob, kx.y, ky.y);
+            P M[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) M[i] = K::make(oa[i], ob[i]);
+            if (above) settle(vq, M, kx, ky, kx, ky);
+            const unsigned at = (unsigned)((r - 1) * pitch + c);
+            const bool sa = inner && c < nx && (collides(cls(vq.x)) || cls(vq.x) == OUTLET);
+            const bool sb = inner && c + 1 < nx && (collides(cls(vq.y)) || cls(vq.y) == OUTLET);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                S* q = O + opp(i) * plane + at;
+                if (sa && sb) {
+                    *reinterpret_cast<P*>(q) = M[i];
+                } else {
+                    if (sa) q[0] = K::first(M[i]);
+                    if (sb) q[1] = K::second(M[i]);
+                }
+            }
+            if (GMODE == G_LAGGED) {
+                if (sa) a.phi_out[at] = kx.x, a.phi_out[plane + at] = ky.x;
+                if (sb) a.phi_out[at + 1] = kx.y, a.phi_out[plane + at + 1] = ky.y;
+            }
+        }
+        B2 = C[2]; B5 = C[5]; B6 = C[6];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) C[i] = N[i];
+        hxc = hx;
+        hym = hyc;
+        hyc = hy;
+        vq = v;
+        above = here;
+        v = vn;
+        vn = v2;
+    }
+}
+
+template <typename S, bool GENERAL, int GMODE, int MAXL>
+__global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_BLOCKS)
+    k_step_pair(const __grid_constant__ PairParams<MAXL> p) {
+    chain_begin();
+    const int b = (int)blockIdx.x;
+    int lo = 0, hi = p.n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.tile_begin[mid] <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    const Args<float>& a = p.a[lo];
+    const int lane = (int)threadIdx.x & 31;
+    int t = b - p.tile_begin[lo];
+    int part = 0;                 // of a split tile
+    if (GENERAL && p.split > 1) {
+        const int one = (p.tile_begin[lo + 1] - p.tile_begin[lo]) / p.split;
+        part = p.split - 1 - t / one;
+        t -= (p.split - 1 - part) * one;
+    }
+    const int w = t * PAIR_WARPS + ((int)threadIdx.x >> 5);
+    int band, strip;
+    tile_divmod(w, p.strips[lo], p.inv_d[lo], band, strip);
+    int y0 = band * p.band[lo];
+    if (y0 >= a.ny) return;   // the whole warp leaves together
+    int y1 = y0 + p.band[lo] < a.ny ? y0 + p.band[lo] : a.ny;
+    S* O = static_cast<S*>(p.out[lo]);
+    if (GENERAL) {
+        // rows y0 - 1 .. y1, wrapped: row 0's and row ny - 1's walls make a band at
+        // an open edge special, so the rows beyond it need no look
+        bool any = false;
+        const unsigned* sp = p.special[lo] + (long long)strip * ((a.ny + 31) / 32);
+        for (int y = y0 - 1 + lane; y <= y1; y += 32) {
+            const int yw = y < 0 ? a.ny - 1 : (y >= a.ny ? 0 : y);
+            any = any || (sp[yw >> 5] >> (yw & 31) & 1u);
+        }
+        if (__any_sync(0xffffffffu, any)) {
+            const int rows = (y1 - y0 + p.split - 1) / p.split;
+            y0 += part * rows;
+            y1 = y0 + rows < y1 ? y0 + rows : y1;
+            if (y0 < y1) pair_walk_general<S, GMODE>(a, O, p.info[lo], strip, y0, y1, lane);
+            return;
+        }
+        if (part > 0) return;
+    }
+    pair_walk<S, GMODE>(a, O, strip, y0, y1, lane);
 }
 
 }  // namespace trt

@@ -148,6 +148,7 @@ void release(trtrlb_lattice* h) {
     if (h->mask) cudaFree(h->mask);
     if (h->ghosts) cudaFree(h->ghosts);
     if (h->seg) cudaFree(h->seg);
+    if (h->pair_map) cudaFree(h->pair_map);
     if (h->stage) cudaFree(h->stage);
     if (h->part) cudaFree(h->part);
     if (h->dout) cudaFree(h->dout);
@@ -183,9 +184,36 @@ bool auto_vector(const trtrlb_lattice* h) {
     return vector_applies(h) && st != TRTRLB_F64 && st != TRTRLB_F64_DW;
 }
 
-// Lattices the two-step kernel advances (lb_pair.cuh).
-bool pair_applies(const trtrlb_params& p) {
-    return p.g_mode != TRTRLB_G_CURRENT && elem_size(p.storage) <= 4 && p.nx >= 32;
+bool collides(uint8_t c) { return c == TRTRLB_FLUID || c == TRTRLB_PRESSURE; }
+
+// Lattices the two-step kernel advances (lb_pair.cuh): not those with the halo
+// classes, whose owner writes them between steps, nor with an outlet ghost that
+// emits into a node on its far side (x + 1), which would take the two steps one
+// column further than a strip reaches.
+bool pair_applies(const trtrlb_params& p, const uint8_t* mask) {
+    if (p.g_mode == TRTRLB_G_CURRENT || elem_size(p.storage) > 4 || p.nx < 32) return false;
+    if (!mask) return true;
+    const size_t n = (size_t)p.nx * p.ny;
+    if (std::memchr(mask, TRTRLB_HALO, n) || std::memchr(mask, TRTRLB_HALO_PRESSURE, n)) return false;
+    const uint8_t* g = mask;
+    while ((g = static_cast<const uint8_t*>(std::memchr(g, TRTRLB_OUTLET, n - (size_t)(g - mask))))) {
+        const int x = (int)((size_t)(g - mask) % p.nx), y = (int)((size_t)(g - mask) / p.nx);
+        const int xr = x + 1 < p.nx ? x + 1 : (p.periodic_x ? 0 : -1);
+        for (int dy = -1; dy <= 1 && xr >= 0; ++dy) {
+            int yr = y + dy;
+            if (yr < 0 || yr >= p.ny) {
+                if (!p.periodic_y) continue;
+                yr = (yr + p.ny) % p.ny;
+            }
+            if (collides(mask[(size_t)yr * p.nx + xr])) return false;
+        }
+        if ((size_t)(++g - mask) == n) break;
+    }
+    return true;
+}
+
+bool two_step_on(const trtrlb_lattice* h) {
+    return h->variant == TRTRLB_KERNEL_AUTO && h->p.g_mode != TRTRLB_G_CURRENT && h->f2;
 }
 
 // Default two-buffer kernel of a G_CURRENT lattice that is periodic without a
@@ -397,7 +425,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     bool ok = alloc(&h->f, es * 9 * plane) && alloc(&h->phi, ps * 4 * plane) &&
               alloc((void**)&h->dout, sizeof(double) * kResultDoubles);
     if (ok && p.g_mode == TRTRLB_G_CURRENT) ok = alloc(&h->f2, es * 9 * plane);
-    if (ok && !mask && p.periodic_x && p.periodic_y && pair_applies(p)) {
+    if (ok && pair_applies(p, mask)) {
         // the two-step kernel's second buffer, never a reason to fail
         if (spare_fits(es * 9 * plane) && cudaMalloc(&h->f2, es * 9 * plane) == cudaSuccess)
             h->bytes += (int64_t)(es * 9 * plane);
@@ -463,7 +491,24 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
         s.seg = h->seg;
         s.segs = (p.nx + 31) / 32;
     }
-    e = cudaMemsetAsync(h->f, 0, es * 9 * plane, h->stream);
+    if (s.general && h->f2 && p.g_mode != TRTRLB_G_CURRENT) {
+        // the two-step kernel's maps; without them the lattice steps singly
+        const size_t words = (size_t)plane + (size_t)trt::pair_strips(p.nx) * ((p.ny + 31) / 32);
+        if (cudaMalloc((void**)&h->pair_map, sizeof(unsigned) * words) == cudaSuccess) {
+            h->bytes += (int64_t)(sizeof(unsigned) * words);
+            s.pinfo = h->pair_map;
+            s.pspecial = h->pair_map + plane;
+            e = TRT_DISPATCH(p.storage, pair_maps(s, h->pair_map, h->pair_map + plane, h->stream));
+        } else {
+            cudaGetLastError();
+            h->pair_map = nullptr;
+            cudaFree(h->f2);
+            h->f2 = nullptr;
+            s.f2 = nullptr;
+            h->bytes -= (int64_t)(es * 9 * plane);
+        }
+    }
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->f, 0, es * 9 * plane, h->stream);
     if (e == cudaSuccess && h->f2 && p.g_mode == TRTRLB_G_CURRENT)   // the two-step kernel writes before it reads
         e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
     if (e == cudaSuccess) e = TRT_DISPATCH(p.storage, phi_static(h->s, h->stream));
@@ -479,7 +524,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     h->variant = TRTRLB_KERNEL_AUTO;
     s.vec = auto_vector(h);
     s.sms = h->sms;
-    s.pair = p.g_mode != TRTRLB_G_CURRENT && h->f2;
+    s.pair = two_step_on(h);
     s.col_h = auto_column(h);
     if (p.g_mode == TRTRLB_G_CURRENT && p.storage == TRTRLB_F32 && !s.general) {
         // the TMA-fed two-buffer kernel; without a descriptor the plain one runs
@@ -691,6 +736,9 @@ int trtrlb_set_f(trtrlb_t h, const double* f, const double* phi) {
     }
     if (e == cudaSuccess) e = TRT_DISPATCH(h->p.storage, set_f(h->s, df, dp, h->stream));
     if (e != cudaSuccess) return cuda_fail(h->err, e, "set_f");
+    // a Phi given for solid and moving-wall nodes sits in one of the two buffers,
+    // which single steps read in turn and the two-step kernel does not
+    h->s.pair = two_step_on(h) && !(phi && h->mask);
     h->t = 0;
     return TRTRLB_OK;
 }
@@ -820,7 +868,7 @@ int trtrlb_set_kernel(trtrlb_t h, int32_t variant, int32_t tile_w) {
     }
     h->variant = variant;
     h->s.vec = vec;
-    h->s.pair = variant == TRTRLB_KERNEL_AUTO && h->p.g_mode != TRTRLB_G_CURRENT && h->f2;
+    h->s.pair = two_step_on(h);
     if (variant == TRTRLB_KERNEL_COLUMN) {
         // the tallest band that still fills the device, else the shortest
         const int es = (int)elem_size(h->p.storage);

@@ -6,10 +6,9 @@ batched, graph-replayed path that the benchmark and the server use, and keeps
 the fastest.  With Phi lagged (the fused AA step) the candidates are the
 scalar kernel with 256-thread tiles of width 32, 64, 128 or 256 nodes, the
 vector kernel (V nodes per thread) where it applies and, for FP32 and 16-bit
-storage on a periodic lattice, the two-step kernel (variant 'auto'); with Phi at
-the current
-level (the two-buffer step) on a periodic lattice without a mask they are the
-plain kernel, the column-walking kernel and, for FP32, the TMA-fed one.
+storage, the two-step kernel (variant 'auto'); with Phi at the current level (the
+two-buffer step) on a periodic lattice without a mask they are the plain kernel,
+the column-walking kernel and, for FP32, the TMA-fed one.
 Results are cached in a JSON file keyed by the bucket, so a shape is measured
 once.  The kernel never changes results beyond rounding (FP64/FP32 are
 bit-identical across kernels).
@@ -81,7 +80,7 @@ class Tuner:
         out = [("scalar", tw) for tw in TILE_WIDTHS if tw <= max(32, 2 * nx)]
         if flavour(periodic, has_mask) == "periodic" and nx % VEC_WIDTH[storage] == 0:
             out.append(("vector", 0))
-        if flavour(periodic, has_mask) == "periodic" and storage in ("f32", "f16", "bf16"):
+        if storage in ("f32", "f16", "bf16"):
             out.append(("auto", 0))            # two steps per launch
         return out
 

@@ -40,20 +40,76 @@ def test_two_steps_equal_single_steps(gpu_lib, storage, g_mode):
             assert a.t == b.t and _same(a, b), (nx, ny, n)
 
 
+def _masks(nx, ny, seed):
+    """(mask or None, periodic, wall_u): walls, obstacles, inlet and both outlets,
+    and an outlet ghost column inside, in the first column a strip stores."""
+    out = [(None, (True, False), (0.0, 0.0)), (None, (False, True), (0.0, 0.0)), (None, (False, False), (0.0, 0.0)),
+           (W.random_mask(nx, ny, seed=seed, solid_frac=0.1), (True, True), (0.0, 0.0))]
+    for outlet in (W.OUTLET, W.PRESSURE):
+        m = W.random_mask(nx, ny, seed=seed + 1, solid_frac=0.05, inlet_outlet=True, outlet=outlet)
+        out.append((m, (False, seed % 2 == 0), (0.03, 0.004)))
+    if ny > 10 and nx > 62:
+        m = np.zeros((ny, nx), np.uint8)
+        m[4:10, 60:62] = W.SOLID
+        m[5:9, 60] = W.OUTLET
+        out.append((m, (True, True), (0.0, 0.0)))
+    return out
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("g_mode", ["lagged", "off"])
+def test_two_steps_equal_single_steps_with_walls_and_masks(gpu_lib, storage, g_mode):
+    """Bands of one part and of several (1500 rows), plain and special tiles, rows and
+    columns past open edges."""
+    for k, (nx, ny) in enumerate([(32, 1), (33, 5), (64, 33), (130, 70), (301, 66), (1300, 1500)]):
+        for mask, periodic, wall_u in _masks(nx, ny, k)[:3 if ny > 1000 else None]:
+            a, b = _lattices(nx, ny, storage, g_mode, k, mask=mask, periodic=periodic, wall_u=wall_u)
+            a.set_kernel("scalar")
+            assert b.two_step() and not a.two_step()
+            for n in (1, 2, 3, 6):
+                a.step(n)
+                b.step(n)
+                assert _same(a, b), (nx, ny, periodic, mask is not None, n)
+
+
+def test_lattices_the_two_step_kernel_leaves_to_single_steps(gpu_lib):
+    """Halo classes, an outlet ghost that emits to its far side, a Phi given for
+    solid nodes; and the same states all the same."""
+    nx, ny = 70, 12
+    halo = np.zeros((ny, nx), np.uint8)
+    halo[0] = 5
+    ghost = np.zeros((ny, nx), np.uint8)
+    ghost[3, 40] = W.OUTLET
+    for m in (halo, ghost):
+        a, b = _lattices(nx, ny, "f32", "lagged", 1, mask=m)
+        a.set_kernel("scalar")
+        assert not b.two_step()
+        assert _same(a.step(5), b.step(5))
+    solid = np.zeros((ny, nx), np.uint8)
+    solid[4:6, 10:12] = W.SOLID
+    a, b = _lattices(nx, ny, "f32", "lagged", 2, mask=solid)
+    a.set_kernel("scalar")
+    phi = np.full((2, ny, nx), 1e-4)
+    f = a.get_f()
+    for lat in (a, b):
+        lat.set_f(f, phi)
+    assert not b.two_step() and _same(a.step(6), b.step(6))
+
+
 def test_two_steps_in_batches(gpu_lib):
     import torch
     from paper_2312_10318_gb300.lattice import Batch
     stream = torch.cuda.Stream()
     alone, members = [], []
     for q, (st, nx, ny) in enumerate([("f32", 130, 70), ("f32", 64, 33), ("f16", 61, 40), ("f64", 40, 20),
-                                      ("bf16", 300, 9), ("f32", 200, 65)]):
-        a, b = _lattices(nx, ny, st, "lagged", q, stream=stream)
+                                      ("bf16", 300, 9), ("f32", 200, 65), ("f32", 130, 40)]):
+        a, b = _lattices(nx, ny, st, "lagged", q, stream=stream, periodic=(True, q != 6))
         a.set_kernel("scalar")
         for lat in (a, b):
             lat.step(q % 2)                    # members at both parities
         alone.append(a)
         members.append(b)
-    for group in ([0, 2, 4], [0, 1, 2, 3, 4, 5]):      # all even, then mixed
+    for group in ([0, 2, 4], [0, 1, 2, 3, 4, 5, 6]):   # all even, then mixed
         batch = Batch(stream).set([members[k] for k in group])
         for n in (3, 32, 33, 70, 64, 1, 65):
             batch.step(n)
