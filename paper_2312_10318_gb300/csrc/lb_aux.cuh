@@ -24,11 +24,6 @@ __device__ __forceinline__ A aux_sel(int c, const A& x) {
     return c > 0 ? x : (c < 0 ? -x : A(0));
 }
 
-// A double-word constant, split at compile time (no FP64 instruction runs).
-__host__ __device__ constexpr df64 dw_const(double x) {
-    return df64((float)x, (float)(x - (double)(float)x));
-}
-
 // Direction I of the initial state in double-word arithmetic (k_init), its
 // lattice constants fixed at compile time.
 template <int I, typename S>

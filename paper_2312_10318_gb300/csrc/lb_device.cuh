@@ -110,9 +110,31 @@ __device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a,
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
+__device__ __forceinline__ float rneg(float a) { return -a; }
+__device__ __forceinline__ double rneg(double a) { return -a; }
 __device__ __forceinline__ df64 radd(const df64& a, const df64& b) { return a + b; }
 __device__ __forceinline__ df64 rsub(const df64& a, const df64& b) { return a - b; }
 __device__ __forceinline__ df64 rmul(const df64& a, const df64& b) { return a * b; }
+
+// FP32 values of two nodes, in sm_103's packed instructions (lb_dw.cuh): the
+// same operations and bits as float's, in half the issue slots.
+struct f2 {
+    f32x2 v;
+    f2() = default;
+    __device__ __forceinline__ explicit f2(f32x2 x) : v(x) {}
+    __device__ __forceinline__ f2(float a, float b) : v(pk(a, b)) {}
+    __device__ __forceinline__ explicit f2(double c) : v(pk((float)c, (float)c)) {}
+};
+__device__ __forceinline__ f2 radd(f2 a, f2 b) { return f2(add2(a.v, b.v)); }
+__device__ __forceinline__ f2 rsub(f2 a, f2 b) { return f2(sub2(a.v, b.v)); }
+__device__ __forceinline__ f2 rmul(f2 a, f2 b) { return f2(mul2(a.v, b.v)); }
+__device__ __forceinline__ f2 rfma(f2 a, f2 b, f2 c) { return f2(fma2(a.v, b.v, c.v)); }
+__device__ __forceinline__ f2 rneg(f2 a) { return f2(neg2(a.v)); }
+__device__ __forceinline__ f2 rrcp(f2 a) {
+    float x, y;
+    unpk(a.v, x, y);
+    return f2(__frcp_rn(x), __frcp_rn(y));
+}
 
 // Zou-He constant-pressure outlet (Sec. III D) on the shifted populations
 // d_i = f_i - w_i rho0 of a node on the last column of a lattice open in x:
@@ -233,70 +255,67 @@ __device__ __forceinline__ long long pop_loc(long long plane, const int (&nb)[9]
 // constants instead of 16), the reciprocal is taken directly, and without a
 // body force (a uniform branch) the forcing terms are skipped -- they would
 // add exact zeros.
-__device__ __forceinline__ df64 scale2(const df64& x, float p) {   // p a power of two
-    return df64(__fmul_rn(x.hi, p), __fmul_rn(x.lo, p));
-}
-
-__device__ __forceinline__ void collide_dw(const df64 (&d)[9], df64 dpx, df64 dpy, const df64 k1,
-                                           const df64 k2, const df64 kf, const df64 gx,
-                                           const df64 gy, const df64 rho0, df64 (&o)[9], df64& phx,
-                                           df64& phy) {
-    const df64 third = df64(1.0 / 3.0);
-    const df64 s13 = d[1] + d[3], m13 = d[1] - d[3];
-    const df64 s24 = d[2] + d[4], m24 = d[2] - d[4];
-    const df64 a57 = d[5] + d[7], m57 = d[5] - d[7];
-    const df64 a68 = d[6] + d[8], m68 = d[6] - d[8];
-    const df64 sd = a57 + a68, pxy = a57 - a68;
-    const df64 qxxy = m57 + m68, qxyy = m57 - m68;
-    const df64 jx = m13 + qxyy, jy = m24 + qxxy;
-    const df64 drho = (d[0] + sd) + (s13 + s24);
-    const df64 rho = rho0 + drho;
-    const df64 inv = recip(rho);
+template <typename D>
+__device__ __forceinline__ void collide_dw(const D (&d)[9], D dpx, D dpy, const df64 k1_, const df64 k2_,
+                                           const df64 kf_, const df64 gx, const df64 gy, const df64 rho0_,
+                                           D (&o)[9], D& phx, D& phy) {
+    const D k1 = D(k1_), k2 = D(k2_), kf = D(kf_), rho0 = D(rho0_);
+    const D third = D(dw_const(1.0 / 3.0));
+    const D s13 = d[1] + d[3], m13 = d[1] - d[3];
+    const D s24 = d[2] + d[4], m24 = d[2] - d[4];
+    const D a57 = d[5] + d[7], m57 = d[5] - d[7];
+    const D a68 = d[6] + d[8], m68 = d[6] - d[8];
+    const D sd = a57 + a68, pxy = a57 - a68;
+    const D qxxy = m57 + m68, qxyy = m57 - m68;
+    const D jx = m13 + qxyy, jy = m24 + qxxy;
+    const D drho = (d[0] + sd) + (s13 + s24);
+    const D rho = rho0 + drho;
+    const D inv = recip(rho);
     const bool forced = gx.hi != 0.f || gx.lo != 0.f || gy.hi != 0.f || gy.lo != 0.f;
-    df64 ux = jx * inv, uy = jy * inv;
+    D ux = jx * inv, uy = jy * inv;
     if (forced) {
-        ux = ux + scale2(gx, 0.5f);
-        uy = uy + scale2(gy, 0.5f);
+        ux = ux + scale2(D(gx), 0.5f);
+        uy = uy + scale2(D(gy), 0.5f);
     }
-    const df64 rux = rho * ux, ruy = rho * uy;
-    const df64 ruxx = rux * ux, ruyy = ruy * uy, ruxy = rux * uy;
-    const df64 rxxy = ruxx * uy, rxyy = ruyy * ux;
-    const df64 drho3 = third * drho;
-    const df64 Axx = ((s13 + sd) - drho3) - ruxx, Ayy = ((s24 + sd) - drho3) - ruyy;
-    const df64 Axy = pxy - ruxy;
-    const df64 Axxy = (qxxy - third * jy) - rxxy, Axyy = (qxyy - third * jx) - rxyy;
-    df64 a1x = jx, a1y = jy;
-    df64 a2xx = (ruxx + k1 * Axx) - kf * dpx;
-    df64 a2yy = (ruyy + k1 * Ayy) - kf * dpy;
-    df64 a2xy = ruxy + k1 * Axy;
+    const D rux = rho * ux, ruy = rho * uy;
+    const D ruxx = rux * ux, ruyy = ruy * uy, ruxy = rux * uy;
+    const D rxxy = ruxx * uy, rxyy = ruyy * ux;
+    const D drho3 = third * drho;
+    const D Axx = ((s13 + sd) - drho3) - ruxx, Ayy = ((s24 + sd) - drho3) - ruyy;
+    const D Axy = pxy - ruxy;
+    const D Axxy = (qxxy - third * jy) - rxxy, Axyy = (qxyy - third * jx) - rxyy;
+    D a1x = jx, a1y = jy;
+    D a2xx = (ruxx + k1 * Axx) - kf * dpx;
+    D a2yy = (ruyy + k1 * Ayy) - kf * dpy;
+    D a2xy = ruxy + k1 * Axy;
     if (forced) {
-        const df64 Fx = rho * gx, Fy = rho * gy;
+        const D Fx = rho * D(gx), Fy = rho * D(gy);
         a1x = a1x + Fx;
         a1y = a1y + Fy;
         a2xx = a2xx + kf * scale2(Fx * ux, 2.f);
         a2yy = a2yy + kf * scale2(Fy * uy, 2.f);
         a2xy = a2xy + kf * (Fx * uy + ux * Fy);
     }
-    const df64 a3xxy = rxxy + k2 * Axxy, a3xyy = rxyy + k2 * Axyy;
+    const D a3xxy = rxxy + k2 * Axxy, a3xyy = rxyy + k2 * Axyy;
     // reconstruction with the weights folded in (see collide)
-    const df64 b9 = third * drho3;                   // drho / 9
-    const df64 hxx = third * a2xx, hyy = third * a2yy;
-    const df64 g1x = third * a1x, g1y = third * a1y;
-    const df64 ht = hxx + hyy;                       // (a2xx + a2yy) / 3
+    const D b9 = third * drho3;                   // drho / 9
+    const D hxx = third * a2xx, hyy = third * a2yy;
+    const D g1x = third * a1x, g1y = third * a1y;
+    const D ht = hxx + hyy;                       // (a2xx + a2yy) / 3
     o[0] = scale2(b9, 4.f) - scale2(ht, 2.f);
-    const df64 c13 = (b9 + hxx) - scale2(hyy, 0.5f);
-    const df64 c24 = (b9 + hyy) - scale2(hxx, 0.5f);
-    const df64 o13 = g1x - scale2(a3xyy, 0.5f);
-    const df64 o24 = g1y - scale2(a3xxy, 0.5f);
+    const D c13 = (b9 + hxx) - scale2(hyy, 0.5f);
+    const D c24 = (b9 + hyy) - scale2(hxx, 0.5f);
+    const D o13 = g1x - scale2(a3xyy, 0.5f);
+    const D o24 = g1y - scale2(a3xxy, 0.5f);
     o[1] = c13 + o13;
     o[3] = c13 - o13;
     o[2] = c24 + o24;
     o[4] = c24 - o24;
-    const df64 cd = scale2(b9 + ht, 0.25f);
-    const df64 q = scale2(a2xy, 0.25f);
-    const df64 c57 = cd + q, c68 = cd - q;
-    const df64 o57 = scale2((g1x + g1y) + (a3xxy + a3xyy), 0.25f);
-    const df64 o68 = scale2((g1y - g1x) + (a3xxy - a3xyy), 0.25f);
+    const D cd = scale2(b9 + ht, 0.25f);
+    const D q = scale2(a2xy, 0.25f);
+    const D c57 = cd + q, c68 = cd - q;
+    const D o57 = scale2((g1x + g1y) + (a3xxy + a3xyy), 0.25f);
+    const D o68 = scale2((g1y - g1x) + (a3xxy - a3xyy), 0.25f);
     o[5] = c57 + o57;
     o[7] = c57 - o57;
     o[6] = c68 + o68;
@@ -342,12 +361,16 @@ __device__ __forceinline__ NodeMom<C> node_moments(const C (&d)[9], const C hgx,
 template <typename C>
 __device__ __forceinline__ C phi_of(const C rho, const C u) { return rmul(rmul(rmul(rho, u), u), u); }
 
+__device__ __forceinline__ bool force_given(double gx, double gy) { return gx != 0.0 || gy != 0.0; }
+template <typename C>
+__device__ __forceinline__ bool force_given(C, C) { return true; }
+
 // The rest of the collision (eq2 with eq9, eq_Gi and eq6) from the moments.
 template <typename C>
 __device__ __forceinline__ void collide_from(const NodeMom<C>& m, C dpx, C dpy, const C k1,
                                              const C k1lo, const C k2, const C k2lo, const C kf,
                                              const C gx, const C gy, C (&o)[9], C& phx, C& phy) {
-    const C third = C(1.0 / 3.0);
+    const C nthird = C(-1.0 / 3.0);
     const C drho = m.drho, rho = m.rho, ux = m.ux, uy = m.uy, jx = m.jx, jy = m.jy;
     const C rux = rmul(rho, ux), ruy = rmul(rho, uy);
     const C ruxx = rmul(rux, ux), ruyy = rmul(ruy, uy), ruxy = rmul(rux, uy);
@@ -356,17 +379,17 @@ __device__ __forceinline__ void collide_from(const NodeMom<C>& m, C dpx, C dpy, 
     // surviving third-order components; minus the equilibrium moments of
     // eq9_2 they are the non-equilibrium projections A of eq9 (A_x = -F_x/2
     // is folded into a1)
-    const C Axx = rsub(rfma(-third, drho, radd(m.s13, m.sd)), ruxx);
-    const C Ayy = rsub(rfma(-third, drho, radd(m.s24, m.sd)), ruyy);
+    const C Axx = rsub(rfma(nthird, drho, radd(m.s13, m.sd)), ruxx);
+    const C Ayy = rsub(rfma(nthird, drho, radd(m.s24, m.sd)), ruyy);
     const C Axy = rsub(m.pxy, ruxy);
-    const C Axxy = rsub(rfma(-third, jy, m.qxxy), rxxy);
-    const C Axyy = rsub(rfma(-third, jx, m.qxyy), rxyy);
+    const C Axxy = rsub(rfma(nthird, jy, m.qxxy), rxxy);
+    const C Axyy = rsub(rfma(nthird, jx, m.qxyy), rxyy);
     // relaxation: (1 - 1/tau) A with 1 - 1/tau carried as hi + lo, so the rate
     // 1/tau stays exact to ~2^-48 even when tau is large (FP32 alone would
     // round 1 - 1/tau to 2^-24 absolute, i.e. 1/tau to 2^-24 tau relative)
     // (FP64 needs no low part: its rounding of 1 - 1/tau is below 1e-11 of the
     // rate for any tau this library accepts in practice)
-    constexpr bool split = sizeof(C) < 8;
+    constexpr bool split = !std::is_same<C, double>::value;
     C r2xx = rfma(k1, Axx, ruxx), r2yy = rfma(k1, Ayy, ruyy), r2xy = rfma(k1, Axy, ruxy);
     C a3xxy = rfma(k2, Axxy, rxxy), a3xyy = rfma(k2, Axyy, rxyy);
     if (split) {
@@ -379,16 +402,16 @@ __device__ __forceinline__ void collide_from(const NodeMom<C>& m, C dpx, C dpy, 
     // body force; FP64, whose pipe bounds the step, skips its terms (exact zeros)
     // without one (a uniform branch)
     C a1x = jx, a1y = jy, a2xx, a2yy, a2xy = r2xy;
-    if (sizeof(C) < 8 || gx != C(0) || gy != C(0)) {
+    if (split || force_given(gx, gy)) {
         const C Fx = rmul(rho, gx), Fy = rmul(rho, gy);
         a1x = radd(jx, Fx);
         a1y = radd(jy, Fy);
-        a2xx = rfma(kf, rfma(radd(Fx, Fx), ux, -dpx), r2xx);
-        a2yy = rfma(kf, rfma(radd(Fy, Fy), uy, -dpy), r2yy);
+        a2xx = rfma(kf, rfma(radd(Fx, Fx), ux, rneg(dpx)), r2xx);
+        a2yy = rfma(kf, rfma(radd(Fy, Fy), uy, rneg(dpy)), r2yy);
         a2xy = rfma(kf, rfma(Fx, uy, rmul(ux, Fy)), r2xy);
     } else {
-        a2xx = rfma(-kf, dpx, r2xx);
-        a2yy = rfma(-kf, dpy, r2yy);
+        a2xx = rfma(rneg(kf), dpx, r2xx);
+        a2yy = rfma(rneg(kf), dpy, r2yy);
     }
     // reconstruction, w_i folded in: w0 = 4/9, w1..4 = 1/9, w5..8 = 1/36
     const C t = radd(a2xx, a2yy);
@@ -420,7 +443,7 @@ __device__ __forceinline__ void collide(const C (&d)[9], C dpx, C dpy, const C k
                                         const C gy, const C hgx, const C hgy, const C rho0, C (&o)[9],
                                         C& phx, C& phy) {
     if constexpr (std::is_same<C, df64>::value) {
-        collide_dw(d, dpx, dpy, k1, k2, kf, gx, gy, rho0, o, phx, phy);
+        collide_dw<df64>(d, dpx, dpy, k1, k2, kf, gx, gy, rho0, o, phx, phy);
     } else {
         collide_from<C>(node_moments<C>(d, hgx, hgy, rho0), dpx, dpy, k1, k1lo, k2, k2lo, kf, gx, gy, o,
                         phx, phy);
@@ -442,24 +465,24 @@ __device__ __forceinline__ void moments_of(const C (&d)[9], C gx, C gy, C rho0, 
 
 // ---- kernels ----------------------------------------------------------------
 
-// Resident 256-thread CTAs per SM the scalar step kernels ask the compiler to
-// allow: the FP32 periodic step with lagged G fits 40 registers without
-// spilling (6 CTAs, 75 % occupancy for the odd step instead of 5), the
-// periodic double-word step 64 (4 CTAs; the odd step took 79 and 3).  The
-// general steps (walls, masks, open edges) run the periodic code on interior
-// row segments, so their own code may spill a little: FP32 and 16-bit 6 CTAs
-// (40 registers; 12-80 bytes of spills in the boundary code), double-word 4
-// (64 registers, no spills with Phi lagged).  Measured on 4096 x 2048 creeping
-// flow and a 4096^2 channel (ms per step, compiler's choice / these): FP32
-// 0.1635 / 0.1442 and 0.2984 / 0.2630, FP16 0.1316 / 0.1138 and 0.2367 /
-// 0.2017, F64_DW 0.3826 / 0.3335 and 0.8070 / 0.7076 (3 CTAs: 0.3587 and
-// 0.7563).  The other variants keep the compiler's choice.
+// Threads per CTA of the scalar step kernels and resident CTAs per SM they ask
+// the compiler to allow: the FP32 periodic step with lagged G fits 40 registers
+// without spilling (6 CTAs, 75 % occupancy for the odd step instead of 5).  The
+// general steps (walls, masks, open edges) run the periodic code on interior row
+// segments, so their own code may spill a little: FP32 and 16-bit 6 CTAs (40
+// registers; 12-80 bytes of spills in the boundary code).  The double-word step
+// collides two nodes per thread (thread_step): 5 CTAs of 128 threads (96 to 102
+// registers).  us per step, one node per thread / two in CTAs of 256 x 2, 256 x 3,
+// 128 x 5, 128 x 6, 128 x 7: 4096^2 periodic 615 / 622, 569, 539, 536, 541; 1024^2
+// 44.0 / 45.0, 39.8, 36.7, 36.9, 37.4.  The other variants keep the compiler's
+// choice.
+template <typename S>
+__host__ __device__ constexpr int step_threads() { return std::is_same<S, f64dw>::value ? 128 : 256; }
 template <typename S, bool GENERAL, int GMODE>
 __host__ __device__ constexpr int step_min_blocks() {
     return (sizeof(S) == 4 && !GENERAL && GMODE == G_LAGGED) ? 6
            : (sizeof(S) <= 4 && GENERAL)                          ? 6
-           : (std::is_same<S, f64dw>::value && !GENERAL)          ? 4
-           : (std::is_same<S, f64dw>::value && GENERAL)           ? 4
+           : std::is_same<S, f64dw>::value                        ? 5
                                                                    : 1;
 }
 
@@ -502,20 +525,17 @@ __device__ __forceinline__ void periodic_load(const Args<typename Fmt<S>::C>& a,
     }
 }
 
-// Its collision and writes, from the values periodic_load read.
+// The writes of its collision.
 template <typename S, bool ODD, int GMODE>
-__device__ __forceinline__ void periodic_finish(const Args<typename Fmt<S>::C>& a, int x, int y,
-                                                const typename Fmt<S>::C (&d)[9], typename Fmt<S>::C dpx,
-                                                typename Fmt<S>::C dpy) {
-    using C = typename Fmt<S>::C;
+__device__ __forceinline__ void periodic_store(const Args<typename Fmt<S>::C>& a, int x, int y,
+                                               const typename Fmt<S>::C (&o)[9], const typename Fmt<S>::C phx,
+                                               const typename Fmt<S>::C phy) {
     const int own = y * a.pitch + x;
     const int pt = a.pitch;
     const int pl = (int)a.plane;
     const int cxp = x == a.nx - 1 ? -a.nx : 0, cxm = x == 0 ? a.nx : 0;
     const int cyp = y == a.ny - 1 ? -pl : 0, cym = y == 0 ? pl : 0;
     S* __restrict__ F = static_cast<S*>(a.f);
-    C o[9], phx, phy;
-    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
     if (GMODE == G_LAGGED) {
         a.phi_out[own] = phx;
         a.phi_out[a.plane + own] = phy;
@@ -531,6 +551,17 @@ __device__ __forceinline__ void periodic_finish(const Args<typename Fmt<S>::C>& 
         }
         F[(long long)k * a.plane + idx] = Fmt<S>::st(o[i]);
     }
+}
+
+// The collision and the writes, from the values periodic_load read.
+template <typename S, bool ODD, int GMODE>
+__device__ __forceinline__ void periodic_finish(const Args<typename Fmt<S>::C>& a, int x, int y,
+                                                const typename Fmt<S>::C (&d)[9], typename Fmt<S>::C dpx,
+                                                typename Fmt<S>::C dpy) {
+    using C = typename Fmt<S>::C;
+    C o[9], phx, phy;
+    collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
+    periodic_store<S, ODD, GMODE>(a, x, y, o, phx, phy);
 }
 
 // The step of a node of a lattice periodic in x and y, without a mask.  The
@@ -667,13 +698,52 @@ __device__ __forceinline__ void node_step(const Args<typename Fmt<S>::C>& a, int
     }
 }
 
+// Most rows a thread of the scalar kernels updates: the double-word step can take
+// the node `dy` rows below with its own, so that both collide in packed operations
+// (df64x2), where neither row segment touches a wall, mask class or open edge.
+template <typename S>
+__host__ __device__ constexpr int rows_per_thread() { return std::is_same<S, f64dw>::value ? 2 : 1; }
+
+// dy: 0 for one row.
 template <typename S, bool ODD, bool GENERAL, int GMODE>
-__global__ void __launch_bounds__(256, step_min_blocks<S, GENERAL, GMODE>()) k_step(Args<typename Fmt<S>::C> a) {
+__device__ __forceinline__ void thread_step(const Args<typename Fmt<S>::C>& a, int x, int y, int dy) {
+    if constexpr (rows_per_thread<S>() == 2) {
+        const int y2 = y + dy;
+        if (dy > 0 && y2 < a.ny) {
+            bool both = true;
+            if (GENERAL) both = a.seg && a.seg[y * a.segs + (x >> 5)] && a.seg[y2 * a.segs + (x >> 5)];
+            // loaded beside the segment map's bytes, not after them
+            df64 d[9], e[9], px, py, qx, qy;
+            periodic_load<S, ODD, GMODE>(a, x, y, d, px, py);
+            periodic_load<S, ODD, GMODE>(a, x, y2, e, qx, qy);
+            if (both) {
+                df64x2 v[9], o[9], hx, hy;
+#pragma unroll
+                for (int i = 0; i < 9; ++i) v[i] = df64x2(d[i], e[i]);
+                collide_dw<df64x2>(v, df64x2(px, qx), df64x2(py, qy), a.k1, a.k2, a.kf, a.gx, a.gy, a.rho0, o, hx, hy);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) o[i].split(d[i], e[i]);
+                hx.split(px, qx);
+                hy.split(py, qy);
+                periodic_store<S, ODD, GMODE>(a, x, y, d, px, py);
+                periodic_store<S, ODD, GMODE>(a, x, y2, e, qx, qy);
+                return;
+            }
+            node_step<S, ODD, GENERAL, GMODE>(a, x, y2);
+        }
+    }
+    node_step<S, ODD, GENERAL, GMODE>(a, x, y);
+}
+
+// rows: nodes per thread, 1 or (rows_per_thread) 2.
+template <typename S, bool ODD, bool GENERAL, int GMODE>
+__global__ void __launch_bounds__(step_threads<S>(), step_min_blocks<S, GENERAL, GMODE>())
+    k_step(Args<typename Fmt<S>::C> a, int rows) {
     chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int y = blockIdx.y * blockDim.y * rows + threadIdx.y;
     if (x >= a.nx || y >= a.ny) return;
-    node_step<S, ODD, GENERAL, GMODE>(a, x, y);
+    thread_step<S, ODD, GENERAL, GMODE>(a, x, y, rows == 2 ? (int)blockDim.y : 0);
 }
 
 // Outlet ghosts, after a step that produced a state of parity ODD_NEW: every

@@ -83,12 +83,12 @@ static inline int scalar_tile(const State& s, int threads) {
     while (tw > threads || (tw > 1 && tw / 2 >= s.nx)) tw /= 2;
     return tw;
 }
-static inline int scalar_threads(const State* const* m, int n) {
-    int t = 256;
+static inline int scalar_threads(const State* const* m, int n, int rows, int most) {
+    int t = most;
     for (; t > 32; t /= 2) {
         long long tiles = 0;
         for (int q = 0; q < n; ++q) {
-            const int tw = scalar_tile(*m[q], t), th = t / tw;
+            const int tw = scalar_tile(*m[q], t), th = t / tw * rows;
             tiles += (long long)((m[q]->nx + tw - 1) / tw) * ((m[q]->ny + th - 1) / th);
         }
         if (tiles >= 2 * m[0]->sms) break;
@@ -96,18 +96,31 @@ static inline int scalar_threads(const State* const* m, int n) {
     return t;
 }
 
+// Nodes per thread of a launch over n lattices (thread_step).  With walls a small
+// lattice's time is that of the threads at them, which step their nodes one after
+// the other: two only where the launch fills the resident warps (64^2 channel
+// 6.2 us per step with one, 9.1 with two; periodic 4.2 and 3.5).
+template <typename S>
+static int scalar_rows(const State* const* m, int n) {
+    if (rows_per_thread<S>() == 1 || !m[0]->general) return rows_per_thread<S>();
+    long long nodes = 0;
+    for (int q = 0; q < n; ++q) nodes += (long long)m[q]->nx * m[q]->ny;
+    return nodes >= 2ll * 5 * step_threads<S>() * m[0]->sms ? 2 : 1;
+}
+
 template <typename S, bool ODD>
 static void launch_step(const State& s, const Args<typename Fmt<S>::C>& a, cudaStream_t st) {
     const State* one = &s;
-    const int t = scalar_threads(&one, 1), tw = scalar_tile(s, t);
+    const int rows = scalar_rows<S>(&one, 1);
+    const int t = scalar_threads(&one, 1, rows, step_threads<S>()), tw = scalar_tile(s, t);
     const dim3 b(tw, t / tw);
-    const dim3 g = grid2d(s, b);
+    const dim3 g = grid2d(s, dim3(tw, t / tw * rows));
     if (s.general) {
-        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, true, G_OFF>, g, b, st, a);
-        else launch_chained(k_step<S, ODD, true, G_LAGGED>, g, b, st, a);
+        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, true, G_OFF>, g, b, st, a, rows);
+        else launch_chained(k_step<S, ODD, true, G_LAGGED>, g, b, st, a, rows);
     } else {
-        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, false, G_OFF>, g, b, st, a);
-        else launch_chained(k_step<S, ODD, false, G_LAGGED>, g, b, st, a);
+        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, false, G_OFF>, g, b, st, a, rows);
+        else launch_chained(k_step<S, ODD, false, G_LAGGED>, g, b, st, a, rows);
     }
 }
 
@@ -354,7 +367,8 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     GroupParams<C, MAXL> p;
     p.n = n;
     int tiles = 0;
-    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n);
+    p.rows = scalar_rows<S>(m, n);
+    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, p.rows, step_threads<S>());
     p.log2_threads = 0;
     while ((1 << p.log2_threads) < threads) ++p.log2_threads;
     for (int q = 0; q < n; ++q) {
@@ -368,7 +382,7 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
             p.log2_tw[q] = 0;
             tiles += (int)(((long long)p.segs[q] * v.ny + 7) / 8);
         } else {
-            const int tw = scalar_tile(v, threads), th = threads / tw;
+            const int tw = scalar_tile(v, threads), th = threads / tw * p.rows;
             p.log2_tw[q] = 0;
             while ((1 << p.log2_tw[q]) < tw) ++p.log2_tw[q];
             p.segs[q] = 0;

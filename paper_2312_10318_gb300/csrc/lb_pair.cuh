@@ -34,7 +34,9 @@
 // the rest is bound by issue (FP16 77 % of the slots, 187 instructions per node
 // and step) and, below 1024^2, by the walk of the band.  4 resident CTAs of 4
 // warps (128 registers, no spills); 5 for the 16-bit formats (102 registers)
-// were slower (4096^2 108.8, 1024^2 11.3).  With walls and masks, whole solves:
+// were slower (4096^2 108.8, 1024^2 11.3).  The collision in packed FP32 (f2)
+// instead of two scalar ones: FP32 1024^2 8.53 to 8.12, 512^2 3.49 to 3.25, FP16
+// 2048^2 28.2 to 27.4, channel 2048 x 1024 FP16 17.4 to 16.1 (chained launches).  With walls and masks, whole solves:
 // creeping flow 4096 x 2048 FP32, 50 steps, 7.3 ms in single steps, 4.4 here;
 // channel 2048 x 1024 FP16, 200 steps, 4.4 and 3.5.
 #pragma once
@@ -128,6 +130,27 @@ template <int MAXL> struct PairParams {
     Args<float> a[MAXL];
 };
 
+// The collision of a pair's two nodes, packed; results rounded to storage.
+template <typename S>
+__device__ __forceinline__ void collide_pair(const Args<float>& a, const typename Pr<S>::P (&D)[9], float2 dpx, float2 dpy,
+                                             typename Pr<S>::P (&N)[9], float2& hx, float2& hy) {
+    using K = Pr<S>;
+    f2 d[9], o[9], px, py;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) d[i] = f2(K::lo(D[i]), K::hi(D[i]));
+    auto both = [](float v) { return f2(v, v); };
+    collide_from<f2>(node_moments<f2>(d, both(a.hgx), both(a.hgy), both(a.rho0)), f2(dpx.x, dpx.y), f2(dpy.x, dpy.y),
+                     both(a.k1), both(a.k1lo), both(a.k2), both(a.k2lo), both(a.kf), both(a.gx), both(a.gy), o, px, py);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        float u, v;
+        unpk(o[i].v, u, v);
+        N[i] = K::make(u, v);
+    }
+    unpk(px.v, hx.x, hx.y);
+    unpk(py.v, hy.x, hy.y);
+}
+
 // The walk of one warp down rows y0 .. y1 - 1 of a strip whose rows y0 - 1 .. y1
 // hold plain fluid nodes only, none of them linked to anything else.
 template <typename S, int GMODE>
@@ -217,51 +240,29 @@ __device__ __forceinline__ void pair_walk(const Args<float>& a, S* __restrict__ 
         if (r < y1) load_row();                    // the next row's, while this one collides
         P N[9];
         float2 hx, hy;
-        {
-            float d[9], e[9], oa[9], ob[9];
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                d[i] = K::lo(D[i]);
-                e[i] = K::hi(D[i]);
-            }
-            collide<float>(d, dpx.x, dpy.x, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, oa,
-                           hx.x, hy.x);
-            collide<float>(e, dpx.y, dpy.y, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, ob,
-                           hx.y, hy.y);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) N[i] = K::make(oa[i], ob[i]);
-        }
+        collide_pair<S>(a, D, dpx, dpy, N, hx, hy);
         // second step at row q = r - 1, from rows q - 1, q and r
         if (r > y0) {
-            float d[9], e[9], oa[9], ob[9];
             const P E[9] = {C0, K::up(C1), B2, K::down(C3), N[4], K::up(B5), K::down(B6), K::down(N[7]), K::up(N[8])};
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                d[i] = K::lo(E[i]);
-                e[i] = K::hi(E[i]);
-            }
+            P M[9];
             float2 qx = make_float2(0.f, 0.f), qy = make_float2(0.f, 0.f), kx, ky;
             if (GMODE == G_LAGGED) {
                 const float l = shfl_up1(hxc.y), rr = shfl_down1(hxc.x);
                 qx = make_float2(0.5f * (hxc.y - l), 0.5f * (rr - hxc.x));
                 qy = make_float2(0.5f * (hy.x - hym.x), 0.5f * (hy.y - hym.y));
             }
-            collide<float>(d, qx.x, qy.x, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, oa,
-                           kx.x, ky.x);
-            collide<float>(e, qx.y, qy.y, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, ob,
-                           kx.y, ky.y);
+            collide_pair<S>(a, E, qx, qy, M, kx, ky);
             const unsigned at = oq + (unsigned)c;
             if (st_b) {
 #pragma unroll
-                for (int i = 0; i < 9; ++i)
-                    *reinterpret_cast<P*>(O + opp(i) * plane + at) = K::make(oa[i], ob[i]);
+                for (int i = 0; i < 9; ++i) *reinterpret_cast<P*>(O + opp(i) * plane + at) = M[i];
                 if (GMODE == G_LAGGED) {
                     *reinterpret_cast<float2*>(a.phi_out + at) = kx;
                     *reinterpret_cast<float2*>(a.phi_out + plane + at) = ky;
                 }
             } else if (st_a) {
 #pragma unroll
-                for (int i = 0; i < 9; ++i) O[opp(i) * plane + at] = Fmt<S>::st(oa[i]);
+                for (int i = 0; i < 9; ++i) O[opp(i) * plane + at] = K::first(M[i]);
                 if (GMODE == G_LAGGED) {
                     a.phi_out[at] = kx.x;
                     a.phi_out[plane + at] = ky.x;
