@@ -322,15 +322,19 @@ int trtrlb_get_kernel(trtrlb_t h, int32_t* vector, int32_t* tile_w);
 #define TRTRLB_STEP_AB_COLUMN 5
 int trtrlb_step_kernel(trtrlb_t h, int32_t* kind);
 
-/* Whether runs of steps advance this lattice two steps per launch (*on = 1): G
- * lagged or off, FP32, FP16 or BF16 storage, nx >= 32, no node of the halo classes
- * and no outlet ghost with a colliding node at x + 1 (any row of the three),
- * TRTRLB_KERNEL_AUTO, and a second population buffer, which
- * trtrlb_create allocates while such buffers take no more than 4 GiB or leave
- * half of the device's memory free, and which goes back when a later allocation of the library would fail.  The
- * two steps start at an odd level: a run from an even one begins with a single
- * step, and an odd rest ends it with one (trtrlb_step_kernel names that
- * kernel).  The bits are those of single steps.  Host only. */
+/* Whether runs of steps advance this lattice two steps per launch (*on = 1):
+ * FP32, FP16 or BF16 storage, nx >= 32, TRTRLB_KERNEL_AUTO and
+ *   - G lagged or off: no node of the halo classes, no outlet ghost with a
+ *     colliding node at x + 1 (any row of the three), and a second population
+ *     buffer, which trtrlb_create allocates while such buffers take no more than
+ *     4 GiB or leave half of the device's memory free, and which goes back when a
+ *     later allocation of the library would fail.  The two steps start at an odd
+ *     level: a run from an even one begins with a single step, and an odd rest
+ *     ends it with one (trtrlb_step_kernel names that kernel).  A Phi given to
+ *     trtrlb_set_f for a lattice with a mask leaves it to single steps;
+ *   - G_CURRENT: periodic in both directions without a mask; an odd rest of a run
+ *     is a single step.
+ * The bits are those of single steps.  Host only. */
 int trtrlb_two_step(trtrlb_t h, int32_t* on);
 
 /* ---- slab decomposition -----------------------------------------------------

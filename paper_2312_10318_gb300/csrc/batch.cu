@@ -83,7 +83,8 @@ std::vector<int> signature(const trtrlb_batch* b, const std::vector<trt::State>&
 
 // Members that take the same launches: of one format, kernel, G mode and parity
 // of the current level.  tma: the small TMA-fed two-buffer members, which share
-// launches; other two-buffer members are classes of their own.
+// launches of single steps; the other two-buffer members take their own, and
+// without launches of two steps are classes of their own.
 struct Class {
     int storage, flavour, g_mode, parity;
     bool pair, tma;
@@ -101,7 +102,7 @@ std::vector<Class> classes_of(const trtrlb_batch* b, const std::vector<trt::Stat
         Class* c = nullptr;
         for (Class& x : out)
             if (x.storage == h->p.storage && x.flavour == flav && x.g_mode == s.g_mode && x.parity == s.parity &&
-                x.pair == s.pair && x.tma == tma && (!ab || tma))
+                x.pair == s.pair && x.tma == tma && (!ab || tma || s.pair))
                 c = &x;
         if (!c) {
             out.push_back(Class{h->p.storage, flav, s.g_mode, s.parity, s.pair, tma, {}, 0});
@@ -129,9 +130,15 @@ cudaError_t launch_class(trtrlb_batch* b, const Class& c, std::vector<trt::State
     int parity = c.parity;
     for (int64_t q = 0; q < n;) {
         cudaError_t e;
-        if (c.g_mode == TRTRLB_G_CURRENT) {
+        if (c.g_mode == TRTRLB_G_CURRENT && c.pair && q + 2 <= n) {
+            e = TRT_DISPATCH_S(c.storage, step_pair(m.data(), k, st));
+            for (int i : c.members) trt::after_pair(sim[i]);
+            q += 2;
+        } else if (c.g_mode == TRTRLB_G_CURRENT) {
             e = c.tma ? trt::Ops<float>::step_ab_group(m.data(), k, st)
-                      : TRT_DISPATCH_S(c.storage, step_ab(*m[0], st));
+                      : cudaSuccess;
+            for (int i = 0; !c.tma && i < k && e == cudaSuccess; ++i)
+                e = TRT_DISPATCH_S(c.storage, step_ab(*m[i], st));
             for (int i : c.members) std::swap(sim[i].f, sim[i].f2);
             q += 1;
         } else if (c.pair && parity == 1 && q + 2 <= last) {
@@ -306,7 +313,8 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
     if (b->stream != nullptr && nsteps >= kGraphSteps) {
         // to odd levels, where the runs of two start, if that is a step for all
         bool odd_pair = false, even_pair = false;
-        for (const trt::State& x : sim) (x.parity ? odd_pair : even_pair) |= x.pair;
+        for (const trt::State& x : sim)
+            if (x.g_mode != TRTRLB_G_CURRENT) (x.parity ? odd_pair : even_pair) |= x.pair;
         if (even_pair && !odd_pair && nsteps > kGraphSteps) {
             e = launch_steps(b, sim, 1);
             done = 1;

@@ -65,10 +65,7 @@ __device__ __forceinline__ void ab_phi(const Args<typename Fmt<S>::C>& a, const 
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = Fmt<S>::ld(F[(long long)i * a.plane + k]);
     if (c == PRESSURE || c == HALO_PRESSURE) zh_fill<C>(d, a.zh_dr);
-    C rho, ux, uy;
-    moments_of<C>(d, a.gx, a.gy, a.rho0, rho, ux, uy);
-    px = rho * ux * ux * ux;
-    py = rho * uy * uy * uy;
+    node_phi<C>(a, d, px, py);
 }
 
 __device__ __forceinline__ int ab_wrap(int v, int n) { return v < 0 ? v + n : (v >= n ? v - n : v); }
@@ -137,20 +134,14 @@ __global__ void __launch_bounds__(AB_TX * AB_TY, 4) k_step_ab(Args<typename Fmt<
         }
         C px = C(0), py = C(0);
         if (inside || past) {
-            C rho, ux, uy;
-            moments_of<C>(d, a.gx, a.gy, a.rho0, rho, ux, uy);
-            px = rho * ux * ux * ux;
-            py = rho * uy * uy * uy;
+            node_phi<C>(a, d, px, py);
         }
         sx[ty][tx + 1] = px;
         sy[ty + 1][tx] = py;
         if (h < 2 * AB_TY + 2 * AB_TX) {
             C qx = C(0), qy = C(0);
             if (hx >= 0) {
-                C rho, ux, uy;
-                moments_of<C>(e, a.gx, a.gy, a.rho0, rho, ux, uy);
-                qx = rho * ux * ux * ux;
-                qy = rho * uy * uy * uy;
+                node_phi<C>(a, e, qx, qy);
             }
             if (h < 2 * AB_TY) sx[h % AB_TY][h / AB_TY ? AB_TX + 1 : 0] = qx;
             else sy[(h - 2 * AB_TY) / AB_TX ? AB_TY + 1 : 0][(h - 2 * AB_TY) % AB_TX] = qy;
@@ -159,10 +150,7 @@ __global__ void __launch_bounds__(AB_TX * AB_TY, 4) k_step_ab(Args<typename Fmt<
     } else if (!g_off) {
         C px = C(0), py = C(0);
         if (fluid) {
-            C rho, ux, uy;
-            moments_of<C>(d, a.gx, a.gy, a.rho0, rho, ux, uy);
-            px = rho * ux * ux * ux;
-            py = rho * uy * uy * uy;
+            node_phi<C>(a, d, px, py);
         } else if (inside || (x == a.nx && y < a.ny) || (y == a.ny && x < a.nx)) {
             ab_phi<S>(a, F, x, y, px, py);
         }

@@ -87,10 +87,7 @@ __device__ __forceinline__ void tma_phi_global(const Args<float>& a, const float
     float d[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = F[(long long)i * a.plane + k];
-    float rho, ux, uy;
-    moments_of<float>(d, a.gx, a.gy, a.rho0, rho, ux, uy);
-    px = rho * ux * ux * ux;
-    py = rho * uy * uy * uy;
+    node_phi<float>(a, d, px, py);
 }
 
 // Phi of box cell (column c, row r) of a stage.
@@ -99,10 +96,7 @@ __device__ __forceinline__ void tma_phi_smem(const Args<float>& a, const TmaStag
     float d[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) d[i] = st.v[i][r][c];
-    float rho, ux, uy;
-    moments_of<float>(d, a.gx, a.gy, a.rho0, rho, ux, uy);
-    px = rho * ux * ux * ux;
-    py = rho * uy * uy * uy;
+    node_phi<float>(a, d, px, py);
 }
 
 // Shared memory of k_step_ab_tma (dynamic; its start is rounded up to 128 B).

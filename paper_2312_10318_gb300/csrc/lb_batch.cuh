@@ -17,11 +17,10 @@ constexpr int GROUP_MAX = 96;
 template <typename C, int MAXL> struct GroupParams {
     int n;                       // lattices in this launch
     int log2_threads;            // threads per CTA, 2^log2_threads
-    int rows;                    // scalar: nodes per thread (thread_step)
     int tile_begin[MAXL + 1];    // prefix sums of tiles; tile_begin[n] = total
     int tiles_x[MAXL];           // tiles per tile row
     int log2_tw[MAXL];           // scalar: tile width 2^log2_tw nodes, height threads / width
-                                 // times rows
+                                 // times ROWS
     int segs[MAXL];              // vector: warp segments per row
     float inv_d[MAXL];           // 1 / tiles_x (scalar) or 1 / segs (vector), rounded
     Args<C> a[MAXL];
@@ -42,8 +41,8 @@ __device__ __forceinline__ void tile_divmod(int t, int d, float inv, int& q, int
     }
 }
 
-template <typename S, bool ODD, bool GENERAL, int GMODE, int MAXL>
-__global__ void __launch_bounds__(step_threads<S>(), step_min_blocks<S, GENERAL, GMODE>())
+template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS, int MAXL>
+__global__ void __launch_bounds__(step_threads<ROWS>(), step_min_blocks<S, GENERAL, GMODE, ROWS>())
     k_step_group(const __grid_constant__ GroupParams<typename Fmt<S>::C, MAXL> p) {
     chain_begin();
     const int b = (int)blockIdx.x;
@@ -59,9 +58,9 @@ __global__ void __launch_bounds__(step_threads<S>(), step_min_blocks<S, GENERAL,
     tile_divmod(t, p.tiles_x[lo], p.inv_d[lo], ty, tx);
     const int x = (tx << lt) + ((int)threadIdx.x & ((1 << lt) - 1));
     const int th = 1 << (p.log2_threads - lt);
-    const int y = ty * th * p.rows + ((int)threadIdx.x >> lt);
+    const int y = ty * th * ROWS + ((int)threadIdx.x >> lt);
     if (x >= p.a[lo].nx || y >= p.a[lo].ny) return;
-    thread_step<S, ODD, GENERAL, GMODE>(p.a[lo], x, y, p.rows == 2 ? th : 0);
+    thread_step<S, ODD, GENERAL, GMODE, ROWS>(p.a[lo], x, y, th);
 }
 
 // Vectorised flavour: a CTA owns 8 consecutive warp segments of one lattice.

@@ -463,6 +463,22 @@ __device__ __forceinline__ void moments_of(const C (&d)[9], C gx, C gy, C rho0, 
     uy = jy * inv + C(0.5) * gy;
 }
 
+// Phi of one node from its populations, as the two-buffer kernels that keep the
+// node's moments for its collision compute it.
+template <typename C>
+__device__ __forceinline__ void node_phi(const Args<C>& a, const C (&d)[9], C& px, C& py) {
+    if constexpr (std::is_same<C, df64>::value) {
+        C rho, ux, uy;
+        moments_of<C>(d, a.gx, a.gy, a.rho0, rho, ux, uy);
+        px = rho * ux * ux * ux;
+        py = rho * uy * uy * uy;
+    } else {
+        const NodeMom<C> m = node_moments<C>(d, a.hgx, a.hgy, a.rho0);
+        px = phi_of(m.rho, m.ux);
+        py = phi_of(m.rho, m.uy);
+    }
+}
+
 // ---- kernels ----------------------------------------------------------------
 
 // Threads per CTA of the scalar step kernels and resident CTAs per SM they ask
@@ -474,15 +490,16 @@ __device__ __forceinline__ void moments_of(const C (&d)[9], C gx, C gy, C rho0, 
 // collides two nodes per thread (thread_step): 5 CTAs of 128 threads (96 to 102
 // registers).  us per step, one node per thread / two in CTAs of 256 x 2, 256 x 3,
 // 128 x 5, 128 x 6, 128 x 7: 4096^2 periodic 615 / 622, 569, 539, 536, 541; 1024^2
-// 44.0 / 45.0, 39.8, 36.7, 36.9, 37.4.  The other variants keep the compiler's
-// choice.
-template <typename S>
-__host__ __device__ constexpr int step_threads() { return std::is_same<S, f64dw>::value ? 128 : 256; }
-template <typename S, bool GENERAL, int GMODE>
+// 44.0 / 45.0, 39.8, 36.7, 36.9, 37.4.  With one node per thread it asks for 4 of
+// 256 (64 registers, no spills with Phi lagged).  The other variants keep the
+// compiler's choice.
+template <int ROWS>
+__host__ __device__ constexpr int step_threads() { return ROWS == 2 ? 128 : 256; }
+template <typename S, bool GENERAL, int GMODE, int ROWS>
 __host__ __device__ constexpr int step_min_blocks() {
     return (sizeof(S) == 4 && !GENERAL && GMODE == G_LAGGED) ? 6
            : (sizeof(S) <= 4 && GENERAL)                          ? 6
-           : std::is_same<S, f64dw>::value                        ? 5
+           : std::is_same<S, f64dw>::value                        ? (ROWS == 2 ? 5 : 4)
                                                                    : 1;
 }
 
@@ -698,52 +715,42 @@ __device__ __forceinline__ void node_step(const Args<typename Fmt<S>::C>& a, int
     }
 }
 
-// Most rows a thread of the scalar kernels updates: the double-word step can take
-// the node `dy` rows below with its own, so that both collide in packed operations
-// (df64x2), where neither row segment touches a wall, mask class or open edge.
-template <typename S>
-__host__ __device__ constexpr int rows_per_thread() { return std::is_same<S, f64dw>::value ? 2 : 1; }
-
-// dy: 0 for one row.
-template <typename S, bool ODD, bool GENERAL, int GMODE>
+// What one thread of the scalar kernels does.  ROWS = 2 (periodic lattices in
+// double-word storage): the node dy rows below too, both in packed operations
+// (df64x2).
+template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS>
 __device__ __forceinline__ void thread_step(const Args<typename Fmt<S>::C>& a, int x, int y, int dy) {
-    if constexpr (rows_per_thread<S>() == 2) {
-        const int y2 = y + dy;
-        if (dy > 0 && y2 < a.ny) {
-            bool both = true;
-            if (GENERAL) both = a.seg && a.seg[y * a.segs + (x >> 5)] && a.seg[y2 * a.segs + (x >> 5)];
-            // loaded beside the segment map's bytes, not after them
-            df64 d[9], e[9], px, py, qx, qy;
-            periodic_load<S, ODD, GMODE>(a, x, y, d, px, py);
-            periodic_load<S, ODD, GMODE>(a, x, y2, e, qx, qy);
-            if (both) {
-                df64x2 v[9], o[9], hx, hy;
+    if constexpr (ROWS == 2) {
+        static_assert(!GENERAL, "two nodes per thread on periodic lattices only");
+        // a last row without a partner is computed twice, and its first copy not stored
+        const bool pair = y + dy < a.ny;
+        const int y2 = pair ? y + dy : y;
+        df64 d[9], e[9], px, py, qx, qy;
+        periodic_load<S, ODD, GMODE>(a, x, y, d, px, py);
+        periodic_load<S, ODD, GMODE>(a, x, y2, e, qx, qy);
+        df64x2 v[9], o[9], hx, hy;
 #pragma unroll
-                for (int i = 0; i < 9; ++i) v[i] = df64x2(d[i], e[i]);
-                collide_dw<df64x2>(v, df64x2(px, qx), df64x2(py, qy), a.k1, a.k2, a.kf, a.gx, a.gy, a.rho0, o, hx, hy);
+        for (int i = 0; i < 9; ++i) v[i] = df64x2(d[i], e[i]);
+        collide_dw<df64x2>(v, df64x2(px, qx), df64x2(py, qy), a.k1, a.k2, a.kf, a.gx, a.gy, a.rho0, o, hx, hy);
 #pragma unroll
-                for (int i = 0; i < 9; ++i) o[i].split(d[i], e[i]);
-                hx.split(px, qx);
-                hy.split(py, qy);
-                periodic_store<S, ODD, GMODE>(a, x, y, d, px, py);
-                periodic_store<S, ODD, GMODE>(a, x, y2, e, qx, qy);
-                return;
-            }
-            node_step<S, ODD, GENERAL, GMODE>(a, x, y2);
-        }
+        for (int i = 0; i < 9; ++i) o[i].split(d[i], e[i]);
+        hx.split(px, qx);
+        hy.split(py, qy);
+        if (pair) periodic_store<S, ODD, GMODE>(a, x, y, d, px, py);
+        periodic_store<S, ODD, GMODE>(a, x, y2, e, qx, qy);
+    } else {
+        node_step<S, ODD, GENERAL, GMODE>(a, x, y);
     }
-    node_step<S, ODD, GENERAL, GMODE>(a, x, y);
 }
 
-// rows: nodes per thread, 1 or (rows_per_thread) 2.
-template <typename S, bool ODD, bool GENERAL, int GMODE>
-__global__ void __launch_bounds__(step_threads<S>(), step_min_blocks<S, GENERAL, GMODE>())
-    k_step(Args<typename Fmt<S>::C> a, int rows) {
+template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS>
+__global__ void __launch_bounds__(step_threads<ROWS>(), step_min_blocks<S, GENERAL, GMODE, ROWS>())
+    k_step(Args<typename Fmt<S>::C> a) {
     chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y * rows + threadIdx.y;
+    const int y = blockIdx.y * blockDim.y * ROWS + threadIdx.y;
     if (x >= a.nx || y >= a.ny) return;
-    thread_step<S, ODD, GENERAL, GMODE>(a, x, y, rows == 2 ? (int)blockDim.y : 0);
+    thread_step<S, ODD, GENERAL, GMODE, ROWS>(a, x, y, (int)blockDim.y);
 }
 
 // Outlet ghosts, after a step that produced a state of parity ODD_NEW: every

@@ -32,6 +32,7 @@ struct trtrlb_lattice {
     int tma_grid;        // persistent grid of the TMA kernel on this device (0: none)
     int sms;             // multiprocessors of the handle's device
     std::mutex spare_mu; // held while launches that use f2 of a lagged lattice are queued
+    bool phi_given;      // trtrlb_set_f gave a Phi to a lattice with a mask
     bool spare_kept;     // f2 is named by a captured graph: not given back before the handle
     char err[256];
 };

@@ -33,7 +33,8 @@ constexpr long long kDefaultWaitLimit = 1ll << 22;
 
 // Two-step kernel (lb_pair.cuh): nodes of a row a warp updates, warps per CTA.
 constexpr int PAIR_W = 60, PAIR_WARPS = 4;
-inline int pair_strips(int nx) { return (nx + PAIR_W - 1) / PAIR_W; }
+constexpr int PAIR_AB_W = 56;   // with Phi at the current level
+inline int pair_strips(int nx, int width = PAIR_W) { return (nx + width - 1) / width; }
 
 struct State {
     void* f;              // populations, S[9][ny][pitch]

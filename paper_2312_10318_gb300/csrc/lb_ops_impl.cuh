@@ -96,32 +96,29 @@ static inline int scalar_threads(const State* const* m, int n, int rows, int mos
     return t;
 }
 
-// Nodes per thread of a launch over n lattices (thread_step).  With walls a small
-// lattice's time is that of the threads at them, which step their nodes one after
-// the other: two only where the launch fills the resident warps (64^2 channel
-// 6.2 us per step with one, 9.1 with two; periodic 4.2 and 3.5).
-template <typename S>
-static int scalar_rows(const State* const* m, int n) {
-    if (rows_per_thread<S>() == 1 || !m[0]->general) return rows_per_thread<S>();
-    long long nodes = 0;
-    for (int q = 0; q < n; ++q) nodes += (long long)m[q]->nx * m[q]->ny;
-    return nodes >= 2ll * 5 * step_threads<S>() * m[0]->sms ? 2 : 1;
+// Nodes per thread: the periodic double-word step takes two (thread_step).  With
+// walls and masks it takes one: a segment at them steps its nodes one after the
+// other, which all but the largest launches wait for at their end (us per step, one
+// / two: channel 64^2 6.2 / 6.8, 512^2 14.7 / 16.1, 1024^2 49.4 / 54.9, 2048^2 178 /
+// 169; periodic 64^2 4.2 / 3.5, 4096^2 615 / 539), and the kernels that hold both
+// forms took five minutes to compile.
+template <typename S, bool GENERAL>
+constexpr int rows_of_step() { return std::is_same<S, f64dw>::value && !GENERAL ? 2 : 1; }
+
+template <typename S, bool ODD, bool GENERAL>
+static void launch_scalar(const State& s, const Args<typename Fmt<S>::C>& a, cudaStream_t st) {
+    constexpr int ROWS = rows_of_step<S, GENERAL>();
+    const State* one = &s;
+    const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>()), tw = scalar_tile(s, t);
+    const dim3 b(tw, t / tw), g = grid2d(s, dim3(tw, t / tw * ROWS));
+    if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, GENERAL, G_OFF, ROWS>, g, b, st, a);
+    else launch_chained(k_step<S, ODD, GENERAL, G_LAGGED, ROWS>, g, b, st, a);
 }
 
 template <typename S, bool ODD>
 static void launch_step(const State& s, const Args<typename Fmt<S>::C>& a, cudaStream_t st) {
-    const State* one = &s;
-    const int rows = scalar_rows<S>(&one, 1);
-    const int t = scalar_threads(&one, 1, rows, step_threads<S>()), tw = scalar_tile(s, t);
-    const dim3 b(tw, t / tw);
-    const dim3 g = grid2d(s, dim3(tw, t / tw * rows));
-    if (s.general) {
-        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, true, G_OFF>, g, b, st, a, rows);
-        else launch_chained(k_step<S, ODD, true, G_LAGGED>, g, b, st, a, rows);
-    } else {
-        if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, false, G_OFF>, g, b, st, a, rows);
-        else launch_chained(k_step<S, ODD, false, G_LAGGED>, g, b, st, a, rows);
-    }
+    if (s.general) launch_scalar<S, ODD, true>(s, a, st);
+    else launch_scalar<S, ODD, false>(s, a, st);
 }
 
 template <typename S, bool ODD>
@@ -367,8 +364,8 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     GroupParams<C, MAXL> p;
     p.n = n;
     int tiles = 0;
-    p.rows = scalar_rows<S>(m, n);
-    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, p.rows, step_threads<S>());
+    constexpr int ROWS = rows_of_step<S, FLAV == FLAV_GENERAL>();
+    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, ROWS, step_threads<ROWS>());
     p.log2_threads = 0;
     while ((1 << p.log2_threads) < threads) ++p.log2_threads;
     for (int q = 0; q < n; ++q) {
@@ -382,7 +379,7 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
             p.log2_tw[q] = 0;
             tiles += (int)(((long long)p.segs[q] * v.ny + 7) / 8);
         } else {
-            const int tw = scalar_tile(v, threads), th = threads / tw * p.rows;
+            const int tw = scalar_tile(v, threads), th = threads / tw * ROWS;
             p.log2_tw[q] = 0;
             while ((1 << p.log2_tw[q]) < tw) ++p.log2_tw[q];
             p.segs[q] = 0;
@@ -395,15 +392,20 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     if (FLAV == FLAV_VECTOR)
         return launch_chained(k_step_group_vec<S, ODD, GMODE, MAXL>, tiles, BATCH_THREADS, st, p);
     else
-        return launch_chained(k_step_group<S, ODD, FLAV == FLAV_GENERAL, GMODE, MAXL>, tiles, threads, st, p);
+        return launch_chained(k_step_group<S, ODD, FLAV == FLAV_GENERAL, GMODE, ROWS, MAXL>, tiles, threads, st, p);
 }
 
 template <typename S, bool ODD, int FLAV, int GMODE>
 static cudaError_t launch_group_sized(const State* const* m, int n, cudaStream_t st) {
     for (int q0 = 0; q0 < n; q0 += GROUP_MAX) {
         const int c = n - q0 < GROUP_MAX ? n - q0 : GROUP_MAX;
-        const cudaError_t e = c <= 4 ? launch_group<S, ODD, FLAV, GMODE, 4>(m + q0, c, st)
-                                     : launch_group<S, ODD, FLAV, GMODE, GROUP_MAX>(m + q0, c, st);
+        cudaError_t e;
+        // the double-word kernels, the longest to compile and to run, have one size
+        if constexpr (std::is_same<S, f64dw>::value)
+            e = launch_group<S, ODD, FLAV, GMODE, GROUP_MAX>(m + q0, c, st);
+        else
+            e = c <= 4 ? launch_group<S, ODD, FLAV, GMODE, 4>(m + q0, c, st)
+                       : launch_group<S, ODD, FLAV, GMODE, GROUP_MAX>(m + q0, c, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -433,8 +435,10 @@ static cudaError_t launch_pair(const State* const* m, int n, cudaStream_t st) {
     PairParams<MAXL> p;
     p.n = n;
     // general lattices leave a sixteenth of the slots to the parts of split tiles
-    const long long slots = (long long)m[0]->sms * PAIR_BLOCKS * PAIR_WARPS;
-    const int band = pair_band_rows(m, n, GENERAL ? slots - slots / 16 : slots);
+    constexpr bool ab = GMODE == G_CURRENT;
+    constexpr int width = ab ? PAIR_AB_W : PAIR_W;
+    const long long slots = (long long)m[0]->sms * (ab ? PAIR_AB_BLOCKS : PAIR_BLOCKS) * PAIR_WARPS;
+    const int band = pair_band_rows(m, n, GENERAL ? slots - slots / 16 : slots, width);
     p.split = GENERAL ? pair_split(band) : 1;
     int tiles = 0;
     for (int q = 0; q < n; ++q) {
@@ -444,18 +448,24 @@ static cudaError_t launch_pair(const State* const* m, int n, cudaStream_t st) {
         p.info[q] = s.pinfo;
         p.special[q] = s.pspecial;
         p.tile_begin[q] = tiles;
-        p.strips[q] = pair_strips(s.nx);
+        p.strips[q] = pair_strips(s.nx, width);
         p.inv_d[q] = 1.0f / (float)p.strips[q];
         p.band[q] = band;
         const long long warps = (long long)p.strips[q] * ((s.ny + band - 1) / band);
         tiles += p.split * (int)((warps + PAIR_WARPS - 1) / PAIR_WARPS);
     }
     p.tile_begin[n] = tiles;
-    return launch_chained(k_step_pair<S, GENERAL, GMODE, MAXL>, tiles, PAIR_WARPS * 32, st, p);
+    if constexpr (ab) return launch_chained(k_step_ab_pair<S, MAXL>, tiles, PAIR_WARPS * 32, st, p);
+    else return launch_chained(k_step_pair<S, GENERAL, GMODE, MAXL>, tiles, PAIR_WARPS * 32, st, p);
 }
 
 template <typename S, bool GENERAL>
 static cudaError_t launch_pair_g(const State* const* m, int n, cudaStream_t st) {
+    if constexpr (!GENERAL) {
+        if (m[0]->g_mode == G_CURRENT)
+            return n <= 4 ? launch_pair<S, false, G_CURRENT, 4>(m, n, st)
+                          : launch_pair<S, false, G_CURRENT, GROUP_MAX>(m, n, st);
+    }
     if (m[0]->g_mode == G_OFF)
         return n <= 4 ? launch_pair<S, GENERAL, G_OFF, 4>(m, n, st) : launch_pair<S, GENERAL, G_OFF, GROUP_MAX>(m, n, st);
     return n <= 4 ? launch_pair<S, GENERAL, G_LAGGED, 4>(m, n, st)

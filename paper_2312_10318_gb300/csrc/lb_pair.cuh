@@ -81,7 +81,7 @@ template <> struct Pr<__half> : Pr16<__half> {};
 template <> struct Pr<__nv_bfloat16> : Pr16<__nv_bfloat16> {};
 
 // Resident CTAs per SM the two-step kernel asks the compiler to allow.
-constexpr int PAIR_BLOCKS = 4;
+constexpr int PAIR_BLOCKS = 4, PAIR_AB_BLOCKS = 3, PAIR_AB_AHEAD = 3;
 
 // Rows per band for n lattices sharing a launch: the smallest number with which
 // every warp is resident at once, or, where that is more than PAIR_ROWS, in the
@@ -89,11 +89,11 @@ constexpr int PAIR_BLOCKS = 4;
 // sequential, so a partial wave costs a whole one: 4096^2 FP32 with 1.25, 1.5
 // and 2 waves of shorter bands 157, 149 and 128 us per step against 126.0 in
 // one; 250 x 246 with bands of 16, 8, 4 and 2 rows 7.15, 5.12, 4.11 and 3.09.
-inline int pair_band_rows(const State* const* m, int n, long long slots) {
+inline int pair_band_rows(const State* const* m, int n, long long slots, int width) {
     auto warps = [&](int h) {
         long long w = 0;
         for (int q = 0; q < n; ++q) {
-            const long long k = (long long)pair_strips(m[q]->nx) * ((m[q]->ny + h - 1) / h);
+            const long long k = (long long)pair_strips(m[q]->nx, width) * ((m[q]->ny + h - 1) / h);
             w += (k + PAIR_WARPS - 1) / PAIR_WARPS * PAIR_WARPS;
         }
         return w;
@@ -574,6 +574,177 @@ __global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_BLOCKS)
         if (part > 0) return;
     }
     pair_walk<S, GMODE>(a, O, strip, y0, y1, lane);
+}
+
+// BYTES (4 or 8) from global to shared memory, asynchronously.
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* to, const void* from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from),
+                 "n"(BYTES)
+                 : "memory");
+}
+
+// ---- Phi at the current level -----------------------------------------------------
+// Two time steps of the two-buffer step (lb_ab.cuh) on a lattice periodic in x and
+// y without a mask, from the canonical f(t) in one buffer to f(t + 2) in the other.
+// The same walk with Phi in it: loading row r gives its moments and Phi(t); row
+// r - 1 collides (d_y Phi from rows r and r - 2, d_x from the lanes beside), which
+// completes f(t + 1) of row r - 2, its moments and Phi(t + 1); row r - 3 collides,
+// which completes f(t + 2) of row r - 4, stored aligned.  Moments are kept for the
+// collision two rows later, the three rows of collided populations per step in
+// registers.  Phi takes two columns more of either side than lagged Phi does: 56
+// of 64 are stored, and a band of h rows loads h + 8.
+//
+// A step of its own moves 72 B per node (FP32) and the TMA-fed kernel issues 378
+// instructions for it; two in one launch move 36 per step.  us per step, the
+// kernels of single steps (TMA-fed, column, plain: the fastest) / this one: FP32
+// 4096^2 229 / 128, 2048^2 61.3 / 34.9, 1024^2 16.0 / 12.7, 512^2 8.2 / 7.0; FP16
+// 4096^2 178 / 120, 2048^2 53.0 / 33.5, 1024^2 16.4 / 12.2.  Bound by latency at 12
+// warps per SM (168 registers; 4 CTAs spill: 2048^2 FP32 144).
+template <typename S, int MAXL>
+__global__ void __launch_bounds__(PAIR_WARPS * 32, PAIR_AB_BLOCKS)
+    k_step_ab_pair(const __grid_constant__ PairParams<MAXL> p) {
+    using K = Pr<S>;
+    using P = typename K::P;
+    chain_begin();
+    const int b = (int)blockIdx.x;
+    int lo = 0, hi = p.n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.tile_begin[mid] <= b) lo = mid;
+        else hi = mid - 1;
+    }
+    const Args<float>& a = p.a[lo];
+    const int lane = (int)threadIdx.x & 31;
+    const int w = (b - p.tile_begin[lo]) * PAIR_WARPS + ((int)threadIdx.x >> 5);
+    int band, strip;
+    tile_divmod(w, p.strips[lo], p.inv_d[lo], band, strip);
+    const int y0 = band * p.band[lo];
+    const int nx = a.nx, ny = a.ny, pitch = a.pitch;
+    if (y0 >= ny) return;   // the whole warp leaves together
+    const int y1 = y0 + p.band[lo] < ny ? y0 + p.band[lo] : ny;
+    const S* __restrict__ F = static_cast<const S*>(a.f);
+    S* __restrict__ O = static_cast<S*>(p.out[lo]);
+    const long long plane = a.plane;
+
+    const int c = strip * PAIR_AB_W - 4 + 2 * lane;
+    const int ca = ((c % nx) + nx) % nx, cb = ca + 1 == nx ? 0 : ca + 1;
+    const bool vec = __all_sync(0xffffffffu, !(ca & 1) && cb == ca + 1);
+    const bool inner = lane >= 2 && lane <= 29;
+    const bool st_a = inner && c < nx, st_b = inner && c + 1 < nx;
+
+    // FP32 rows arrive through a ring of shared memory that each lane fills for
+    // itself (asynchronous copies, PAIR_AB_AHEAD - 1 rows in flight per warp): one
+    // row ahead in registers kept 27 KB in flight per SM, a third of what HBM's
+    // latency needs (2048^2 60 us per step, 35 with the ring).  16-bit rows, half
+    // the bytes and four-byte copies, are loaded into registers one row ahead
+    // (33.5, and 38.7 through the ring).
+    constexpr bool RING = sizeof(S) == 4;
+    __shared__ P ring[PAIR_WARPS][RING ? PAIR_AB_AHEAD : 1][9][32];
+    P(*slot)[9][32] = ring[threadIdx.x >> 5];
+    P ahead[9];
+    const int rl = y1 + 3;                           // last row the band needs
+    int yl = ((y0 - 4) % ny + ny) % ny, rn = y0 - 4; // the row copied next, wrapped and not
+    auto copy_row = [&]() {
+        if (rn <= rl) {
+            const unsigned r = (unsigned)(yl * pitch);
+            P(*to)[32] = slot[RING ? (rn - y0 + 4) % PAIR_AB_AHEAD : 0];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const S* q = F + i * plane + r;
+                if constexpr (!RING) {
+                    ahead[i] = vec ? *reinterpret_cast<const P*>(q + ca) : K::join(q[ca], q[cb]);
+                } else if (vec) {
+                    copy_async<8>(&to[i][lane], q + ca);
+                } else {
+                    copy_async<4>(&to[i][lane], q + ca);
+                    copy_async<4>(reinterpret_cast<char*>(&to[i][lane]) + 4, q + cb);
+                }
+            }
+            yl = yl == ny - 1 ? 0 : yl + 1;
+        }
+        ++rn;
+        if (RING) asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto both = [](float v) { return f2(v, v); };
+    auto moments = [&](const P (&E)[9]) {
+        f2 d[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) d[i] = f2(K::lo(E[i]), K::hi(E[i]));
+        return node_moments<f2>(d, both(a.hgx), both(a.hgy), both(a.rho0));
+    };
+    // the collision of a row from its moments and the Phi around it
+    auto collide_row = [&](const NodeMom<f2>& m, f2 hx, f2 up, f2 down, P (&N)[9]) {
+        float x0, x1;
+        unpk(hx.v, x0, x1);
+        const float l = shfl_up1(x1), r = shfl_down1(x0);
+        const f2 half = f2(0.5);
+        const f2 dpx = rmul(half, rsub(f2(x1, r), f2(l, x0))), dpy = rmul(half, rsub(up, down));
+        f2 o[9], px, py;
+        collide_from<f2>(m, dpx, dpy, both(a.k1), both(a.k1lo), both(a.k2), both(a.k2lo), both(a.kf), both(a.gx),
+                         both(a.gy), o, px, py);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            float u, v;
+            unpk(o[i].v, u, v);
+            N[i] = K::make(u, v);
+        }
+    };
+    // three rows of collided populations, of which the middle one's streamed state
+    // is complete when the third arrives
+    struct Ring {
+        P B2, B5, B6, C0, C1, C3, C2, C5, C6;
+        __device__ __forceinline__ void take(const P (&N)[9], P (&E)[9]) {
+            E[0] = C0; E[1] = K::up(C1); E[2] = B2; E[3] = K::down(C3); E[4] = N[4];
+            E[5] = K::up(B5); E[6] = K::down(B6); E[7] = K::down(N[7]); E[8] = K::up(N[8]);
+            B2 = C2; B5 = C5; B6 = C6;
+            C0 = N[0]; C1 = N[1]; C3 = N[3]; C2 = N[2]; C5 = N[5]; C6 = N[6];
+        }
+    };
+    const f2 zero = f2(0.0);
+    Ring R{}, Q{};
+    NodeMom<f2> mp{}, mq{};
+    f2 hxp = zero, hyp = zero, hypp = zero, hxq = zero, hyq = zero, hyqq = zero;
+#pragma unroll
+    for (int k = 0; k < (RING ? PAIR_AB_AHEAD - 1 : 1); ++k) copy_row();
+    for (int r = y0 - 4; r <= rl; ++r) {
+        if (RING) asm volatile("cp.async.wait_group %0;" ::"n"(PAIR_AB_AHEAD - 2) : "memory");
+        P L[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) L[i] = RING ? slot[(r - y0 + 4) % PAIR_AB_AHEAD][i][lane] : ahead[i];
+        copy_row();                                  // into the slot read a row ago
+        const NodeMom<f2> m = moments(L);
+        const f2 hy = phi_of(m.rho, m.uy);
+        if (r > y0 - 3) {                            // rows up to y0 - 4 do not collide
+            P N[9], E[9];
+            collide_row(mp, hxp, hy, hypp, N);       // row r - 1
+            R.take(N, E);                            // f(t + 1) of row r - 2
+            const NodeMom<f2> m2 = moments(E);
+            const f2 hy2 = phi_of(m2.rho, m2.uy);
+            if (r > y0 + 1) {
+                collide_row(mq, hxq, hy2, hyqq, N);  // row r - 3
+                Q.take(N, E);                        // f(t + 2) of row r - 4
+                if (r >= y0 + 4) {
+                    const unsigned at = (unsigned)((r - 4) * pitch + c);
+                    if (st_b) {
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) *reinterpret_cast<P*>(O + i * plane + at) = E[i];
+                    } else if (st_a) {
+#pragma unroll
+                        for (int i = 0; i < 9; ++i) O[i * plane + at] = K::first(E[i]);
+                    }
+                }
+            }
+            mq = m2;
+            hxq = phi_of(m2.rho, m2.ux);
+            hyqq = hyq;
+            hyq = hy2;
+        }
+        mp = m;
+        hxp = phi_of(m.rho, m.ux);
+        hypp = hyp;
+        hyp = hy;
+    }
 }
 
 }  // namespace trt

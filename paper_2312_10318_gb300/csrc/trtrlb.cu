@@ -213,7 +213,8 @@ bool pair_applies(const trtrlb_params& p, const uint8_t* mask) {
 }
 
 bool two_step_on(const trtrlb_lattice* h) {
-    return h->variant == TRTRLB_KERNEL_AUTO && h->p.g_mode != TRTRLB_G_CURRENT && h->f2;
+    if (h->variant != TRTRLB_KERNEL_AUTO || !h->f2 || h->phi_given) return false;
+    return h->p.g_mode != TRTRLB_G_CURRENT || (!h->s.general && elem_size(h->p.storage) <= 4 && h->p.nx >= 32);
 }
 
 // Default two-buffer kernel of a G_CURRENT lattice that is periodic without a
@@ -550,7 +551,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
             cudaGetLastError();
         }
     }
-    if (s.pair) {
+    if (s.pair && p.g_mode != TRTRLB_G_CURRENT) {
         std::lock_guard<std::mutex> lk(g_spares_mu);
         g_spares.push_back(h);
         g_spares_bytes += es * 9 * (size_t)plane;
@@ -738,7 +739,8 @@ int trtrlb_set_f(trtrlb_t h, const double* f, const double* phi) {
     if (e != cudaSuccess) return cuda_fail(h->err, e, "set_f");
     // a Phi given for solid and moving-wall nodes sits in one of the two buffers,
     // which single steps read in turn and the two-step kernel does not
-    h->s.pair = two_step_on(h) && !(phi && h->mask);
+    if (phi && h->mask) h->phi_given = true;
+    h->s.pair = two_step_on(h);
     h->t = 0;
     return TRTRLB_OK;
 }
@@ -959,7 +961,7 @@ cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st) {
     while (n > 0) {
         cudaError_t e;
         int k = 1;
-        if (h->s.pair && h->s.parity == 1 && n >= 2) {
+        if (h->s.pair && (h->s.parity == 1 || h->s.g_mode == TRTRLB_G_CURRENT) && n >= 2) {
             const State* one = &h->s;
             e = TRT_DISPATCH(h->p.storage, step_pair(&one, 1, st));
             if (e == cudaSuccess) after_pair(h->s);

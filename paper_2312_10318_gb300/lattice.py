@@ -266,9 +266,10 @@ class Lattice:
 
 
 class Batch:
-    """Several lattices advanced together: one kernel launch per storage format and
-    time step, replayed from a CUDA graph for runs of 32+ steps on a non-default
-    stream.  Results equal stepping each lattice alone."""
+    """Several lattices advanced together: one kernel launch per storage format,
+    boundary flavour and time step (or two steps, Lattice.two_step), the formats
+    beside one another, replayed from a CUDA graph for runs of 32+ steps on a
+    non-default stream.  Results equal stepping each lattice alone."""
 
     def __init__(self, stream=None):
         lib = _lib.load()

@@ -64,8 +64,10 @@ class Result:
 
 
 def lattice_bytes(n_x: int, n_y: int, storage: str) -> int:
-    """Device bytes of one lattice as the library allocates it: populations
-    (9 per node), two Phi buffers of two components, the diagnostics scratch."""
+    """Device bytes a lattice needs: populations (9 per node), two Phi buffers of two
+    components, the diagnostics scratch.  The two-step kernel's second population
+    buffer is not counted: the library allocates it only while half of the device
+    stays free (or such buffers take at most 4 GiB in all)."""
     pitch = (n_x + 63) // 64 * 64
     plane = pitch * n_y
     phi = 8 if storage in ("f64", "f64dw") else 4

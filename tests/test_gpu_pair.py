@@ -166,3 +166,32 @@ def test_many_narrow_lattices_share_launches(gpu_lib):
     torch.cuda.synchronize()
     for q, (a, b) in enumerate(zip(alone, members)):
         assert _same(a, b), q
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+def test_two_current_phi_steps_equal_single_steps(gpu_lib, storage):
+    """With Phi at the current level (56 nodes stored per strip): the same bits as
+    the plain and the column kernel's single steps."""
+    for k, (nx, ny) in enumerate([(32, 1), (33, 2), (55, 3), (56, 5), (57, 130), (58, 4), (113, 9), (250, 246)]):
+        a, c, b = _lattices(nx, ny, storage, "current", k, n=3)
+        a.set_kernel("scalar")
+        c.set_kernel("column")
+        assert b.two_step() and not a.two_step()
+        for n in (1, 2, 3, 6):
+            for lat in (a, b, c):
+                lat.step(n)
+            assert _same(a, b) and _same(c, b), (nx, ny, n)
+
+
+@pytest.mark.parametrize("g_mode", ["lagged", "off"])
+def test_double_word_two_nodes_per_thread(gpu_lib, g_mode):
+    """The periodic double-word step's pairs of rows (heights with a row left over,
+    narrow and wide tiles) against FP64 storage."""
+    for nx, ny, kw in [(64, 1, {}), (5, 3, {}), (40, 3, {}), (130, 33, {}), (300, 131, {}), (900, 901, {})]:
+        rho, ux, uy = W.random_fields(nx, ny, seed=nx, u_amp=0.05, rho_amp=0.01)
+        from paper_2312_10318_gb300 import Lattice
+        a, b = [Lattice(nx, ny, 0.7, tau_s2=0.9, g=(2e-5, -1e-5), storage=s, g_mode=g_mode, **kw)
+                .init(ux, uy, rho).step(5) for s in ("f64", "f64dw")]
+        fa, fb = a.get_f(), b.get_f()
+        # 5 steps of the format's 2^-47 relative to the largest population
+        assert np.abs(fa - fb).max() <= 1e-12 * np.abs(fa).max(), (nx, ny)
