@@ -109,7 +109,25 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
+// FP64 on this GPU: an instruction holds a quarter of an SM's pipe for 64 cycles, so
+// what can be done without one is.  The reciprocal is the 20-bit approximation and
+// one third-order (Halley) step, r (1 + e + e^2) with e = 1 - a r: three FMAs, error
+// below 2^-60 before the last rounding.
+__device__ __forceinline__ double rrcp(double a) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
+    const double e = __fma_rn(-a, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+// x 2^-K, exact: the exponent field in integer arithmetic (zero and values whose
+// exponent could leave the normal range take the multiplication).
+template <int K>
+__device__ __forceinline__ double rscale(double x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x);
+    const unsigned e = (unsigned)hi & 0x7ff00000u;
+    if (e - (8u << 20) < (2030u << 20)) return __hiloint2double(hi - (K << 20), lo);
+    return x == 0.0 ? x : __dmul_rn(x, 1.0 / (1 << K));
+}
 __device__ __forceinline__ float rneg(float a) { return -a; }
 __device__ __forceinline__ double rneg(double a) { return -a; }
 __device__ __forceinline__ df64 radd(const df64& a, const df64& b) { return a + b; }
@@ -134,6 +152,23 @@ __device__ __forceinline__ f2 rrcp(f2 a) {
     float x, y;
     unpk(a.v, x, y);
     return f2(__frcp_rn(x), __frcp_rn(y));
+}
+
+// Scalings by powers of two: a multiplication, in FP64 integer arithmetic.
+template <typename C>
+__device__ __forceinline__ C half_of(const C& d) {
+    if constexpr (std::is_same<C, double>::value) return rscale<1>(d);
+    else return C(0.5) * d;
+}
+template <typename C>
+__device__ __forceinline__ C minus_half_of(const C& d) {
+    if constexpr (std::is_same<C, double>::value) return -rscale<1>(d);
+    else return rmul(C(-0.5), d);
+}
+template <typename C>
+__device__ __forceinline__ C quarter_of(const C& d) {
+    if constexpr (std::is_same<C, double>::value) return rscale<2>(d);
+    else return rmul(C(0.25), d);
 }
 
 // Zou-He constant-pressure outlet (Sec. III D) on the shifted populations
@@ -418,17 +453,17 @@ __device__ __forceinline__ void collide_from(const NodeMom<C>& m, C dpx, C dpy, 
     o[0] = rfma(C(4.0 / 9.0), drho, rmul(C(-2.0 / 3.0), t));
     const C b9 = rmul(C(1.0 / 9.0), drho);
     const C c13 = rfma(C(-1.0 / 6.0), a2yy, rfma(C(1.0 / 3.0), a2xx, b9));
-    const C o13 = rfma(C(1.0 / 3.0), a1x, rmul(C(-0.5), a3xyy));
+    const C o13 = rfma(C(1.0 / 3.0), a1x, minus_half_of<C>(a3xyy));
     const C c24 = rfma(C(-1.0 / 6.0), a2xx, rfma(C(1.0 / 3.0), a2yy, b9));
-    const C o24 = rfma(C(1.0 / 3.0), a1y, rmul(C(-0.5), a3xxy));
+    const C o24 = rfma(C(1.0 / 3.0), a1y, minus_half_of<C>(a3xxy));
     o[1] = radd(c13, o13);
     o[3] = rsub(c13, o13);
     o[2] = radd(c24, o24);
     o[4] = rsub(c24, o24);
     const C cd = rfma(C(1.0 / 12.0), t, rmul(C(1.0 / 36.0), drho));
     const C c57 = rfma(C(0.25), a2xy, cd), c68 = rfma(C(-0.25), a2xy, cd);
-    const C o57 = rfma(C(1.0 / 12.0), radd(a1x, a1y), rmul(C(0.25), radd(a3xxy, a3xyy)));
-    const C o68 = rfma(C(1.0 / 12.0), rsub(a1y, a1x), rmul(C(0.25), rsub(a3xxy, a3xyy)));
+    const C o57 = rfma(C(1.0 / 12.0), radd(a1x, a1y), quarter_of<C>(radd(a3xxy, a3xyy)));
+    const C o68 = rfma(C(1.0 / 12.0), rsub(a1y, a1x), quarter_of<C>(rsub(a3xxy, a3xyy)));
     o[5] = radd(c57, o57);
     o[7] = rsub(c57, o57);
     o[6] = radd(c68, o68);
@@ -537,8 +572,8 @@ __device__ __forceinline__ void periodic_load(const Args<typename Fmt<S>::C>& a,
     if (GMODE == G_LAGGED) {
         const C* Px = a.phi_in + own;
         const C* Py = a.phi_in + a.plane + own;
-        dpx = C(0.5) * (Px[1 + cxp] - Px[-1 + cxm]);
-        dpy = C(0.5) * (Py[pt + cyp] - Py[-pt + cym]);
+        dpx = half_of<C>(Px[1 + cxp] - Px[-1 + cxm]);
+        dpy = half_of<C>(Py[pt + cyp] - Py[-pt + cym]);
     }
 }
 
@@ -615,8 +650,8 @@ __device__ __forceinline__ void node_step_periodic(const Args<typename Fmt<S>::C
     if (GMODE == G_LAGGED) {
         const C* Px = a.phi_in + own;
         const C* Py = a.phi_in + a.plane + own;
-        dpx = C(0.5) * (Px[1 + cxp] - Px[-1 + cxm]);
-        dpy = C(0.5) * (Py[pt + cyp] - Py[-pt + cym]);
+        dpx = half_of<C>(Px[1 + cxp] - Px[-1 + cxm]);
+        dpy = half_of<C>(Py[pt + cyp] - Py[-pt + cym]);
     }
     C o[9], phx, phy;
     collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
@@ -693,8 +728,8 @@ __device__ __forceinline__ void node_step(const Args<typename Fmt<S>::C>& a, int
         const C pxm = (GENERAL && n.oxm) ? C(0) : Px[y * a.pitch + n.xm];
         const C pyp = (GENERAL && n.oyp) ? C(0) : Py[n.yp * a.pitch + x];
         const C pym = (GENERAL && n.oym) ? C(0) : Py[n.ym * a.pitch + x];
-        dpx = C(0.5) * (pxp - pxm);
-        dpy = C(0.5) * (pyp - pym);
+        dpx = half_of<C>(pxp - pxm);
+        dpy = half_of<C>(pyp - pym);
     }
     C o[9], phx, phy;
     collide<C>(d, dpx, dpy, a.k1, a.k1lo, a.k2, a.k2lo, a.kf, a.gx, a.gy, a.hgx, a.hgy, a.rho0, o, phx, phy);
