@@ -116,23 +116,22 @@ std::vector<Class> classes_of(const trtrlb_batch* b, const std::vector<trt::Stat
 
 // n steps of the members of class c from the states `sim`, which it advances.
 // Where the two-step kernel runs them: a single step to an odd level, two at a
-// time, and a single step for an odd rest.  closed: n is kGraphSteps and the
-// members must end at the parity and on the buffers they began with, so that the
-// launches can be replayed: every count of flips must be even, which 16 launches
-// of two steps from an odd level are, and, from an even one, a single step, 14
-// launches of two and three single steps.
+// time, and single steps for the rest.  closed: the members end on the buffers
+// that single steps would have left them at (trt::pair_launches); with n =
+// kGraphSteps those are the ones they began on, and the launches can be replayed.
 cudaError_t launch_class(trtrlb_batch* b, const Class& c, std::vector<trt::State>& sim, int64_t n, bool closed,
                          cudaStream_t st) {
     std::vector<const trt::State*> m;
     for (int i : c.members) m.push_back(&sim[i]);
     const int k = (int)m.size();
-    const int64_t last = closed && c.parity == 0 ? n - 3 : n;   // no launch of two steps ends after it
+    int64_t pairs = trt::pair_launches(*m[0], n, closed);
     int parity = c.parity;
     for (int64_t q = 0; q < n;) {
         cudaError_t e;
-        if (c.g_mode == TRTRLB_G_CURRENT && c.pair && q + 2 <= n) {
+        if (pairs > 0 && (parity == 1 || c.g_mode == TRTRLB_G_CURRENT)) {
             e = TRT_DISPATCH_S(c.storage, step_pair(m.data(), k, st));
             for (int i : c.members) trt::after_pair(sim[i]);
+            --pairs;
             q += 2;
         } else if (c.g_mode == TRTRLB_G_CURRENT) {
             e = c.tma ? trt::Ops<float>::step_ab_group(m.data(), k, st)
@@ -141,10 +140,6 @@ cudaError_t launch_class(trtrlb_batch* b, const Class& c, std::vector<trt::State
                 e = TRT_DISPATCH_S(c.storage, step_ab(*m[i], st));
             for (int i : c.members) std::swap(sim[i].f, sim[i].f2);
             q += 1;
-        } else if (c.pair && parity == 1 && q + 2 <= last) {
-            e = TRT_DISPATCH_S(c.storage, step_pair(m.data(), k, st));
-            for (int i : c.members) trt::after_pair(sim[i]);
-            q += 2;
         } else {
             e = TRT_DISPATCH_S(c.storage, step_group(m.data(), k, parity != 0, c.flavour, c.g_mode, st));
             for (int i : c.members) {
@@ -167,7 +162,7 @@ cudaError_t launch_class(trtrlb_batch* b, const Class& c, std::vector<trt::State
 // Kernels that issue bounds (double-word) and kernels that memory bounds then
 // share the SMs, and small classes run beside large ones: the 240 channels of
 // three formats in 20.0 us per step (60 in line before, with 32-wide tiles).
-cudaError_t launch_steps(trtrlb_batch* b, std::vector<trt::State>& sim, int64_t n, bool closed = false) {
+cudaError_t launch_steps(trtrlb_batch* b, std::vector<trt::State>& sim, int64_t n, bool closed) {
     if (n == 0) return cudaSuccess;
     std::vector<Class> cs = classes_of(b, sim);
     if (b->stream == nullptr || cs.size() == 1) {
@@ -303,20 +298,24 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
     b->err[0] = 0;
     if (nsteps < 0) return fail(b, TRTRLB_EINVAL, "nsteps must be >= 0");
     if (nsteps == 0 || b->lats.empty()) return TRTRLB_OK;
+    bool capturing = false, closed = false;
+    cudaError_t e = trt::capturing(b->stream, &capturing);
+    if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
     std::vector<trt::State> sim;
     for (trtrlb_lattice* h : b->lats) {
         trt::keep_spare(h);   // graphs name it
+        h->captured = h->captured || capturing;
+        closed = closed || h->captured;
         sim.push_back(h->s);
     }
     int64_t done = 0;
-    cudaError_t e = cudaSuccess;
     if (b->stream != nullptr && nsteps >= kGraphSteps) {
         // to odd levels, where the runs of two start, if that is a step for all
         bool odd_pair = false, even_pair = false;
         for (const trt::State& x : sim)
             if (x.g_mode != TRTRLB_G_CURRENT) (x.parity ? odd_pair : even_pair) |= x.pair;
         if (even_pair && !odd_pair && nsteps > kGraphSteps) {
-            e = launch_steps(b, sim, 1);
+            e = launch_steps(b, sim, 1, closed);
             done = 1;
             if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
         }
@@ -327,7 +326,7 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
             if (e != cudaSuccess) return cuda_fail(b, e, "graph launch");
         }
     }
-    e = launch_steps(b, sim, nsteps - done);
+    e = launch_steps(b, sim, nsteps - done, closed);
     if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
     for (size_t i = 0; i < sim.size(); ++i) {
         b->lats[i]->s = sim[i];

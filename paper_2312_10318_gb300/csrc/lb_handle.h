@@ -34,6 +34,7 @@ struct trtrlb_lattice {
     std::mutex spare_mu; // held while launches that use f2 of a lagged lattice are queued
     bool phi_given;      // trtrlb_set_f gave a Phi to a lattice with a mask
     bool spare_kept;     // f2 is named by a captured graph: not given back before the handle
+    bool captured;       // a caller's graph holds steps of it: see trt::pair_launches
     char err[256];
 };
 
@@ -52,6 +53,29 @@ namespace trt {
 // Keeps the two-step kernel's second buffer of h for the handle's lifetime
 // (launches that use it are captured, or queued outside advance()).
 void keep_spare(trtrlb_lattice* h);
+
+// Whether st is being captured into a caller's graph.
+inline cudaError_t capturing(cudaStream_t st, bool* on) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+    *on = cs != cudaStreamCaptureStatusNone;
+    return e;
+}
+
+// Launches of two steps in a run of n steps of a lattice that takes them (the
+// other steps are single ones): from odd levels with Phi lagged or no G, so that
+// a run from an even one begins with a single step, from any level with Phi at
+// the current one.  Each swaps the population buffers, and with Phi lagged the
+// Phi buffers once for two steps.  even: an even number of them, after which the
+// lattice is at the parity and on the buffers that single steps would have left
+// it at; graphs that are replayed need that, and so does every run of a lattice
+// that a caller's graph names.
+inline int64_t pair_launches(const State& s, int64_t n, bool even) {
+    if (!s.pair) return 0;
+    const int64_t first = s.g_mode != TRTRLB_G_CURRENT && s.parity == 0 ? 1 : 0;
+    const int64_t k = n > first ? (n - first) / 2 : 0;
+    return even ? k & ~(int64_t)1 : k;
+}
 
 // Advances h by n time steps on st: two at a time from odd levels where the
 // two-step kernel runs the lattice.

@@ -952,19 +952,20 @@ void keep_spare(trtrlb_lattice* h) {
 
 cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(h->spare_mu);
-    if (h->s.pair && !h->spare_kept) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+    if (h->s.f2 && !h->captured) {
+        const cudaError_t e = capturing(st, &h->captured);
         if (e != cudaSuccess) return e;
-        h->spare_kept = cs != cudaStreamCaptureStatusNone;
+        h->spare_kept = h->spare_kept || h->captured;
     }
+    int64_t pairs = pair_launches(h->s, n, h->captured);
     while (n > 0) {
         cudaError_t e;
         int k = 1;
-        if (h->s.pair && (h->s.parity == 1 || h->s.g_mode == TRTRLB_G_CURRENT) && n >= 2) {
+        if (pairs > 0 && (h->s.parity == 1 || h->s.g_mode == TRTRLB_G_CURRENT)) {
             const State* one = &h->s;
             e = TRT_DISPATCH(h->p.storage, step_pair(&one, 1, st));
             if (e == cudaSuccess) after_pair(h->s);
+            --pairs;
             k = 2;
         } else {
             e = TRT_DISPATCH(h->p.storage, step(h->s, st));
