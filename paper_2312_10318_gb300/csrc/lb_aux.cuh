@@ -106,6 +106,21 @@ __global__ void k_phi_static(const uint8_t* __restrict__ mask, int nx, int ny, i
     phi1[k] = vx; phi1[plane + k] = vy;
 }
 
+// *differ = 1 if the two Phi buffers differ in a bit at a node whose Phi no step
+// changes (a Phi given to trtrlb_set_f sits in one of them).
+static __global__ void k_phi_static_differs(const uint8_t* __restrict__ mask, int nx, int ny, int pitch,
+                                            long long plane, const float* __restrict__ phi0,
+                                            const float* __restrict__ phi1, int* differ) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x;
+    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= nx || y >= ny) return;
+    const long long k = (long long)y * pitch + x;
+    if (collides(mask[k]) || mask[k] == OUTLET) return;
+    if (__float_as_uint(phi0[k]) != __float_as_uint(phi1[k]) ||
+        __float_as_uint(phi0[plane + k]) != __float_as_uint(phi1[plane + k]))
+        *differ = 1;
+}
+
 // Phi(s) := Phi(s - (1,0)) for every outlet ghost s, in one buffer.
 template <typename C>
 __global__ void k_ghost_phi(const int* __restrict__ ghosts, int nghost, int nx, int pitch,

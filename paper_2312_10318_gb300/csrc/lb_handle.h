@@ -32,7 +32,7 @@ struct trtrlb_lattice {
     int tma_grid;        // persistent grid of the TMA kernel on this device (0: none)
     int sms;             // multiprocessors of the handle's device
     std::mutex spare_mu; // held while launches that use f2 of a lagged lattice are queued
-    bool phi_given;      // trtrlb_set_f gave a Phi to a lattice with a mask
+    bool phi_given;      // the Phi buffers may differ at nodes whose Phi no step changes
     bool spare_kept;     // f2 is named by a captured graph: not given back before the handle
     bool captured;       // a caller's graph holds steps of it: see trt::pair_launches
     char err[256];

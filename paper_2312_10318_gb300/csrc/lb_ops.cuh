@@ -84,6 +84,9 @@ template <typename S> struct Ops {
     // Fills a general lattice's maps of the two-step kernel.
     static cudaError_t pair_maps(const State& s, unsigned* info, unsigned* special, cudaStream_t st);
     static cudaError_t phi_static(State& s, cudaStream_t st);
+    // *differ (device) := whether the Phi buffers of a lattice with a mask differ
+    // at nodes whose Phi no step changes; formats of the two-step kernel only.
+    static cudaError_t phi_static_differs(const State& s, int* differ, cudaStream_t st);
     static cudaError_t init(State& s, const double* rho, const double* ux, const double* uy,
                             cudaStream_t st);
     static cudaError_t moments(const State& s, double* rho, double* ux, double* uy,

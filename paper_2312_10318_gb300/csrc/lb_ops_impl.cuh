@@ -288,6 +288,22 @@ cudaError_t Ops<S>::phi_static(State& s, cudaStream_t st) {
 }
 
 template <typename S>
+cudaError_t Ops<S>::phi_static_differs(const State& s, int* differ, cudaStream_t st) {
+    if constexpr (sizeof(S) <= 4) {
+        const cudaError_t e = cudaMemsetAsync(differ, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
+        const dim3 b(32, 8);
+        k_phi_static_differs<<<grid2d(s, b), b, 0, st>>>(s.mask, s.nx, s.ny, s.pitch, s.plane,
+                                                         static_cast<const float*>(s.phi[0]),
+                                                         static_cast<const float*>(s.phi[1]), differ);
+        return cudaGetLastError();
+    } else {
+        (void)s; (void)differ; (void)st;
+        return cudaErrorInvalidValue;
+    }
+}
+
+template <typename S>
 cudaError_t Ops<S>::init(State& s, const double* rho, const double* ux, const double* uy,
                          cudaStream_t st) {
     using C = typename Fmt<S>::C;

@@ -217,6 +217,20 @@ bool two_step_on(const trtrlb_lattice* h) {
     return h->p.g_mode != TRTRLB_G_CURRENT || (!h->s.general && elem_size(h->p.storage) <= 4 && h->p.nx >= 32);
 }
 
+// Whether the Phi buffers of h differ at nodes whose Phi no step changes, which
+// single steps read in turn and the two-step kernel does not (synchronises the
+// stream of a lattice that the kernel could take).
+cudaError_t phi_given_now(trtrlb_lattice* h, bool* given) {
+    *given = false;
+    if (!h->mask || h->p.g_mode != TRTRLB_G_LAGGED || elem_size(h->p.storage) > 4) return cudaSuccess;
+    int differ = 0, *flag = reinterpret_cast<int*>(h->dout);
+    cudaError_t e = TRT_DISPATCH(h->p.storage, phi_static_differs(h->s, flag, h->stream));
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&differ, flag, sizeof differ, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    *given = differ != 0;
+    return e;
+}
+
 // Default two-buffer kernel of a G_CURRENT lattice that is periodic without a
 // mask: for FP64, FP16 and BF16 storage the column-walking kernel wherever its
 // bands give enough warps (trt::col_band_rows; on 3 x 4096^2 it stepped FP16
@@ -709,10 +723,14 @@ int trtrlb_load(trtrlb_t h, const void* image) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(h->phi, in + sizeof hd + image_pop_bytes(h), image_phi_bytes(h),
                             cudaMemcpyDefault, h->stream);
+    bool given = false;
+    if (e == cudaSuccess) e = phi_given_now(h, &given);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h->err, e, "load");
     h->s.parity = hd.parity;
     h->s.cur = hd.cur;
+    h->phi_given = given;
+    h->s.pair = two_step_on(h);
     h->t = hd.t;
     return TRTRLB_OK;
 }
