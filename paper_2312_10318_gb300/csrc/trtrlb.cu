@@ -524,8 +524,8 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
         }
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(h->f, 0, es * 9 * plane, h->stream);
-    if (e == cudaSuccess && h->f2 && p.g_mode == TRTRLB_G_CURRENT)   // the two-step kernel writes before it reads
-        e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
+    // no step writes padding columns and solid nodes, and images hold them
+    if (e == cudaSuccess && h->f2) e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
     if (e == cudaSuccess) e = TRT_DISPATCH(p.storage, phi_static(h->s, h->stream));
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
