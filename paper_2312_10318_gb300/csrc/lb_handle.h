@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "lb_ops.cuh"
@@ -24,14 +25,17 @@ struct trtrlb_lattice {
     int stage_fields;    // its size in fields of nx * ny doubles (3, 4 or 11)
     double* part;        // diagnostics partials (scratch)
     double* dout;        // result of diagnostics (8 doubles) and comparisons (TRTRLB_CMP_N)
-    int64_t bytes;
+    std::atomic<int64_t> bytes;   // (another thread's reclaim_spares lowers it)
     int tile_w;          // scalar-kernel tile width in the batched path (32 .. 256 nodes)
     int variant;         // TRTRLB_KERNEL_AUTO / SCALAR / VECTOR
     void* tmaps;         // two CUtensorMap (host) of the FP32 periodic G_CURRENT kernel, or null
     int* kerr;           // device flag set when a kernel's bounded wait ran out, or null
     int tma_grid;        // persistent grid of the TMA kernel on this device (0: none)
     int sms;             // multiprocessors of the handle's device
-    std::mutex spare_mu; // held while launches that use f2 of a lagged lattice are queued
+    // Another thread's failed allocation may give back f2 of a lagged lattice
+    // (reclaim_spares): held there, and by every call that reads or writes f2, s.f2
+    // or s.pair after create.
+    std::mutex spare_mu;
     bool phi_given;      // the Phi buffers may differ at nodes whose Phi no step changes
     bool spare_kept;     // f2 is named by a captured graph: not given back before the handle
     bool captured;       // a caller's graph holds steps of it: see trt::pair_launches

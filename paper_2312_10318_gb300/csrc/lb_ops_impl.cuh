@@ -509,6 +509,8 @@ cudaError_t Ops<S>::pair_maps(const State& s, unsigned* info, unsigned* special,
 template <typename S>
 cudaError_t Ops<S>::step_pair(const State* const* m, int n, cudaStream_t st) {
     if constexpr (sizeof(S) <= 4) {
+        for (int q = 0; q < n; ++q)
+            if (!m[q]->f2) return cudaErrorInvalidValue;
         for (int q0 = 0; q0 < n; q0 += GROUP_MAX) {
             const int c = n - q0 < GROUP_MAX ? n - q0 : GROUP_MAX;
             const cudaError_t e = m[q0]->general ? launch_pair_g<S, true>(m + q0, c, st)

@@ -112,8 +112,9 @@ void reclaim_spares() {
     std::lock_guard<std::mutex> lk(g_spares_mu);
     for (size_t i = 0; i < g_spares.size();) {
         trtrlb_lattice* h = g_spares[i];
-        std::unique_lock<std::mutex> hl(h->spare_mu, std::try_to_lock);
-        if (!hl.owns_lock() || h->spare_kept) {
+        // (a thread that is queueing steps is waited for; none allocates meanwhile)
+        std::lock_guard<std::mutex> hl(h->spare_mu);
+        if (h->spare_kept) {
             ++i;
             continue;
         }
@@ -212,6 +213,7 @@ bool pair_applies(const trtrlb_params& p, const uint8_t* mask) {
     return true;
 }
 
+// (h->spare_mu held, or h not yet known to other threads)
 bool two_step_on(const trtrlb_lattice* h) {
     if (h->variant != TRTRLB_KERNEL_AUTO || !h->f2 || h->phi_given) return false;
     return h->p.g_mode != TRTRLB_G_CURRENT || (!h->s.general && elem_size(h->p.storage) <= 4 && h->p.nx >= 32);
@@ -729,9 +731,10 @@ int trtrlb_load(trtrlb_t h, const void* image) {
     if (e != cudaSuccess) return cuda_fail(h->err, e, "load");
     h->s.parity = hd.parity;
     h->s.cur = hd.cur;
-    h->phi_given = given;
-    h->s.pair = two_step_on(h);
     h->t = hd.t;
+    h->phi_given = given;
+    std::lock_guard<std::mutex> lk(h->spare_mu);
+    h->s.pair = two_step_on(h);
     return TRTRLB_OK;
 }
 
@@ -758,8 +761,9 @@ int trtrlb_set_f(trtrlb_t h, const double* f, const double* phi) {
     // a Phi given for solid and moving-wall nodes sits in one of the two buffers,
     // which single steps read in turn and the two-step kernel does not
     if (phi && h->mask) h->phi_given = true;
-    h->s.pair = two_step_on(h);
     h->t = 0;
+    std::lock_guard<std::mutex> lk(h->spare_mu);
+    h->s.pair = two_step_on(h);
     return TRTRLB_OK;
 }
 
@@ -860,7 +864,7 @@ int trtrlb_compare_lattices(trtrlb_t a, trtrlb_t b, double* out) {
 
 extern "C" {
 
-int64_t trtrlb_device_bytes(trtrlb_t h) { return h ? h->bytes : -1; }
+int64_t trtrlb_device_bytes(trtrlb_t h) { return h ? h->bytes.load() : -1; }
 
 int trtrlb_set_kernel(trtrlb_t h, int32_t variant, int32_t tile_w) {
     if (!h) return TRTRLB_EINVAL;
@@ -888,7 +892,10 @@ int trtrlb_set_kernel(trtrlb_t h, int32_t variant, int32_t tile_w) {
     }
     h->variant = variant;
     h->s.vec = vec;
-    h->s.pair = two_step_on(h);
+    {
+        std::lock_guard<std::mutex> lk(h->spare_mu);
+        h->s.pair = two_step_on(h);
+    }
     if (variant == TRTRLB_KERNEL_COLUMN) {
         // the tallest band that still fills the device, else the shortest
         const int es = (int)elem_size(h->p.storage);
@@ -921,6 +928,7 @@ int trtrlb_get_kernel(trtrlb_t h, int32_t* vector, int32_t* tile_w) {
 
 int trtrlb_two_step(trtrlb_t h, int32_t* on) {
     if (!h || !on) return TRTRLB_EINVAL;
+    std::lock_guard<std::mutex> lk(h->spare_mu);
     *on = h->s.pair ? 1 : 0;
     return TRTRLB_OK;
 }
