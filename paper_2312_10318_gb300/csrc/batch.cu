@@ -39,6 +39,7 @@ struct trtrlb_batch {
     // runs of kGraphSteps steps, captured once per start (parity, Phi buffer and
     // population buffer of every member), at most kMaxGraphs of them
     std::map<std::vector<int>, cudaGraphExec_t> graphs;
+    std::vector<SparePins*> held;      // the members' second buffers, while there are graphs
     char err[256] = "";
 };
 
@@ -57,7 +58,21 @@ int cuda_fail(trtrlb_batch* b, cudaError_t e, const char* where) {
 void drop_graphs(trtrlb_batch* b) {
     for (const auto& kv : b->graphs) cudaGraphExecDestroy(kv.second);
     b->graphs.clear();
+    for (SparePins* x : b->held) x->unpin();
+    b->held.clear();
 }
+
+// Pins the members' second buffers for the length of a call.
+struct CallPins {
+    std::vector<SparePins*> held;
+    ~CallPins() {
+        for (SparePins* x : held) x->unpin();
+    }
+    void add(SparePins* x) {
+        held.push_back(x);
+        x->pin();
+    }
+};
 
 std::vector<int> signature(const trtrlb_batch* b, const std::vector<trt::State>& sim) {
     std::vector<int> sig;
@@ -227,6 +242,11 @@ int graph_from(trtrlb_batch* b, const std::vector<trt::State>& sim, cudaGraphExe
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_fail(b, e, "graph instantiate");
     b->graphs[sig] = x;
+    if (b->held.empty())               // (pinned already for this call)
+        for (trtrlb_lattice* h : b->lats) {
+            b->held.push_back(h->pins);
+            h->pins->pin();
+        }
     *out = x;
     return TRTRLB_OK;
 }
@@ -302,8 +322,10 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
     cudaError_t e = trt::capturing(b->stream, &capturing);
     if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
     std::vector<trt::State> sim;
+    CallPins pins;
     for (trtrlb_lattice* h : b->lats) {
-        trt::keep_spare(h);   // graphs name it
+        std::lock_guard<std::mutex> lk(h->spare_mu);
+        pins.add(h->pins);
         h->captured = h->captured || capturing;
         closed = closed || h->captured;
         sim.push_back(h->s);

@@ -9,6 +9,18 @@
 #include "lb_ops.cuh"
 #include "trtrlb.h"
 
+// Who, beside the handle, names a lattice's second buffer: batches while a call or
+// a captured graph of theirs does.  A batch may outlive its members, so this does
+// too: refs counts the handle and the batches that hold it.
+struct SparePins {
+    std::atomic<int> refs{1}, pins{0};
+    void unref() {
+        if (--refs == 0) delete this;
+    }
+    void pin() { ++refs, ++pins; }
+    void unpin() { --pins, unref(); }
+};
+
 struct trtrlb_lattice {
     trtrlb_params p;
     trt::State s;
@@ -37,8 +49,8 @@ struct trtrlb_lattice {
     // or s.pair after create.
     std::mutex spare_mu;
     bool phi_given;      // the Phi buffers may differ at nodes whose Phi no step changes
-    bool spare_kept;     // f2 is named by a captured graph: not given back before the handle
-    bool captured;       // a caller's graph holds steps of it: see trt::pair_launches
+    SparePins* pins;     // f2 is not given back while something pins it
+    bool captured;       // nor ever, once a caller's graph holds steps of it (trt::pair_launches)
     char err[256];
 };
 
@@ -54,10 +66,6 @@ inline bool shares_tma_launch(const trtrlb_lattice* h) {
 }
 
 namespace trt {
-// Keeps the two-step kernel's second buffer of h for the handle's lifetime
-// (launches that use it are captured, or queued outside advance()).
-void keep_spare(trtrlb_lattice* h);
-
 // Whether st is being captured into a caller's graph.
 inline cudaError_t capturing(cudaStream_t st, bool* on) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

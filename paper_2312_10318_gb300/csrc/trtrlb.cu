@@ -104,8 +104,8 @@ bool spare_fits(size_t bytes) {
     return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b > bytes && free_b - bytes >= total_b / 2;
 }
 
-// Gives back the second buffers that no queued or captured launch will name
-// (cudaFree waits for the queued ones); the lattices go on with single steps.
+// Gives back the second buffers that no captured launch names (cudaFree waits for
+// the queued ones); the lattices go on with single steps.
 // Called when an allocation fails, so that the buffers never cost a caller a
 // lattice that would have fit without them.
 void reclaim_spares() {
@@ -114,7 +114,7 @@ void reclaim_spares() {
         trtrlb_lattice* h = g_spares[i];
         // (a thread that is queueing steps is waited for; none allocates meanwhile)
         std::lock_guard<std::mutex> hl(h->spare_mu);
-        if (h->spare_kept) {
+        if (h->captured || h->pins->pins > 0) {
             ++i;
             continue;
         }
@@ -155,6 +155,7 @@ void release(trtrlb_lattice* h) {
     if (h->dout) cudaFree(h->dout);
     if (h->kerr) cudaFree(h->kerr);
     delete[] static_cast<CUtensorMap*>(h->tmaps);
+    h->pins->unref();
     delete h;
 }
 
@@ -421,7 +422,11 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     }
 
     trtrlb_lattice* h = new (std::nothrow) trtrlb_lattice();
-    if (!h) return fail(err, TRTRLB_ENOMEM, "host allocation failed");
+    if (h) h->pins = new (std::nothrow) SparePins();
+    if (!h || !h->pins) {
+        delete h;
+        return fail(err, TRTRLB_ENOMEM, "host allocation failed");
+    }
     h->p = p;
     h->p.tau_s2 = tau2;
     h->p.magic = (p.tau_s - 0.5) * (tau2 - 0.5);
@@ -431,7 +436,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) {
-        delete h;
+        release(h);
         return cuda_fail(err, e, "device query");
     }
     auto alloc = [&](void** ptr, size_t bytes) {
@@ -971,17 +976,11 @@ static T* at(T* const* a, int k) {
     return a ? a[k] : nullptr;
 }
 
-void keep_spare(trtrlb_lattice* h) {
-    std::lock_guard<std::mutex> lk(h->spare_mu);
-    h->spare_kept = true;
-}
-
 cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(h->spare_mu);
     if (h->s.f2 && !h->captured) {
         const cudaError_t e = capturing(st, &h->captured);
         if (e != cudaSuccess) return e;
-        h->spare_kept = h->spare_kept || h->captured;
     }
     int64_t pairs = pair_launches(h->s, n, h->captured);
     while (n > 0) {
