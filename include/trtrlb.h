@@ -323,19 +323,33 @@ int trtrlb_get_kernel(trtrlb_t h, int32_t* vector, int32_t* tile_w);
 int trtrlb_step_kernel(trtrlb_t h, int32_t* kind);
 
 /* Whether runs of steps advance this lattice two steps per launch (*on = 1):
- * FP32, FP16 or BF16 storage, nx >= 32, TRTRLB_KERNEL_AUTO and
+ * FP32, FP16 or BF16 storage, nx >= 32, TRTRLB_KERNEL_AUTO (or
+ * trtrlb_set_two_step) and
  *   - G lagged or off: no node of the halo classes, no outlet ghost with a
  *     colliding node at x + 1 (any row of the three), and a second population
  *     buffer, which trtrlb_create allocates while such buffers take no more than
- *     4 GiB or leave half of the device's memory free, and which goes back when a
- *     later allocation of the library would fail.  The two steps start at an odd
- *     level: a run from an even one begins with a single step, and an odd rest
- *     ends it with one (trtrlb_step_kernel names that kernel).  A Phi given to
- *     trtrlb_set_f for a lattice with a mask leaves it to single steps;
+ *     64 MiB in all, or no more than a quarter of the device's memory with half of
+ *     it left free.  It goes back when a later allocation of the library would
+ *     fail, unless a captured run names it: a batch's (until trtrlb_batch_set or
+ *     trtrlb_batch_destroy) or a caller's graph with steps of the lattice (until
+ *     trtrlb_destroy); trtrlb_set_two_step(h, 0) gives it back for allocations
+ *     outside the library.  The two steps start at an odd level: a run from an
+ *     even one begins with a single step, and an odd rest ends it with one
+ *     (trtrlb_step_kernel names that kernel).  Where the two Phi buffers differ at
+ *     solid or moving-wall nodes (a Phi given to trtrlb_set_f) it is single steps;
  *   - G_CURRENT: periodic in both directions without a mask; an odd rest of a run
  *     is a single step.
- * The bits are those of single steps.  Host only. */
+ * The bits are those of single steps.  An even number of steps captured into a
+ * caller's graph can be replayed; such a lattice takes an even number of
+ * launches of two steps per run from then on.  Host only. */
 int trtrlb_two_step(trtrlb_t h, int32_t* on);
+
+/* Two steps per launch on (where the conditions above but the kernel variant
+ * hold) or off; trtrlb_set_kernel sets it back to on for TRTRLB_KERNEL_AUTO and
+ * off for the others.  Off gives the second buffer of a lattice with G lagged or
+ * off back, waiting for the device's queued work, unless a captured run names it;
+ * it is not allocated again. */
+int trtrlb_set_two_step(trtrlb_t h, int32_t on);
 
 /* ---- slab decomposition -----------------------------------------------------
  * One lattice split into nslabs sub-lattices of consecutive rows (y), the

@@ -39,7 +39,8 @@ struct trtrlb_lattice {
     double* dout;        // result of diagnostics (8 doubles) and comparisons (TRTRLB_CMP_N)
     std::atomic<int64_t> bytes;   // (another thread's reclaim_spares lowers it)
     int tile_w;          // scalar-kernel tile width in the batched path (32 .. 256 nodes)
-    int variant;         // TRTRLB_KERNEL_AUTO / SCALAR / VECTOR
+    int variant;         // TRTRLB_KERNEL_AUTO / SCALAR / VECTOR / COLUMN
+    bool two_step;       // two steps per launch where the lattice allows it (AUTO, or set_two_step)
     void* tmaps;         // two CUtensorMap (host) of the FP32 periodic G_CURRENT kernel, or null
     int* kerr;           // device flag set when a kernel's bounded wait ran out, or null
     int tma_grid;        // persistent grid of the TMA kernel on this device (0: none)

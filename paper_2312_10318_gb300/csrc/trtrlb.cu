@@ -91,40 +91,48 @@ void forget_spare(trtrlb_lattice* h) {
         }
 }
 
-// Whether another second buffer of `bytes` may be allocated: while they take up
-// no more than kSparesFree in all, or leave half of the device's memory free
-// (the query costs a small lattice's create a tenth).
-constexpr size_t kSparesFree = (size_t)4 << 30;
+// Whether another second buffer of `bytes` may be allocated: while they take up no
+// more than kSparesFree in all (the query of what is free costs a small lattice's
+// create a tenth), else at most a quarter of the device, of which half stays free.
+// Allocations outside the library do not make the buffers go back, so what they
+// may take from a program is bounded.
+constexpr size_t kSparesFree = (size_t)64 << 20;
 bool spare_fits(size_t bytes) {
+    size_t all;
     {
         std::lock_guard<std::mutex> lk(g_spares_mu);
-        if (g_spares_bytes + bytes <= kSparesFree) return true;
+        all = g_spares_bytes + bytes;
     }
+    if (all <= kSparesFree) return true;
     size_t free_b = 0, total_b = 0;
-    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && free_b > bytes && free_b - bytes >= total_b / 2;
+    return cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && all <= total_b / 4 && free_b > bytes &&
+           free_b - bytes >= total_b / 2;
 }
 
-// Gives back the second buffers that no captured launch names (cudaFree waits for
-// the queued ones); the lattices go on with single steps.
-// Called when an allocation fails, so that the buffers never cost a caller a
-// lattice that would have fit without them.
+// Gives the second buffer of h back unless a captured launch names it (cudaFree
+// waits for the queued ones); the lattice goes on with single steps.  Whether it
+// did (g_spares_mu and h->spare_mu held).
+bool give_back(trtrlb_lattice* h) {
+    if (h->captured || h->pins->pins > 0) return false;
+    if (h->s.f == h->f2) std::swap(h->f, h->f2);
+    cudaFree(h->f2);
+    h->bytes -= (int64_t)(elem_size(h->p.storage) * 9 * (size_t)h->s.plane);
+    h->f2 = nullptr;
+    h->s.f2 = nullptr;
+    h->s.pair = false;
+    forget_spare(h);
+    return true;
+}
+
+// Gives back all of them.  Called when an allocation fails, so that the buffers
+// never cost a caller a lattice that would have fit without them.
 void reclaim_spares() {
     std::lock_guard<std::mutex> lk(g_spares_mu);
     for (size_t i = 0; i < g_spares.size();) {
         trtrlb_lattice* h = g_spares[i];
         // (a thread that is queueing steps is waited for; none allocates meanwhile)
         std::lock_guard<std::mutex> hl(h->spare_mu);
-        if (h->captured || h->pins->pins > 0) {
-            ++i;
-            continue;
-        }
-        if (h->s.f == h->f2) std::swap(h->f, h->f2);
-        cudaFree(h->f2);
-        h->bytes -= (int64_t)(elem_size(h->p.storage) * 9 * (size_t)h->s.plane);
-        h->f2 = nullptr;
-        h->s.f2 = nullptr;
-        h->s.pair = false;
-        forget_spare(h);
+        if (!give_back(h)) ++i;
     }
 }
 
@@ -216,7 +224,7 @@ bool pair_applies(const trtrlb_params& p, const uint8_t* mask) {
 
 // (h->spare_mu held, or h not yet known to other threads)
 bool two_step_on(const trtrlb_lattice* h) {
-    if (h->variant != TRTRLB_KERNEL_AUTO || !h->f2 || h->phi_given) return false;
+    if (!h->two_step || !h->f2 || h->phi_given) return false;
     return h->p.g_mode != TRTRLB_G_CURRENT || (!h->s.general && elem_size(h->p.storage) <= 4 && h->p.nx >= 32);
 }
 
@@ -544,6 +552,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     h->tile_w = p.nx >= 128 ? 128 : (p.nx >= 64 ? 64 : 32);
     s.tile_w = h->tile_w;
     h->variant = TRTRLB_KERNEL_AUTO;
+    h->two_step = true;
     s.vec = auto_vector(h);
     s.sms = h->sms;
     s.pair = two_step_on(h);
@@ -899,6 +908,7 @@ int trtrlb_set_kernel(trtrlb_t h, int32_t variant, int32_t tile_w) {
     h->s.vec = vec;
     {
         std::lock_guard<std::mutex> lk(h->spare_mu);
+        h->two_step = variant == TRTRLB_KERNEL_AUTO;
         h->s.pair = two_step_on(h);
     }
     if (variant == TRTRLB_KERNEL_COLUMN) {
@@ -935,6 +945,17 @@ int trtrlb_two_step(trtrlb_t h, int32_t* on) {
     if (!h || !on) return TRTRLB_EINVAL;
     std::lock_guard<std::mutex> lk(h->spare_mu);
     *on = h->s.pair ? 1 : 0;
+    return TRTRLB_OK;
+}
+
+int trtrlb_set_two_step(trtrlb_t h, int32_t on) {
+    if (!h) return TRTRLB_EINVAL;
+    h->err[0] = 0;
+    std::lock_guard<std::mutex> lk(g_spares_mu);
+    std::lock_guard<std::mutex> hl(h->spare_mu);
+    h->two_step = on != 0;
+    if (!on && h->f2 && h->p.g_mode != TRTRLB_G_CURRENT) give_back(h);
+    h->s.pair = two_step_on(h);
     return TRTRLB_OK;
 }
 

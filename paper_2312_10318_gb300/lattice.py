@@ -183,6 +183,13 @@ class Lattice:
         self._chk(self._lib.trtrlb_two_step(self._h, C.byref(k)))
         return bool(k.value)
 
+    def set_two_step(self, on: bool):
+        """Two steps per launch where the lattice allows it, beside whatever kernel
+        set_kernel chose for single steps; off also gives the second population buffer
+        back (unless a captured run names it), for good.  set_kernel resets it."""
+        self._chk(self._lib.trtrlb_set_two_step(self._h, int(bool(on))))
+        return self
+
     def step_kernel(self) -> str:
         """The step kernel the current settings select: 'aa' | 'aa_vector' (fused
         AA stream-collide), 'ab' | 'ab_tma' | 'ab_tma_shared' | 'ab_column'
