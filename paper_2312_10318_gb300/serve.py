@@ -65,14 +65,22 @@ class Result:
 
 def lattice_bytes(n_x: int, n_y: int, storage: str) -> int:
     """Device bytes a lattice needs: populations (9 per node), two Phi buffers of two
-    components, the diagnostics scratch.  The two-step kernel's second population
-    buffer is not counted: the library allocates it only while half of the device
-    stays free (or such buffers take at most 4 GiB in all)."""
+    components, the diagnostics scratch; what it takes beyond is
+    second_buffer_bytes."""
     pitch = (n_x + 63) // 64 * 64
     plane = pitch * n_y
     phi = 8 if storage in ("f64", "f64dw") else 4
     blocks = max(1, min(1216, -(-n_x * n_y // 256)))
     return 9 * STORAGE_BYTES[storage] * plane + 4 * phi * plane + 8 * 8 * blocks + 8 * 16
+
+
+def second_buffer_bytes(lat, periodic) -> int:
+    """Device bytes of the two-step kernel's second population buffer (and its map of
+    a walled lattice) of a lattice just made, which it can do without."""
+    if not lat.two_step():
+        return 0
+    plane = (lat.nx + 63) // 64 * 64 * lat.ny
+    return (9 * STORAGE_BYTES[lat.storage] + (0 if all(periodic) else 4)) * plane
 
 
 def make_stream(n_requests: int, seed: int = 0, rate: float = 1.0, n_min: int = 64,
@@ -353,12 +361,15 @@ class _Active:
     nbytes: int
     storage: str
     fallback: bool = False
+    extra: int = 0            # bytes of the second population buffer
 
 
 class Server:
     """Continuous batching of lattice solves on the current CUDA device.
 
-    hbm_budget: bytes the admitted lattices may occupy.  chunk: the most steps
+    hbm_budget: bytes the admitted lattices may occupy; second population buffers
+    (two steps per launch) only take what is left of it, and go back when a waiting
+    request needs their room.  chunk: the most steps
     advanced between two scheduling points.  check_every: chunks between
     NaN/instability checks of every active lattice (0: only at retirement).
     guard: optional callable(request, lattice) -> lattice applied on admission
@@ -406,7 +417,9 @@ class Server:
         if guard is not None and hasattr(guard, "release"):
             guard.release = self._release
         self.active_nodes = 0
-        self.used = 0
+        self.used = 0                 # bytes the admitted lattices need
+        self.extra = 0                # bytes of their second population buffers
+        self._trim = False            # a request waits for these bytes
         self.node_updates = 0
         self.log = []
 
@@ -416,6 +429,9 @@ class Server:
         storage = self.fp64_as if req.storage == "f64" else req.storage
         nbytes = lattice_bytes(req.n, req.n, storage)
         if self.used + nbytes > self.budget:
+            return None
+        if self.used + self.extra + nbytes > self.budget:
+            self._trim = True          # the second buffers go at the next scheduling point
             return None
         # enough nodes in flight saturate HBM; admitting more only stretches
         # every solve (the first request is always admitted)
@@ -439,9 +455,14 @@ class Server:
                     act.nbytes = lattice_bytes(req.n, req.n, lat2.storage)
                     self._release(lat)
                     act.lat = lat2
+            act.extra = second_buffer_bytes(act.lat, pr.periodic)
+            if self.used + act.nbytes + self.extra + act.extra > self.budget:
+                act.lat.set_two_step(False)
+                act.extra = 0
             if self.tuner is not None:
                 self.tuner.apply(act.lat, pr.periodic)
         self.used += act.nbytes
+        self.extra += act.extra
         self.active_nodes += req.n * req.n
         return act
 
@@ -450,6 +471,7 @@ class Server:
             self.on_retire(a.req, a.lat, status)
         self._release(a.lat)
         self.used -= a.nbytes
+        self.extra -= a.extra
         self.active_nodes -= a.req.n * a.req.n
         return Result(a.req.rid, status, a.storage, a.req.steps - a.remaining, diag, a.req.arrival,
                       a.t_admit, now, a.fallback)
@@ -547,6 +569,14 @@ class Server:
                     a.lat.set_stream(self.stream)
                 active.extend(admitted)
             self._flush()          # nothing in flight: freeing waits for no kernel
+            if self._trim:
+                self.batch.set([])     # its captured runs name the buffers
+                members = None
+                for a in active:
+                    a.lat.set_two_step(False)
+                    self.extra -= a.extra
+                    a.extra = 0
+                self._trim = False
             if active:
                 lats = [a.lat for a in active]
                 if members is None or len(members) != len(lats) or any(x is not y for x, y in zip(members, lats)):
