@@ -109,18 +109,11 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double rmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double rfma(double a, double b, double c) { return __fma_rn(a, b, c); }
-// FP64 on this GPU: an instruction holds a quarter of an SM's pipe for 64 cycles, so
-// what can be done without one is.  The reciprocal is the 20-bit approximation and
-// one third-order (Halley) step, r (1 + e + e^2) with e = 1 - a r: three FMAs, error
-// below 2^-60 before the last rounding.
-__device__ __forceinline__ double rrcp(double a) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(a));
-    const double e = __fma_rn(-a, r, 1.0);
-    return __fma_rn(r, __fma_rn(e, e, e), r);
-}
+__device__ __forceinline__ double rrcp(double a) { return __drcp_rn(a); }
 // x 2^-K, exact: the exponent field in integer arithmetic (zero and values whose
-// exponent could leave the normal range take the multiplication).
+// exponent could leave the normal range take the multiplication).  An FP64
+// instruction holds a quarter of an SM's pipe for 64 cycles, so what can be done
+// exactly without one is.
 template <int K>
 __device__ __forceinline__ double rscale(double x) {
     const int hi = __double2hiint(x), lo = __double2loint(x);
