@@ -161,8 +161,10 @@ int trtrlb_get_f(trtrlb_t h, double* f, double* phi);
 
 /* Replaces the populations of the current state (9*nx*ny FP64 values, rounded
  * to the storage format).  phi == NULL: the previous-level Phi becomes that of
- * the new state; otherwise 2*nx*ny values are taken as given.  Values at
- * non-fluid nodes are ignored. */
+ * the new state; otherwise 2*nx*ny values are taken as given.  Populations at
+ * non-fluid nodes are ignored.  With a mask and phi in pageable host memory the
+ * call synchronises the stream (it looks whether the Phi of solid and moving-wall
+ * nodes is the one they have, see trtrlb_two_step). */
 int trtrlb_set_f(trtrlb_t h, const double* f, const double* phi);
 
 /* Number of steps taken since the last init / set_f. */

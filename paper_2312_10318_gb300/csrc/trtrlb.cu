@@ -75,6 +75,16 @@ bool on_device(const void* p) {
         }                                                                        \
     }()
 
+// Ordinary host memory: neither device, managed nor page-locked.
+bool pageable(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return a.type == cudaMemoryTypeUnregistered;
+}
+
 // Handles whose two-step kernel has a second population buffer.
 std::mutex g_spares_mu;
 std::vector<trtrlb_lattice*> g_spares;
@@ -773,8 +783,16 @@ int trtrlb_set_f(trtrlb_t h, const double* f, const double* phi) {
     if (e == cudaSuccess) e = TRT_DISPATCH(h->p.storage, set_f(h->s, df, dp, h->stream));
     if (e != cudaSuccess) return cuda_fail(h->err, e, "set_f");
     // a Phi given for solid and moving-wall nodes sits in one of the two buffers,
-    // which single steps read in turn and the two-step kernel does not
-    if (phi && h->mask) h->phi_given = true;
+    // which single steps read in turn and the two-step kernel does not; from pageable
+    // memory (whose copy waits anyway) look whether it is another than theirs, as it
+    // is not on a restore of what trtrlb_get_f gave
+    if (phi && h->mask) {
+        bool given = true, captured = false;
+        e = pageable(phi) ? trt::capturing(h->stream, &captured) : cudaSuccess;
+        if (e == cudaSuccess && pageable(phi) && !captured) e = phi_given_now(h, &given);
+        if (e != cudaSuccess) return cuda_fail(h->err, e, "set_f");
+        h->phi_given = given;
+    }
     h->t = 0;
     std::lock_guard<std::mutex> lk(h->spare_mu);
     h->s.pair = two_step_on(h);
