@@ -8,9 +8,11 @@ scalar kernel with 256-thread tiles of width 32, 64, 128 or 256 nodes, the
 vector kernel (V nodes per thread) where it applies and, for FP32 and 16-bit
 storage, the two-step kernel (variant 'auto'); with Phi at the current level (the
 two-buffer step) on a periodic lattice without a mask they are the plain kernel,
-the column-walking kernel and, for FP32, the TMA-fed one.
+the column-walking kernel and, for FP32, the two-step kernel (variant 'auto', odd
+steps TMA-fed); for the 16-bit formats the two-step kernel is timed beside the
+chosen single-step kernel and, where it is faster, put on with it.
 Results are cached in a JSON file keyed by the bucket, so a shape is measured
-once.  The kernel never changes results beyond rounding (FP64/FP32 are
+once per KERNELS.  The kernel never changes results beyond rounding (FP64/FP32 are
 bit-identical across kernels).
 """
 from __future__ import annotations
@@ -22,6 +24,9 @@ from typing import Optional
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "trtrlb_tune.json")
 TILE_WIDTHS = (32, 64, 128, 256)
+# Generation of the measured kernels: entries of a cache written with another one
+# are measured again (raise it when a candidate's kernel changes).
+KERNELS = 2
 VEC_WIDTH = {"f64": 2, "f64dw": 2, "f32": 4, "f16": 4, "bf16": 4}
 
 
@@ -73,7 +78,7 @@ class Tuner:
             out = [("scalar", 0)]
             if flavour(periodic, has_mask) == "periodic":
                 if storage == "f32":
-                    out.append(("auto", 0))        # TMA-fed
+                    out.append(("auto", 0))        # two steps per launch; single ones TMA-fed
                 if storage != "f64dw":
                     out.append(("column", 0))
             return out
@@ -84,10 +89,17 @@ class Tuner:
             out.append(("auto", 0))            # two steps per launch
         return out
 
+    @staticmethod
+    def two_step_beside(storage: str, periodic, has_mask: bool, g_mode="lagged") -> bool:
+        """Whether the two-step kernel is timed beside the candidates, none of which
+        has it: with Phi at the current level for the 16-bit formats."""
+        return g_mode == "current" and storage in ("f16", "bf16") and flavour(periodic, has_mask) == "periodic"
+
     def measure(self, storage: str, nx: int, ny: int, periodic=(True, True),
                 tau_s: float = 0.8, tau_s2: float = 1.0, g=(0.0, 0.0), stream=None,
                 g_mode: str = "lagged") -> dict:
-        """ms per step of every candidate on a scratch lattice (at rest, rho0)."""
+        """ms per step of every candidate on a scratch lattice (at rest, rho0), and of
+        the two-step kernel as 'two_step' where it is timed beside them."""
         import numpy as np
         import torch
         from .lattice import Batch, Lattice
@@ -99,7 +111,10 @@ class Tuner:
             lat.init(z, z)
         batch = Batch(stream).set([lat])
         times = {}
-        for variant, tw in self.candidates(storage, nx, periodic, False, g_mode):
+        runs = [(f"{v}:{tw}", v, tw) for v, tw in self.candidates(storage, nx, periodic, False, g_mode)]
+        if self.two_step_beside(storage, periodic, False, g_mode):
+            runs.append(("two_step", "auto", 0))
+        for name, variant, tw in runs:
             lat.set_kernel(variant, tw)
             batch.set([lat])
             batch.step(self.steps)          # capture + warm up
@@ -112,7 +127,7 @@ class Tuner:
                 e1.record(stream)
                 e1.synchronize()
                 best = min(best, e0.elapsed_time(e1) / self.steps)
-            times[f"{variant}:{tw}"] = best
+            times[name] = best
         batch.close()
         lat.close()
         return times
@@ -131,16 +146,19 @@ class Tuner:
         if len(cands) == 1:
             return cands[0]
         k = key(storage, nx, ny, periodic, has_mask, g_mode)
-        # measured already, and with every candidate there is now
-        known = self.table.get(k, {}).get("candidates", {})
-        if any(f"{v}:{tw}" not in known for v, tw in cands):
+        # measured already, with the kernels and every candidate there are now
+        known = self.table.get(k, {})
+        if known.get("kernels") != KERNELS or any(f"{v}:{tw}" not in known["candidates"] for v, tw in cands):
             bx, by = bucket(nx), bucket(ny)
             per = (True, True) if flavour(periodic, has_mask) == "periodic" else (True, False)
             times = self.measure(storage, bx, by, per, g_mode=g_mode, **kw)
+            two = times.pop("two_step", None)
             best = min(times, key=times.get)
             variant, tw = best.split(":")
             self.table[k] = {"variant": variant, "tile_w": int(tw), "ms_per_step": times[best],
-                             "candidates": times}
+                             "candidates": times, "kernels": KERNELS}
+            if two is not None:
+                self.table[k]["two_step_ms"] = two
             self.measured[k] = times
             self.save()
         e = self.table[k]
@@ -161,4 +179,8 @@ class Tuner:
             lat.set_kernel(variant, tw)
         except Exception:
             lat.set_kernel("scalar", tw)
+        if self.two_step_beside(lat.storage, periodic, has_mask, g_mode):
+            e = self.table[key(lat.storage, lat.nx, lat.ny, periodic, has_mask, g_mode)]
+            if e["two_step_ms"] < e["ms_per_step"]:
+                lat.set_two_step(True)
         return variant, tw
