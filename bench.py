@@ -199,15 +199,41 @@ BATCH_KERNEL_NAMES = {
                      "up to 16 lattices in one launch)",
 }
 TMA_GROUP_MAX = 16      # lattices per shared TMA-fed launch
+GROUP_MAX = 96          # lattices per launch of two steps
 # the kernel that runs of steps use where the library reports it (Lattice.two_step)
-TWO_STEP_NAME = "trt::k_step_pair (two fused stream-collide steps per launch{}; single steps at the ends of a run)"
+TWO_STEP_NAMES = {
+    "lagged": "trt::k_step_pair (two fused stream-collide steps per launch{}; single steps at the ends of a run)",
+    "off": "trt::k_step_pair (two fused stream-collide steps per launch{}; single steps at the ends of a run)",
+    "current": "trt::k_step_ab_pair (two two-buffer steps per launch, Phi at the current level{}; an odd step single)",
+}
+GRAPH_STEPS = 32        # steps of a batch's captured run
 
 
-def two_step_launches(steps: int, odd: bool) -> int:
-    """Launches of a run of `steps` steps of lattices that advance two steps at a
-    time from odd levels: a single step to an odd level, and one for an odd rest."""
-    first = 0 if odd or steps == 0 else 1
-    return first + (steps - first) // 2 + (steps - first) % 2
+def two_step_run(steps: int, odd: bool, g_mode: str, batch: bool):
+    """(launches of two steps, single steps) of a run of `steps` steps of lattices that
+    advance two steps at a time: with Phi at the current level from any level, else
+    from odd ones, after a single step.  A batch's captured run from an even level
+    (taken when the run is no longer than it) holds an even number of the former."""
+    first = 0 if odd or g_mode == "current" else min(1, steps)
+    pairs = (steps - first) // 2
+    if batch and first and steps == GRAPH_STEPS:
+        pairs -= pairs % 2
+    return pairs, steps - 2 * pairs
+
+
+def run_launches(mode: str, kinds, two: bool, steps: int, odd: bool, g_mode: str) -> int:
+    """Step-kernel launches of a run: those of single steps (step_launches each) and,
+    where the lattices take two steps at a time, one per GROUP_MAX lattices of a
+    batch (one per lattice outside a batch) for two steps."""
+    if not two:
+        return steps * step_launches(mode, kinds)
+    pairs, singles = two_step_run(steps, odd, g_mode, mode == "batch")
+    return pairs * pair_launches(mode, kinds) + singles * step_launches(mode, kinds)
+
+
+def pair_launches(mode: str, kinds) -> int:
+    """Launches that advance all lattices two steps (one flavour and parity)."""
+    return -(-len(list(kinds)) // GROUP_MAX) if mode == "batch" else len(list(kinds))
 
 
 def kernel_label(mode: str, kinds) -> str:
@@ -663,11 +689,12 @@ def main():
     # roofline of the step kernel: algorithmic bytes per launch / mean launch time
     kinds = [lat.step_kernel() for lat in lats]
     per_step_launches = step_launches(args.mode, kinds)
-    # lattices that advance two steps per launch share the launches as the single
-    # steps do, and a launch moves the bytes of one state for two steps
+    # a launch of two steps moves the bytes of one state
     two = all(lat.two_step() for lat in lats)
     per_launch = 2 if two else 1
-    launches = per_step_launches * (two_step_launches(args.steps, bool(level & 1)) if two else args.steps)
+    launches = run_launches(args.mode, kinds, two, args.steps, bool(level & 1), args.g_mode)
+    if two:
+        per_step_launches = pair_launches(args.mode, kinds)
     launch_s = local_ms / 1e3 / launches
     masked = any(p.mask is not None for p in problems)
     per_launch_bytes = bytes_per_node(storage, args.g_mode, masked) * nodes / per_step_launches
@@ -745,7 +772,8 @@ def main():
             "clocks": clk,
             "fp64_fma_tflops": fp64_tflops,
         }
-        line["roofline"]["kernel"] = (TWO_STEP_NAME.format(", all lattices in one launch" if args.mode == "batch" else "")
+        line["roofline"]["kernel"] = (TWO_STEP_NAMES[args.g_mode].format(
+                                          ", all lattices in one launch" if args.mode == "batch" else "")
                                       if two else kernel_label(args.mode, kinds))
         line["roofline"]["launch_ms"] = launch_s * 1e3
         line["roofline"]["hbm_gbs"] = achieved        # algorithmic bytes / time, every format
