@@ -549,8 +549,13 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
         }
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(h->f, 0, es * 9 * plane, h->stream);
-    // no step writes padding columns and solid nodes, and images hold them
-    if (e == cudaSuccess && h->f2) e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
+    // no step writes padding columns and the nodes of a mask that do not collide, and
+    // images hold them; the two-step kernel writes all others before it reads them
+    if (e == cudaSuccess && h->f2 && (mask || p.g_mode == TRTRLB_G_CURRENT))
+        e = cudaMemsetAsync(h->f2, 0, es * 9 * plane, h->stream);
+    else if (e == cudaSuccess && h->f2 && pitch > p.nx)
+        e = cudaMemset2DAsync(static_cast<char*>(h->f2) + es * p.nx, es * pitch, 0, es * (pitch - p.nx),
+                              (size_t)9 * p.ny, h->stream);
     if (e == cudaSuccess) e = TRT_DISPATCH(p.storage, phi_static(h->s, h->stream));
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
