@@ -268,8 +268,9 @@ int trtrlb_fp64_fma_rate(void* stream, double seconds, double* tflops);
  * below in registers; bands of 32, 16 or 8 rows (FP64: 16, 8 or 4), the
  * tallest that fills the device; ENOTSUP unless the lattice is periodic in
  * both directions, has no mask and stores FP64, FP32, FP16 or BF16).
- * tile_w: width in nodes of the scalar kernel's 256-thread tile (32, 64, 128
- * or 256; 0 keeps the current one). */
+ * tile_w: width in nodes of the scalar kernel's tile (32, 64, 128 or 256; 0 keeps
+ * the current one; a narrower lattice or a small launch takes a smaller tile).
+ * Whether runs of steps advance two at a time: trtrlb_two_step. */
 #define TRTRLB_KERNEL_AUTO 0
 #define TRTRLB_KERNEL_SCALAR 1
 #define TRTRLB_KERNEL_VECTOR 2
@@ -295,7 +296,8 @@ int trtrlb_load(trtrlb_t h, const void* image);
  * drains its copies in flight and returns, and the next trtrlb_moments /
  * trtrlb_get_f / trtrlb_diagnostics with host outputs reports TRTRLB_ETIMEOUT
  * (the state of that step is then undefined).  polls = 0 makes every such wait
- * give up at once, to exercise that path. */
+ * give up at once, to exercise that path.  Launches of two steps
+ * (trtrlb_two_step) wait for nothing. */
 int trtrlb_set_wait_limit(trtrlb_t h, int64_t polls);
 
 /* The kernel in use: *vector = 1 for the vector kernel; *tile_w as above.
@@ -367,9 +369,7 @@ int trtrlb_set_two_step(trtrlb_t h, int32_t on);
  * before, out after); around a two-buffer step (G_CURRENT), all nine
  * populations of the boundary rows before it (the halo's Phi is then taken at
  * the current level from them) and the populations pushed into the halo rows
- * after it.  Results equal the undivided lattice's bit for bit (G_CURRENT in
- * FP32 against its plain two-buffer kernel: the TMA-fed one contracts into FMAs
- * differently).  Masks with outlet ghosts (or halo nodes) give ENOTSUP; host or
+ * after it.  Results equal the undivided lattice's bit for bit.  Masks with outlet ghosts (or halo nodes) give ENOTSUP; host or
  * device pointers are accepted where fields are passed (global [ny][nx] /
  * [9][ny][nx] layouts); calls synchronise except step. */
 typedef struct trtrlb_slabs* trtrlb_slabs_t;
@@ -396,11 +396,11 @@ const char* trtrlb_slabs_last_error(trtrlb_slabs_t s);
  * per storage format covers every tile of every lattice in the batch (the
  * same per-node update as trtrlb_step, so results are those of stepping each
  * lattice alone).  G_CURRENT members take the two-buffer kernel: FP32 periodic
- * ones without a mask share its TMA-fed launches (up to 16 lattices each; the
- * results equal the single-lattice launch's up to the compiler's FMA
- * contraction, a few FP32 ulps), the others take one launch each.  Runs of 32
- * or more steps replay a captured CUDA graph when
- * the batch's stream is not the legacy default stream.  Lattices keep their
+ * ones without a mask share its TMA-fed launches (up to 16 lattices each), the
+ * others take one launch each.  Members that take two steps at a time
+ * (trtrlb_two_step) share one launch per format, flavour and G mode for two steps
+ * (up to 96 lattices each).  Runs of 32 or more steps replay a captured CUDA graph
+ * when the batch's stream is not the legacy default stream.  Lattices keep their
  * own parity and step count; all of them must live on the batch's device and
  * their other work must be ordered with the batch's stream by the caller
  * (simplest: create them on the same stream).  A lattice must stay alive while

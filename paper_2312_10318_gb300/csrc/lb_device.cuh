@@ -516,11 +516,9 @@ __device__ __forceinline__ void node_phi(const Args<C>& a, const C (&d)[9], C& p
 // segments, so their own code may spill a little: FP32 and 16-bit 6 CTAs (40
 // registers; 12-80 bytes of spills in the boundary code).  The double-word step
 // collides two nodes per thread (thread_step): 5 CTAs of 128 threads (96 to 102
-// registers).  us per step, one node per thread / two in CTAs of 256 x 2, 256 x 3,
-// 128 x 5, 128 x 6, 128 x 7: 4096^2 periodic 615 / 622, 569, 539, 536, 541; 1024^2
-// 44.0 / 45.0, 39.8, 36.7, 36.9, 37.4.  With one node per thread it asks for 4 of
-// 256 (64 registers, no spills with Phi lagged).  The other variants keep the
-// compiler's choice.
+// registers; us per step, one node per thread / two, 1024^2 44.0 / 36.7, 4096^2
+// 615 / 539).  With one node per thread it asks for 4 of 256 (64 registers, no
+// spills with Phi lagged).  The other variants keep the compiler's choice.
 template <int ROWS>
 __host__ __device__ constexpr int step_threads() { return ROWS == 2 ? 128 : 256; }
 template <typename S, bool GENERAL, int GMODE, int ROWS>

@@ -59,7 +59,8 @@ struct State {
     bool vec;             // the vectorised kernel runs this lattice
     int col_h;            // G_CURRENT: rows per band of the column-walking two-buffer
                           // kernel, which runs the step; 0: another kernel
-    int tile_w;           // scalar kernels: block of tile_w x (256 / tile_w) nodes
+    int tile_w;           // scalar kernels: widest tile (narrow lattices and small launches
+                          // take less: scalar_tile, scalar_threads)
     int g_mode;
     double tau1, tau2, gx, gy, rho0;
     double wall_ux, wall_uy, wall_rho;
@@ -78,8 +79,8 @@ template <typename S> struct Ops {
     // One time step (plus the outlet-ghost pass); flips parity and Phi buffers.
     static cudaError_t step(State& s, cudaStream_t st);
     // Two time steps of n lattices (State::pair, at an odd level, same flavour
-    // and G mode) in one launch per 64; the caller swaps f and f2, and with Phi
-    // lagged the Phi buffers.
+    // and G mode) in one launch per GROUP_MAX of them; the caller swaps f and f2,
+    // and with Phi lagged the Phi buffers.
     static cudaError_t step_pair(const State* const* members, int n, cudaStream_t st);
     // Fills a general lattice's maps of the two-step kernel.
     static cudaError_t pair_maps(const State& s, unsigned* info, unsigned* special, cudaStream_t st);

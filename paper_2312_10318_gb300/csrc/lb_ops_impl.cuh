@@ -49,12 +49,10 @@ static inline dim3 grid2d(const State& s, dim3 b) {
 }
 
 // Launches a step kernel (one that begins with chain_begin()) so that its set-up
-// overlaps the end of the previous kernel of the stream.  Dependent launches of
-// an empty kernel: 2.1 to 3.9 us apart without, 1.45 to 1.9 with (the host's
-// rate).  Us per step without / with: FP64 64^2 6.17 / 4.13, FP32 250 x 246 3.09 /
-// 2.22, 512^2 5.15 / 3.59, 1024^2 10.2 / 8.7, 4096^2 within noise.  Captured
-// launches keep full edges: a replay's dependent kernels start 0.6 to 0.8 us
-// apart, and 0.7 to 1.7 with programmatic ones.
+// overlaps the end of the previous kernel of the stream.  Us per step without /
+// with: FP64 64^2 6.2 / 4.1, FP32 250 x 246 3.1 / 2.2, 1024^2 10.2 / 8.7, 4096^2
+// within noise.  Captured launches keep full edges, which a replay runs faster
+// (240 channels, 256 steps: 5.1 ms, with programmatic edges 6.6).
 template <typename P, typename... A>
 static cudaError_t launch_chained(void (*kernel)(P, A...), dim3 g, dim3 b, cudaStream_t st, const P& p, A... rest) {
     cudaLaunchConfig_t c = {};
@@ -99,9 +97,8 @@ static inline int scalar_threads(const State* const* m, int n, int rows, int mos
 // Nodes per thread: the periodic double-word step takes two (thread_step).  With
 // walls and masks it takes one: a segment at them steps its nodes one after the
 // other, which all but the largest launches wait for at their end (us per step, one
-// / two: channel 64^2 6.2 / 6.8, 512^2 14.7 / 16.1, 1024^2 49.4 / 54.9, 2048^2 178 /
-// 169; periodic 64^2 4.2 / 3.5, 4096^2 615 / 539), and the kernels that hold both
-// forms took five minutes to compile.
+// / two: channel 1024^2 49.4 / 54.9, 2048^2 178 / 169; periodic 4096^2 615 / 539),
+// and the kernels that hold both forms took five minutes to compile.
 template <typename S, bool GENERAL>
 constexpr int rows_of_step() { return std::is_same<S, f64dw>::value && !GENERAL ? 2 : 1; }
 

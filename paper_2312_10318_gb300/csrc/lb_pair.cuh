@@ -26,19 +26,13 @@
 // The same arithmetic in the same order as two single steps, each population
 // rounded to the storage type between them: the same bits.
 //
-// Measured on GB300, one lattice, us per step, single steps (vector kernel) /
-// this kernel: FP32 4096^2 227.4 / 126.0 (133 GLUPS; the 44 B per node of a step
-// are 111 us at the copy bandwidth), 2048^2 62.7 / 33.4, 1024^2 15.4 / 10.2,
-// 512^2 7.3 / 5.2, 250 x 246 4.1 / 3.1; FP16 4096^2 147.0 / 105.2, 2048^2 42.1 /
-// 29.2, 1024^2 12.8 / 9.8, 512^2 6.2 / 4.7.  FP32 at 4096^2 is near its traffic;
-// the rest is bound by issue (FP16 77 % of the slots, 187 instructions per node
-// and step) and, below 1024^2, by the walk of the band.  4 resident CTAs of 4
-// warps (128 registers, no spills); 5 for the 16-bit formats (102 registers)
-// were slower (4096^2 108.8, 1024^2 11.3).  The collision in packed FP32 (f2)
-// instead of two scalar ones: FP32 1024^2 8.53 to 8.12, 512^2 3.49 to 3.25, FP16
-// 2048^2 28.2 to 27.4, channel 2048 x 1024 FP16 17.4 to 16.1 (chained launches).  With walls and masks, whole solves:
-// creeping flow 4096 x 2048 FP32, 50 steps, 7.3 ms in single steps, 4.4 here;
-// channel 2048 x 1024 FP16, 200 steps, 4.4 and 3.5.
+// Measured on GB300, us per step, single steps / this kernel: FP32 4096^2 227 /
+// 123, 1024^2 15.4 / 8.1; FP16 2048^2 42.1 / 27.4; whole solves, ms: creeping flow
+// 4096 x 2048 FP32, 50 steps, 7.5 / 4.3, channel 2048 x 1024 FP16, 200 steps, 4.9 /
+// 3.3.  FP32 at 4096^2 is near its traffic (44 B per node and step, 111 us at the
+// copy bandwidth); the rest waits for its own results at 16 warps per SM (4
+// resident CTAs of 4 warps, 125 of 128 registers, no spills).  The two collisions
+// of a lane run in packed FP32 (f2), half the issue slots of two scalar ones.
 #pragma once
 #include "lb_batch.cuh"
 #include "lb_device.cuh"
@@ -86,9 +80,9 @@ constexpr int PAIR_BLOCKS = 4, PAIR_AB_BLOCKS = 3, PAIR_AB_AHEAD = 3;
 // Rows per band for n lattices sharing a launch: the smallest number with which
 // every warp is resident at once, or, where that is more than PAIR_ROWS, in the
 // fewest whole waves of bands of at most PAIR_ROWS rows.  A band's walk is
-// sequential, so a partial wave costs a whole one: 4096^2 FP32 with 1.25, 1.5
-// and 2 waves of shorter bands 157, 149 and 128 us per step against 126.0 in
-// one; 250 x 246 with bands of 16, 8, 4 and 2 rows 7.15, 5.12, 4.11 and 3.09.
+// sequential, so a partial wave costs a whole one: 4096^2 FP32 in one wave 126 us
+// per step, in 1.25 waves of shorter bands 157; and a small lattice's launch is as
+// long as one walk: 250 x 246 with bands of 16 and 2 rows 7.2 and 3.1.
 inline int pair_band_rows(const State* const* m, int n, long long slots, int width) {
     auto warps = [&](int h) {
         long long w = 0;
@@ -112,9 +106,8 @@ inline int pair_band_rows(const State* const* m, int n, long long slots, int wid
 // (walls on the way in and out, elementwise loads), and in one wave the longest
 // walk is the launch's length: such a tile is walked by up to 8 warps of at least
 // 8 rows each.  They come first; where the tile is plain they leave at once.
-// Whole solves, ms, 1 / 2 / 8 parts at most: creeping flow 4096 x 2048 FP32 6.2 /
-// 5.4 / 4.4, channel 2048 x 1024 FP16 (bands of 16 rows) 4.2 / 3.5 / 3.5; parts of
-// 4 rows and more, channel 3.6.
+// Whole solves, ms, unsplit / split: creeping flow 4096 x 2048 FP32 6.2 / 4.4,
+// channel 2048 x 1024 FP16 (bands of 16 rows) 4.2 / 3.5.
 inline int pair_split(int band) { return band < 16 ? 1 : (band >= 64 ? 8 : band / 8); }
 
 template <int MAXL> struct PairParams {
