@@ -124,8 +124,11 @@ bool spare_fits(size_t bytes) {
 // did (g_spares_mu and h->spare_mu held).
 bool give_back(trtrlb_lattice* h) {
     if (h->captured || h->pins->pins > 0) return false;
-    if (h->s.f == h->f2) std::swap(h->f, h->f2);
-    cudaFree(h->f2);
+    if (cudaFree(h->s.f == h->f2 ? h->f : h->f2) != cudaSuccess) {   // (a capture in progress forbids it)
+        cudaGetLastError();
+        return false;
+    }
+    if (h->s.f == h->f2) h->f = h->f2;
     h->bytes -= (int64_t)(elem_size(h->p.storage) * 9 * (size_t)h->s.plane);
     h->f2 = nullptr;
     h->s.f2 = nullptr;
