@@ -690,7 +690,8 @@ def main():
     kinds = [lat.step_kernel() for lat in lats]
     per_step_launches = step_launches(args.mode, kinds)
     # a launch of two steps moves the bytes of one state
-    two = all(lat.two_step() for lat in lats)
+    two = batch.two_step_run(args.steps >= GRAPH_STEPS) if args.mode == "batch" else \
+        all(lat.two_step_run() for lat in lats)
     per_launch = 2 if two else 1
     launches = run_launches(args.mode, kinds, two, args.steps, bool(level & 1), args.g_mode)
     if two:

@@ -326,9 +326,8 @@ int trtrlb_get_kernel(trtrlb_t h, int32_t* vector, int32_t* tile_w);
 #define TRTRLB_STEP_AB_COLUMN 5
 int trtrlb_step_kernel(trtrlb_t h, int32_t* kind);
 
-/* Whether runs of steps advance this lattice two steps per launch (*on = 1):
- * FP32, FP16 or BF16 storage, nx >= 32, TRTRLB_KERNEL_AUTO (or
- * trtrlb_set_two_step) and
+/* Whether launches of two steps are available to this lattice (*on = 1): FP32, FP16
+ * or BF16 storage, nx >= 32, TRTRLB_KERNEL_AUTO (or trtrlb_set_two_step) and
  *   - G lagged or off: no node of the halo classes, no outlet ghost with a
  *     colliding node at x + 1 (any row of the three), and a second population
  *     buffer, which trtrlb_create allocates while such buffers take no more than
@@ -343,16 +342,26 @@ int trtrlb_step_kernel(trtrlb_t h, int32_t* kind);
  *     solid or moving-wall nodes (a Phi given to trtrlb_set_f) it is single steps;
  *   - G_CURRENT: periodic in both directions without a mask; an odd rest of a run
  *     is a single step.
- * The bits are those of single steps.  An even number of steps captured into a
- * caller's graph can be replayed; such a lattice takes an even number of
- * launches of two steps per run from then on.  Host only. */
+ * A run takes them where that is the faster way (trtrlb_two_step_run), or always
+ * after trtrlb_set_two_step(h, 1).  The bits are those of single steps.  An even
+ * number of steps captured into a caller's graph can be replayed; such a lattice
+ * takes an even number of launches of two steps per run from then on.  Host only. */
 int trtrlb_two_step(trtrlb_t h, int32_t* on);
 
-/* Two steps per launch on (where the conditions above but the kernel variant
- * hold) or off; trtrlb_set_kernel sets it back to on for TRTRLB_KERNEL_AUTO and
- * off for the others.  Off gives the second buffer of a lattice with G lagged or
- * off back, waiting for the device's queued work, unless a captured run names it;
- * it is not allocated again. */
+/* Whether a run of these count >= 1 lattices together, all of one format, boundary
+ * flavour (periodic or not) and G mode, takes two steps per launch (*on = 1): of one
+ * lattice by trtrlb_step, or of a batch's members; replayed: from a captured graph
+ * (a batch's runs of 32 steps or more, or a caller's).  A rule on the sizes: few
+ * nodes, and columns just past a multiple of 60 (56 with G_CURRENT), step faster
+ * singly.  EINVAL for a null handle or output.  Host only. */
+int trtrlb_two_step_run(const trtrlb_t* lattices, int32_t count, int32_t replayed, int32_t* on);
+
+/* Two steps per launch in every run (where the conditions above but the kernel
+ * variant hold), or in none; trtrlb_set_kernel sets it back: for
+ * TRTRLB_KERNEL_AUTO to where they are the faster way, for the others to none.
+ * Off gives the second buffer of a lattice with G lagged or off back, waiting for
+ * the device's queued work, unless a captured run names it; it is not allocated
+ * again. */
 int trtrlb_set_two_step(trtrlb_t h, int32_t on);
 
 /* ---- slab decomposition -----------------------------------------------------

@@ -59,6 +59,7 @@ SIGNATURES = {
     "trtrlb_get_kernel": (C.c_int, [_vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32)]),
     "trtrlb_two_step": (C.c_int, [_vp, C.POINTER(C.c_int32)]),
     "trtrlb_set_two_step": (C.c_int, [_vp, C.c_int32]),
+    "trtrlb_two_step_run": (C.c_int, [C.POINTER(_vp), C.c_int32, C.c_int32, C.POINTER(C.c_int32)]),
     "trtrlb_step_kernel": (C.c_int, [_vp, C.POINTER(C.c_int32)]),
     "trtrlb_set_wait_limit": (C.c_int, [_vp, _i64]),
     "trtrlb_state_bytes": (C.c_int64, [_vp]),

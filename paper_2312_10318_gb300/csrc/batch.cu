@@ -23,7 +23,7 @@ namespace {
 constexpr int kGraphSteps = 32;  // steps per captured graph (even: parity and Phi
                                  // buffers return to their start after a replay)
 constexpr size_t kMaxGraphs = 4;
-constexpr size_t kSideStreams = 5;
+constexpr size_t kSideStreams = trt::kBatchStreams - 1;
 
 }  // namespace
 
@@ -127,6 +127,29 @@ std::vector<Class> classes_of(const trtrlb_batch* b, const std::vector<trt::Stat
         c->nodes += (long long)s.nx * s.ny;
     }
     return out;
+}
+
+// Turns off the launches of two steps, in the states `sim` of a run, of members that
+// they would not pay for: decided over those of one format, flavour and G mode,
+// which share launches when their parities agree.
+void choose_two_steps(const trtrlb_batch* b, std::vector<trt::State>& sim, bool replayed) {
+    std::vector<bool> seen(sim.size(), false);
+    for (size_t i = 0; i < sim.size(); ++i) {
+        if (seen[i] || !sim[i].pair) continue;
+        std::vector<trtrlb_lattice*> m;
+        std::vector<size_t> at;
+        for (size_t k = i; k < sim.size(); ++k) {
+            const trt::State &x = sim[k], &y = sim[i];
+            if (!x.pair || b->lats[k]->p.storage != b->lats[i]->p.storage || x.g_mode != y.g_mode ||
+                x.general != y.general || x.vec != y.vec)
+                continue;
+            seen[k] = true;
+            m.push_back(b->lats[k]);
+            at.push_back(k);
+        }
+        if (trt::run_pays(m.data(), (int)m.size(), replayed)) continue;
+        for (size_t k : at) sim[k].pair = false;
+    }
 }
 
 // n steps of the members of class c from the states `sim`, which it advances.
@@ -330,8 +353,10 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
         closed = closed || h->captured;
         sim.push_back(h->s);
     }
+    const bool graphs = b->stream != nullptr && nsteps >= kGraphSteps;
+    choose_two_steps(b, sim, graphs || capturing);
     int64_t done = 0;
-    if (b->stream != nullptr && nsteps >= kGraphSteps) {
+    if (graphs) {
         // to odd levels, where the runs of two start, if that is a step for all
         bool odd_pair = false, even_pair = false;
         for (const trt::State& x : sim)
@@ -351,6 +376,7 @@ int trtrlb_batch_step(trtrlb_batch_t b, int64_t nsteps) {
     e = launch_steps(b, sim, nsteps - done, closed);
     if (e != cudaSuccess) return cuda_fail(b, e, "batch step");
     for (size_t i = 0; i < sim.size(); ++i) {
+        sim[i].pair = b->lats[i]->s.pair;
         b->lats[i]->s = sim[i];
         b->lats[i]->t += nsteps;
     }

@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "lb_ops.cuh"
+#include "lb_pair_rule.h"
 #include "trtrlb.h"
 
 // Who, beside the handle, names a lattice's second buffer: batches while a call or
@@ -20,6 +21,10 @@ struct SparePins {
     void pin() { ++refs, ++pins; }
     void unpin() { --pins, unref(); }
 };
+
+// never (a kernel of single steps was chosen), in runs in which it pays
+// (TRTRLB_KERNEL_AUTO: two_steps_pay), or always (trtrlb_set_two_step).
+enum class TwoStep : unsigned char { OFF, AUTO, ALWAYS };
 
 struct trtrlb_lattice {
     trtrlb_params p;
@@ -40,7 +45,7 @@ struct trtrlb_lattice {
     std::atomic<int64_t> bytes;   // (another thread's reclaim_spares lowers it)
     int tile_w;          // scalar-kernel tile width in the batched path (32 .. 256 nodes)
     int variant;         // TRTRLB_KERNEL_AUTO / SCALAR / VECTOR / COLUMN
-    bool two_step;       // two steps per launch where the lattice allows it (AUTO, or set_two_step)
+    TwoStep two_step;    // two steps per launch where the lattice allows it
     void* tmaps;         // two CUtensorMap (host) of the FP32 periodic G_CURRENT kernel, or null
     int* kerr;           // device flag set when a kernel's bounded wait ran out, or null
     int tma_grid;        // persistent grid of the TMA kernel on this device (0: none)
@@ -67,6 +72,27 @@ inline bool shares_tma_launch(const trtrlb_lattice* h) {
 }
 
 namespace trt {
+constexpr int kTmaShare = 16;     // lattices per shared TMA-fed launch
+constexpr int kBatchStreams = 6;  // a batch's own stream and those beside it
+
+// Adds lattice h, at state s, to the run r that it would share launches in (r of
+// n - 1 such lattices before: {} for n = 1).
+inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed) {
+    const State& s = h->s;
+    r.current = s.g_mode == TRTRLB_G_CURRENT;
+    r.off = s.g_mode == TRTRLB_G_OFF;
+    const int width = r.current ? PAIR_AB_W : PAIR_W, together = shares_tma_launch(h) ? kTmaShare : kBatchStreams;
+    r.nodes += (long long)s.nx * s.ny;
+    r.columns += (long long)pair_strips(s.nx, width) * width * s.ny;
+    r.tiled += (long long)(s.nx + 31) / 32 * 32 * s.ny;
+    r.elem = h->p.storage == TRTRLB_F32 ? 4 : 2;
+    r.general = s.general;
+    r.ghosts = r.ghosts || s.nghost > 0;
+    r.vec = s.vec;
+    r.depth = (n + together - 1) / together;
+    r.replayed = replayed;
+}
+
 // Whether st is being captured into a caller's graph.
 inline cudaError_t capturing(cudaStream_t st, bool* on) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -89,6 +115,10 @@ inline int64_t pair_launches(const State& s, int64_t n, bool even) {
     const int64_t k = n > first ? (n - first) / 2 : 0;
     return even ? k & ~(int64_t)1 : k;
 }
+
+// Whether a run of the n lattices h, all of one format, flavour and G mode and all
+// able to, takes two steps per launch.
+bool run_pays(trtrlb_lattice* const* h, int n, bool replayed);
 
 // Advances h by n time steps on st: two at a time from odd levels where the
 // two-step kernel runs the lattice.

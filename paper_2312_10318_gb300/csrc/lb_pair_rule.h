@@ -1,0 +1,48 @@
+// When a run takes two steps per launch (lb_pair.cuh): host code, sizes only.
+#pragma once
+
+namespace trt {
+
+// The lattices that would share the launches of a run.
+struct PairRun {
+    long long nodes;      // in all
+    long long columns;    // nodes that their strips store, lattice or not (strips x width x ny)
+    long long tiled;      // G_CURRENT: nodes that the 32-wide tiles of its single steps cover
+    int elem;             // bytes of a stored population, 4 or 2
+    bool current, off;    // Phi at the current level, no G; else lagged
+    bool general;         // walls, a mask or open edges
+    bool ghosts;          // outlet ghosts, whose single steps take a second launch per lattice
+    bool vec;             // the vector kernel would run the single steps
+    int depth;            // G_CURRENT: launches of a single step one after the other
+    bool replayed;        // launches from a captured graph, not by the host one by one
+};
+
+// Small launches of two steps last as long as one warp's walk: a band of two rows
+// takes four row collisions in a row, 3.7 us periodic and 8 us with walls (a step:
+// half), whatever the lattice's size.  Single steps of few nodes are faster than
+// that where the host does not bound their launches.  us per step, two steps per
+// launch / single, on GB300, replayed unless stated:
+//  - lagged or off, periodic: 64^2 1.9 / 2.6, 512^2 3.3 / 4.9 against the vector
+//    kernel; the scalar one, where nx is no multiple of the vector, is faster below
+//    about 130,000 nodes: 250 x 246 2.3 / 2.0, 250 x 512 2.8 / 2.7;
+//  - outlet ghosts: always faster, 64^2 5.2 / 9.0, 1024^2 19.7 / 21.3;
+//  - walls, lagged: 64^2 4.1 / 2.7, 512^2 5.6 / 5.3, 768^2 8.4 / 8.9; 16 lattices of
+//    64 x 1024, whose strips store 60 of their 64 columns and then 4, 19.9 / 14.9,
+//    of 100 x 1024 22.6 / 31.8: nodes weighted by the square of the share of the
+//    strips' columns that are in the lattice, from 400,000 on; without G 448^2
+//    3.8 / 4.1: from 160,000.  Below a share of 0.6 only out of L2: FP32 24 lattices
+//    of 32 x 4096 50 / 54, 16-bit 54 / 49, 90 of them 170 / 178;
+//  - Phi at the current level: launched one by one, single steps are bound by the
+//    host (64^2 3.7 / 6.1, 512^2 6.9 / 8.2); replayed, FP32 512^2 7.0 / 6.0, 640^2 8.4 /
+//    8.3, 16-bit 640^2 8.6 / 7.2, 768^2 9.3 / 10.9, and 40 lattices of 64^2, which take
+//    three launches one after the other, 7.1 / 11.4.
+inline bool two_steps_pay(const PairRun& r) {
+    if (r.current) return !r.replayed || r.depth >= 2 || r.tiled >= (r.elem == 4 ? 400000 : 500000);
+    if (!r.general) return r.vec || r.nodes >= 130000;
+    if (r.ghosts) return true;
+    const double share = (double)r.nodes / (double)r.columns;
+    const double least = share < 0.6 ? (r.elem == 4 ? 800e3 : 3e6) : (r.off ? 160e3 : 400e3);
+    return (double)r.nodes * share * share >= least;
+}
+
+}  // namespace trt

@@ -237,7 +237,7 @@ bool pair_applies(const trtrlb_params& p, const uint8_t* mask) {
 
 // (h->spare_mu held, or h not yet known to other threads)
 bool two_step_on(const trtrlb_lattice* h) {
-    if (!h->two_step || !h->f2 || h->phi_given) return false;
+    if (h->two_step == TwoStep::OFF || !h->f2 || h->phi_given) return false;
     return h->p.g_mode != TRTRLB_G_CURRENT || (!h->s.general && elem_size(h->p.storage) <= 4 && h->p.nx >= 32);
 }
 
@@ -570,7 +570,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
     h->tile_w = p.nx >= 128 ? 128 : (p.nx >= 64 ? 64 : 32);
     s.tile_w = h->tile_w;
     h->variant = TRTRLB_KERNEL_AUTO;
-    h->two_step = true;
+    h->two_step = TwoStep::AUTO;
     s.vec = auto_vector(h);
     s.sms = h->sms;
     s.pair = two_step_on(h);
@@ -934,7 +934,7 @@ int trtrlb_set_kernel(trtrlb_t h, int32_t variant, int32_t tile_w) {
     h->s.vec = vec;
     {
         std::lock_guard<std::mutex> lk(h->spare_mu);
-        h->two_step = variant == TRTRLB_KERNEL_AUTO;
+        h->two_step = variant == TRTRLB_KERNEL_AUTO ? TwoStep::AUTO : TwoStep::OFF;
         h->s.pair = two_step_on(h);
     }
     if (variant == TRTRLB_KERNEL_COLUMN) {
@@ -974,12 +974,25 @@ int trtrlb_two_step(trtrlb_t h, int32_t* on) {
     return TRTRLB_OK;
 }
 
+int trtrlb_two_step_run(const trtrlb_t* lattices, int32_t count, int32_t replayed, int32_t* on) {
+    if (!lattices || count < 1 || !on) return TRTRLB_EINVAL;
+    std::vector<trtrlb_lattice*> l(lattices, lattices + count);
+    bool all = true;
+    for (trtrlb_lattice* h : l) {
+        if (!h) return TRTRLB_EINVAL;
+        std::lock_guard<std::mutex> lk(h->spare_mu);
+        all = all && h->s.pair;
+    }
+    *on = all && trt::run_pays(l.data(), count, replayed != 0) ? 1 : 0;
+    return TRTRLB_OK;
+}
+
 int trtrlb_set_two_step(trtrlb_t h, int32_t on) {
     if (!h) return TRTRLB_EINVAL;
     h->err[0] = 0;
     std::lock_guard<std::mutex> lk(g_spares_mu);
     std::lock_guard<std::mutex> hl(h->spare_mu);
-    h->two_step = on != 0;
+    h->two_step = on ? TwoStep::ALWAYS : TwoStep::OFF;
     if (!on && h->f2 && h->p.g_mode != TRTRLB_G_CURRENT) give_back(h);
     h->s.pair = two_step_on(h);
     return TRTRLB_OK;
@@ -1023,13 +1036,24 @@ static T* at(T* const* a, int k) {
     return a ? a[k] : nullptr;
 }
 
+bool run_pays(trtrlb_lattice* const* h, int n, bool replayed) {
+    PairRun r{};
+    for (int k = 0; k < n; ++k) {
+        if (h[k]->two_step == TwoStep::ALWAYS) return true;
+        add_to_run(r, h[k], k + 1, replayed);
+    }
+    return two_steps_pay(r);
+}
+
 cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(h->spare_mu);
-    if (h->s.f2 && !h->captured) {
-        const cudaError_t e = capturing(st, &h->captured);
+    bool replayed = false;
+    if (h->s.f2) {
+        const cudaError_t e = capturing(st, &replayed);
         if (e != cudaSuccess) return e;
+        h->captured = h->captured || replayed;
     }
-    int64_t pairs = pair_launches(h->s, n, h->captured);
+    int64_t pairs = run_pays(&h, 1, replayed) ? pair_launches(h->s, n, h->captured) : 0;
     while (n > 0) {
         cudaError_t e;
         int k = 1;

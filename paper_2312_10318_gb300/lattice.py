@@ -48,6 +48,12 @@ def _as_f64(a, shape):
     return a
 
 
+def _two_step_run(lib, lattices, replayed: bool) -> bool:
+    arr, on = (C.c_void_p * max(1, len(lattices)))(*[l._h for l in lattices]), C.c_int32()
+    _lib.check(lib.trtrlb_two_step_run(arr, len(lattices), int(replayed), C.byref(on)))
+    return bool(on.value)
+
+
 class Lattice:
     """One lattice on the current CUDA device.
 
@@ -178,17 +184,24 @@ class Lattice:
         return bool(vec.value), tw.value
 
     def two_step(self) -> bool:
-        """Whether runs of steps advance two at a time (one launch for two steps)."""
+        """Whether launches of two steps are available to this lattice; runs take them
+        where that is the faster way (two_step_run), or always after
+        set_two_step(True)."""
         k = C.c_int32()
         self._chk(self._lib.trtrlb_two_step(self._h, C.byref(k)))
         return bool(k.value)
 
     def set_two_step(self, on: bool):
-        """Two steps per launch where the lattice allows it, beside whatever kernel
-        set_kernel chose for single steps; off also gives the second population buffer
-        back (unless a captured run names it), for good.  set_kernel resets it."""
+        """On: two steps per launch in every run, where the lattice allows it, beside
+        whatever kernel set_kernel chose for single steps.  Off: single steps; this
+        also gives the second population buffer back (unless a captured run names it),
+        for good.  set_kernel resets it."""
         self._chk(self._lib.trtrlb_set_two_step(self._h, int(bool(on))))
         return self
+
+    def two_step_run(self) -> bool:
+        """Whether step() takes two steps per launch (trtrlb_two_step_run)."""
+        return _two_step_run(self._lib, [self], False)
 
     def step_kernel(self) -> str:
         """The step kernel the current settings select: 'aa' | 'aa_vector' (fused
@@ -304,6 +317,12 @@ class Batch:
     def step(self, n: int = 1):
         self._chk(self._lib.trtrlb_batch_step(self._h, int(n)))
         return self
+
+    def two_step_run(self, replayed: bool = True) -> bool:
+        """Whether runs of the members, all of one format, flavour and G mode, take two
+        steps per launch: replayed ones (32 steps or more on a non-default stream), or
+        shorter ones."""
+        return _two_step_run(self._lib, self.members, replayed)
 
     def solve(self, fields, steps: int, out=None):
         """End-to-end solve of every member (trtrlb_batch_solve): member k starts

@@ -116,6 +116,8 @@ class Tuner:
             runs.append(("two_step", "auto", 0))
         for name, variant, tw in runs:
             lat.set_kernel(variant, tw)
+            if name == "two_step":
+                lat.set_two_step(True)
             batch.set([lat])
             batch.step(self.steps)          # capture + warm up
             best = float("inf")

@@ -49,7 +49,7 @@ def test_captured_even_runs_replay(gpu_lib, storage, g_mode, periodic, start):
     stream = torch.cuda.Stream()
     for n in (2, 4, 6, 8, 64):
         one = _lattice(70, 33, storage, g_mode, n, stream, periodic=periodic).set_kernel("scalar")
-        two = _lattice(70, 33, storage, g_mode, n, stream, periodic=periodic)
+        two = _lattice(70, 33, storage, g_mode, n, stream, periodic=periodic).set_two_step(True)
         assert two.two_step()
         one.step(start)
         two.step(start)
@@ -79,6 +79,8 @@ def test_captured_batches_replay(gpu_lib, n):
             lat = _lattice(nx, ny, st, g_mode, q, stream)
             if out is ones:
                 lat.set_kernel("scalar")
+            else:
+                lat.set_two_step(True)
             out.append(lat.step(q % 2))
     batch = Batch(stream).set(twos)
     g = _graph(batch.step, n, stream)

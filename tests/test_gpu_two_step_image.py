@@ -29,7 +29,7 @@ def test_images_of_equal_runs_are_equal(gpu_lib, storage, masked):
             lat.diagnostics()
         for lat in old[1::2]:                  # the others keep the blocks they share
             lat.close()
-        lat = Lattice(100, ny, 0.7, tau_s2=0.9, storage=storage, mask=mask).init(ux, uy, rho)
+        lat = Lattice(100, ny, 0.7, tau_s2=0.9, storage=storage, mask=mask).init(ux, uy, rho).set_two_step(True)
         assert lat.two_step()
         images.append(lat.step(3).save())      # one launch of two steps: the second buffer
         lat.close()

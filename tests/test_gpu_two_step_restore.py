@@ -16,7 +16,7 @@ def test_restored_masked_lattices_keep_two_steps(gpu_lib, storage, first):
     mask = W.random_mask(nx, ny, seed=5, solid_frac=0.05, inlet_outlet=True, outlet=W.OUTLET)
     rho, ux, uy = W.random_fields(nx, ny, seed=9, u_amp=0.05, rho_amp=0.01)
     make = lambda: Lattice(nx, ny, 0.72, tau_s2=1.15, periodic=(False, True), wall_u=(0.03, 0.0), storage=storage,
-                           mask=mask)
+                           mask=mask).set_two_step(True)
     run = make().init(ux, uy, rho).step(first)
     f, phi = run.get_f(with_phi=True)
     one, two = [make().set_f(f, phi) for _ in range(2)]

@@ -11,7 +11,7 @@ def _masked(storage="f32", nx=70, ny=24):
     from paper_2312_10318_gb300 import Lattice
     solid = np.zeros((ny, nx), np.uint8)
     solid[8:12, 20:24] = W.SOLID
-    return Lattice(nx, ny, 0.72, tau_s2=1.15, storage=storage, mask=solid), solid
+    return Lattice(nx, ny, 0.72, tau_s2=1.15, storage=storage, mask=solid).set_two_step(True), solid
 
 
 @pytest.mark.parametrize("storage", ["f32", "f16"])
