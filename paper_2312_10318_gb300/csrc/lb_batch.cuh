@@ -41,8 +41,8 @@ __device__ __forceinline__ void tile_divmod(int t, int d, float inv, int& q, int
     }
 }
 
-template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS, int MAXL>
-__global__ void __launch_bounds__(step_threads<ROWS>(), step_min_blocks<S, GENERAL, GMODE, ROWS>())
+template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS, bool FEW, int MAXL>
+__global__ void __launch_bounds__(step_threads<ROWS>(), step_min_blocks<S, GENERAL, GMODE, ROWS, FEW>())
     k_step_group(const __grid_constant__ GroupParams<typename Fmt<S>::C, MAXL> p) {
     chain_begin();
     const int b = (int)blockIdx.x;

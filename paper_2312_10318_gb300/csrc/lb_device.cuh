@@ -521,9 +521,16 @@ __device__ __forceinline__ void node_phi(const Args<C>& a, const C (&d)[9], C& p
 // spills with Phi lagged).  The other variants keep the compiler's choice.
 template <int ROWS>
 __host__ __device__ constexpr int step_threads() { return ROWS == 2 ? 128 : 256; }
-template <typename S, bool GENERAL, int GMODE, int ROWS>
+// FEW: launches whose CTAs are all resident at 4 per SM, to which the tighter
+// bound only brings its spills: FP32 with walls, 64 registers and none (us per
+// step, replayed, 6 CTAs / 4: 64^2 2.63 / 2.37, 384^2 3.80 / 3.60; 8 lattices of 256^2, 13
+// CTAs per SM, 8.55 / 8.89).
+template <typename S, bool GENERAL>
+constexpr bool few_variant() { return std::is_same<S, float>::value && GENERAL; }
+template <typename S, bool GENERAL, int GMODE, int ROWS, bool FEW>
 __host__ __device__ constexpr int step_min_blocks() {
-    return (sizeof(S) == 4 && !GENERAL && GMODE == G_LAGGED) ? 6
+    return FEW                                             ? 4
+           : (sizeof(S) == 4 && !GENERAL && GMODE == G_LAGGED) ? 6
            : (sizeof(S) <= 4 && GENERAL)                          ? 6
            : std::is_same<S, f64dw>::value                        ? (ROWS == 2 ? 5 : 4)
                                                                    : 1;
@@ -769,8 +776,8 @@ __device__ __forceinline__ void thread_step(const Args<typename Fmt<S>::C>& a, i
     }
 }
 
-template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS>
-__global__ void __launch_bounds__(step_threads<ROWS>(), step_min_blocks<S, GENERAL, GMODE, ROWS>())
+template <typename S, bool ODD, bool GENERAL, int GMODE, int ROWS, bool FEW>
+__global__ void __launch_bounds__(step_threads<ROWS>(), step_min_blocks<S, GENERAL, GMODE, ROWS, FEW>())
     k_step(Args<typename Fmt<S>::C> a) {
     chain_begin();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;

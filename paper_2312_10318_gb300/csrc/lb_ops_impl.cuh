@@ -94,6 +94,10 @@ static inline int scalar_threads(const State* const* m, int n, int rows, int mos
     return t;
 }
 
+// Whether a launch's CTAs are all resident at 4 of 256 threads per SM
+// (step_min_blocks).
+static inline bool few_ctas(long long ctas, int threads, int sms) { return ctas * threads <= 4ll * 256 * sms; }
+
 // Nodes per thread: the periodic double-word step takes two (thread_step).  With
 // walls and masks it takes one: a segment at them steps its nodes one after the
 // other, which all but the largest launches wait for at their end (us per step, one
@@ -108,8 +112,15 @@ static void launch_scalar(const State& s, const Args<typename Fmt<S>::C>& a, cud
     const State* one = &s;
     const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>()), tw = scalar_tile(s, t);
     const dim3 b(tw, t / tw), g = grid2d(s, dim3(tw, t / tw * ROWS));
-    if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, GENERAL, G_OFF, ROWS>, g, b, st, a);
-    else launch_chained(k_step<S, ODD, GENERAL, G_LAGGED, ROWS>, g, b, st, a);
+    if constexpr (few_variant<S, GENERAL>()) {
+        if (few_ctas((long long)g.x * g.y, t, s.sms)) {
+            if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, GENERAL, G_OFF, ROWS, true>, g, b, st, a);
+            else launch_chained(k_step<S, ODD, GENERAL, G_LAGGED, ROWS, true>, g, b, st, a);
+            return;
+        }
+    }
+    if (s.g_mode == G_OFF) launch_chained(k_step<S, ODD, GENERAL, G_OFF, ROWS, false>, g, b, st, a);
+    else launch_chained(k_step<S, ODD, GENERAL, G_LAGGED, ROWS, false>, g, b, st, a);
 }
 
 template <typename S, bool ODD>
@@ -404,8 +415,13 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     p.tile_begin[n] = tiles;
     if (FLAV == FLAV_VECTOR)
         return launch_chained(k_step_group_vec<S, ODD, GMODE, MAXL>, tiles, BATCH_THREADS, st, p);
-    else
-        return launch_chained(k_step_group<S, ODD, FLAV == FLAV_GENERAL, GMODE, ROWS, MAXL>, tiles, threads, st, p);
+    else {
+        constexpr bool GENERAL = FLAV == FLAV_GENERAL;
+        if constexpr (few_variant<S, GENERAL>())
+            if (few_ctas(tiles, threads, m[0]->sms))
+                return launch_chained(k_step_group<S, ODD, GENERAL, GMODE, ROWS, true, MAXL>, tiles, threads, st, p);
+        return launch_chained(k_step_group<S, ODD, GENERAL, GMODE, ROWS, false, MAXL>, tiles, threads, st, p);
+    }
 }
 
 template <typename S, bool ODD, int FLAV, int GMODE>
