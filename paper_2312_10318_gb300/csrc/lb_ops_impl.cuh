@@ -98,7 +98,8 @@ static inline int scalar_threads(const State* const* m, int n, int rows, int mos
 // (step_min_blocks).
 static inline bool few_ctas(long long ctas, int threads, int sms) { return ctas * threads <= 4ll * 256 * sms; }
 
-// Nodes per thread: the periodic double-word step takes two (thread_step).  With
+// Nodes per thread: the periodic double-word step takes two (thread_step), unless a
+// launch has too few nodes to fill the SMs with them (two_rows).  With
 // walls and masks it takes one: a segment at them steps its nodes one after the
 // other, which all but the largest launches wait for at their end (us per step, one
 // / two: channel 1024^2 49.4 / 54.9, 2048^2 178 / 169; periodic 4096^2 615 / 539),
@@ -106,10 +107,21 @@ static inline bool few_ctas(long long ctas, int threads, int sms) { return ctas 
 template <typename S, bool GENERAL>
 constexpr int rows_of_step() { return std::is_same<S, f64dw>::value && !GENERAL ? 2 : 1; }
 
-template <typename S, bool ODD, bool GENERAL>
+// Whether a launch of the periodic double-word step takes two nodes per thread: from
+// 512 nodes per SM on, 8 warps of two.  Below, a launch is as long as one thread's
+// work (us per step, replayed, one / two: 64^2 3.0 / 3.7, 256^2 4.0 / 4.3, 320^2 6.7 /
+// 6.7, 512^2 10.9 / 10.4, 16 lattices of 64^2 4.2 / 4.4, 8 of 128^2 6.9 / 6.8).
+static inline bool two_rows(const State* const* m, int n) {
+    long long nodes = 0;
+    for (int q = 0; q < n; ++q) nodes += (long long)m[q]->nx * m[q]->ny;
+    return nodes > 512ll * m[0]->sms;
+}
+
+template <typename S, bool ODD, bool GENERAL, int ROWS>
 static void launch_scalar(const State& s, const Args<typename Fmt<S>::C>& a, cudaStream_t st) {
-    constexpr int ROWS = rows_of_step<S, GENERAL>();
     const State* one = &s;
+    if constexpr (ROWS == 2)
+        if (!two_rows(&one, 1)) return launch_scalar<S, ODD, GENERAL, 1>(s, a, st);
     const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>()), tw = scalar_tile(s, t);
     const dim3 b(tw, t / tw), g = grid2d(s, dim3(tw, t / tw * ROWS));
     if constexpr (few_variant<S, GENERAL>()) {
@@ -125,8 +137,8 @@ static void launch_scalar(const State& s, const Args<typename Fmt<S>::C>& a, cud
 
 template <typename S, bool ODD>
 static void launch_step(const State& s, const Args<typename Fmt<S>::C>& a, cudaStream_t st) {
-    if (s.general) launch_scalar<S, ODD, true>(s, a, st);
-    else launch_scalar<S, ODD, false>(s, a, st);
+    if (s.general) launch_scalar<S, ODD, true, rows_of_step<S, true>()>(s, a, st);
+    else launch_scalar<S, ODD, false, rows_of_step<S, false>()>(s, a, st);
 }
 
 template <typename S, bool ODD>
@@ -381,14 +393,15 @@ cudaError_t Ops<S>::diagnostics(const State& s, double* part, double* out, cudaS
 }
 
 // FLAV: FLAV_GENERAL, FLAV_PERIODIC (scalar kernels) or FLAV_VECTOR.
-template <typename S, bool ODD, int FLAV, int GMODE, int MAXL>
+template <typename S, bool ODD, int FLAV, int GMODE, int ROWS, int MAXL>
 static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
+    if constexpr (ROWS == 2 && FLAV == FLAV_PERIODIC)
+        if (!two_rows(m, n)) return launch_group<S, ODD, FLAV, GMODE, 1, MAXL>(m, n, st);
     using C = typename Fmt<S>::C;
     constexpr int V = Pk<S>::V;
     GroupParams<C, MAXL> p;
     p.n = n;
     int tiles = 0;
-    constexpr int ROWS = rows_of_step<S, FLAV == FLAV_GENERAL>();
     const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, ROWS, step_threads<ROWS>());
     p.log2_threads = 0;
     while ((1 << p.log2_threads) < threads) ++p.log2_threads;
@@ -426,15 +439,16 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
 
 template <typename S, bool ODD, int FLAV, int GMODE>
 static cudaError_t launch_group_sized(const State* const* m, int n, cudaStream_t st) {
+    constexpr int ROWS = rows_of_step<S, FLAV == FLAV_GENERAL>();
     for (int q0 = 0; q0 < n; q0 += GROUP_MAX) {
         const int c = n - q0 < GROUP_MAX ? n - q0 : GROUP_MAX;
         cudaError_t e;
         // the double-word kernels, the longest to compile and to run, have one size
         if constexpr (std::is_same<S, f64dw>::value)
-            e = launch_group<S, ODD, FLAV, GMODE, GROUP_MAX>(m + q0, c, st);
+            e = launch_group<S, ODD, FLAV, GMODE, ROWS, GROUP_MAX>(m + q0, c, st);
         else
-            e = c <= 4 ? launch_group<S, ODD, FLAV, GMODE, 4>(m + q0, c, st)
-                       : launch_group<S, ODD, FLAV, GMODE, GROUP_MAX>(m + q0, c, st);
+            e = c <= 4 ? launch_group<S, ODD, FLAV, GMODE, ROWS, 4>(m + q0, c, st)
+                       : launch_group<S, ODD, FLAV, GMODE, ROWS, GROUP_MAX>(m + q0, c, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

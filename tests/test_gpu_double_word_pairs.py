@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("g_mode", ["lagged", "off"])
-@pytest.mark.parametrize("nx,ny", [(1, 2), (5, 3), (64, 1), (40, 3), (130, 33), (300, 131), (900, 901)])
+@pytest.mark.parametrize("nx,ny", [(1, 80001), (5, 16001), (90000, 1), (33, 2500), (130, 1033), (300, 331), (900, 901),
+                                   (64, 1), (40, 3), (130, 33)])       # the last three: one node per thread too
 def test_two_nodes_per_thread_give_the_bits_of_one(gpu_lib, nx, ny, g_mode):
     from paper_2312_10318_gb300 import Lattice
     rho, ux, uy = W.random_fields(nx, ny, seed=nx, u_amp=0.05, rho_amp=0.01)
