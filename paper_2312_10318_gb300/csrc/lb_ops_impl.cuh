@@ -76,17 +76,28 @@ static cudaError_t launch_chained(void (*kernel)(P, A...), dim3 g, dim3 b, cudaS
 // lanes (8-wide channels ran on a quarter of theirs, and FP64's pipe is busy for
 // all 32).  A launch that would leave SMs without a CTA halves its CTAs, down to
 // a warp: FP64 64^2 in 16 CTAs used 16 SMs' FP64 pipes.
-static inline int scalar_tile(const State& s, int threads) {
+// least: the narrowest tile.  With walls a warp of several rows runs the code of
+// plain rows and that of rows at walls one after the other, so as long as every
+// warp of one row has an SM quarter to itself, where idle lanes cost nothing, they
+// stay that wide (us per step, replayed, tiles of 8 / 32: one channel of 8 x 256
+// double-word 6.0 / 4.2, BF16 3.3 / 2.7, FP64 9.1 / 5.9; 16 of them 6.3 / 8.1, 4.0 / 4.0,
+// 13.3 / 30.2).
+static inline int least_tile(const State* const* m, int n) {
+    long long warps = 0;
+    for (int q = 0; q < n; ++q) warps += (long long)((m[q]->nx + 31) / 32) * m[q]->ny;
+    return m[0]->general && warps <= 4ll * m[0]->sms ? 32 : 1;
+}
+static inline int scalar_tile(const State& s, int threads, int least) {
     int tw = s.tile_w > 0 ? s.tile_w : 128;
-    while (tw > threads || (tw > 1 && tw / 2 >= s.nx)) tw /= 2;
+    while (tw > threads || (tw > least && tw / 2 >= s.nx)) tw /= 2;
     return tw;
 }
-static inline int scalar_threads(const State* const* m, int n, int rows, int most) {
+static inline int scalar_threads(const State* const* m, int n, int rows, int most, int least) {
     int t = most;
     for (; t > 32; t /= 2) {
         long long tiles = 0;
         for (int q = 0; q < n; ++q) {
-            const int tw = scalar_tile(*m[q], t), th = t / tw * rows;
+            const int tw = scalar_tile(*m[q], t, least), th = t / tw * rows;
             tiles += (long long)((m[q]->nx + tw - 1) / tw) * ((m[q]->ny + th - 1) / th);
         }
         if (tiles >= 2 * m[0]->sms) break;
@@ -122,7 +133,8 @@ static void launch_scalar(const State& s, const Args<typename Fmt<S>::C>& a, cud
     const State* one = &s;
     if constexpr (ROWS == 2)
         if (!two_rows(&one, 1)) return launch_scalar<S, ODD, GENERAL, 1>(s, a, st);
-    const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>()), tw = scalar_tile(s, t);
+    const int least = least_tile(&one, 1);
+    const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>(), least), tw = scalar_tile(s, t, least);
     const dim3 b(tw, t / tw), g = grid2d(s, dim3(tw, t / tw * ROWS));
     if constexpr (few_variant<S, GENERAL>()) {
         if (few_ctas((long long)g.x * g.y, t, s.sms)) {
@@ -402,7 +414,8 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     GroupParams<C, MAXL> p;
     p.n = n;
     int tiles = 0;
-    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, ROWS, step_threads<ROWS>());
+    const int least = least_tile(m, n);
+    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, ROWS, step_threads<ROWS>(), least);
     p.log2_threads = 0;
     while ((1 << p.log2_threads) < threads) ++p.log2_threads;
     for (int q = 0; q < n; ++q) {
@@ -416,7 +429,7 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
             p.log2_tw[q] = 0;
             tiles += (int)(((long long)p.segs[q] * v.ny + 7) / 8);
         } else {
-            const int tw = scalar_tile(v, threads), th = threads / tw * ROWS;
+            const int tw = scalar_tile(v, threads, least), th = threads / tw * ROWS;
             p.log2_tw[q] = 0;
             while ((1 << p.log2_tw[q]) < tw) ++p.log2_tw[q];
             p.segs[q] = 0;
