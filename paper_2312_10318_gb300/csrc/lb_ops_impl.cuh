@@ -92,9 +92,18 @@ static inline int scalar_tile(const State& s, int threads, int least) {
     while (tw > threads || (tw > least && tw / 2 >= s.nx)) tw /= 2;
     return tw;
 }
-static inline int scalar_threads(const State* const* m, int n, int rows, int most, int least) {
+// With a mask only FP64 halves them: a node's accesses depend on its neighbours'
+// classes, which a CTA of several rows finds in its SM's L1 (us per step, replayed,
+// CTAs of 256 / down to a warp: 128^2 with an obstacle FP32 3.4 / 4.0, double-word
+// 4.6 / 5.6, FP64, whose pipe counts, 9.4 / 7.4).
+static inline bool halves_ctas(const State* const* m, int n, bool fp64) {
+    bool masks = false;
+    for (int q = 0; q < n; ++q) masks = masks || m[q]->mask != nullptr;
+    return fp64 || !masks;
+}
+static inline int scalar_threads(const State* const* m, int n, int rows, int most, int least, bool fp64) {
     int t = most;
-    for (; t > 32; t /= 2) {
+    for (const int floor = halves_ctas(m, n, fp64) ? 32 : most; t > floor; t /= 2) {
         long long tiles = 0;
         for (int q = 0; q < n; ++q) {
             const int tw = scalar_tile(*m[q], t, least), th = t / tw * rows;
@@ -134,7 +143,8 @@ static void launch_scalar(const State& s, const Args<typename Fmt<S>::C>& a, cud
     if constexpr (ROWS == 2)
         if (!two_rows(&one, 1)) return launch_scalar<S, ODD, GENERAL, 1>(s, a, st);
     const int least = least_tile(&one, 1);
-    const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>(), least), tw = scalar_tile(s, t, least);
+    const int t = scalar_threads(&one, 1, ROWS, step_threads<ROWS>(), least, std::is_same<S, double>::value),
+              tw = scalar_tile(s, t, least);
     const dim3 b(tw, t / tw), g = grid2d(s, dim3(tw, t / tw * ROWS));
     if constexpr (few_variant<S, GENERAL>()) {
         if (few_ctas((long long)g.x * g.y, t, s.sms)) {
@@ -415,7 +425,9 @@ static cudaError_t launch_group(const State* const* m, int n, cudaStream_t st) {
     p.n = n;
     int tiles = 0;
     const int least = least_tile(m, n);
-    const int threads = FLAV == FLAV_VECTOR ? BATCH_THREADS : scalar_threads(m, n, ROWS, step_threads<ROWS>(), least);
+    const int threads = FLAV == FLAV_VECTOR
+                            ? BATCH_THREADS
+                            : scalar_threads(m, n, ROWS, step_threads<ROWS>(), least, std::is_same<S, double>::value);
     p.log2_threads = 0;
     while ((1 << p.log2_threads) < threads) ++p.log2_threads;
     for (int q = 0; q < n; ++q) {
