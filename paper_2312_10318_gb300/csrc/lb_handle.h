@@ -88,6 +88,9 @@ inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed
     r.elem = h->p.storage == TRTRLB_F32 ? 4 : 2;
     r.general = s.general;
     r.ghosts = r.ghosts || s.nghost > 0;
+    r.crowded = (n == 1 || r.crowded) && s.crowded;
+    r.mask = r.mask || s.mask != nullptr;
+    r.padded += s.plane;
     r.vec = s.vec;
     r.depth = (n + together - 1) / together;
     r.replayed = replayed;

@@ -44,6 +44,7 @@ struct State {
     const unsigned* pinfo;     // its maps of a general lattice (lb_pair.cuh): a word per node,
     const unsigned* pspecial;  // [ny][pitch], and a bit per strip and row, [strips][(ny + 31) / 32]
     int sms;              // multiprocessors of the device
+    bool crowded;         // general: at least half of the row segments (seg) are not interior
     void* phi[2];         // Phi buffers, C[2][ny][pitch]
     int cur;              // phi[cur] holds the previous level
     const uint8_t* mask;  // device [ny][pitch] or nullptr

@@ -12,6 +12,8 @@ struct PairRun {
     bool current, off;    // Phi at the current level, no G; else lagged
     bool general;         // walls, a mask or open edges
     bool ghosts;          // outlet ghosts, whose single steps take a second launch per lattice
+    bool mask, crowded;   // a mask; at least half of the row segments near its walls
+    long long padded;     // nodes with the rows' padding
     bool vec;             // the vector kernel would run the single steps
     int depth;            // G_CURRENT: launches of a single step one after the other
     bool replayed;        // launches from a captured graph, not by the host one by one
@@ -32,6 +34,11 @@ struct PairRun {
 //    strips' columns that are in the lattice, from 400,000 on; without G 448^2
 //    3.8 / 4.1: from 160,000.  Below a share of 0.6 only out of L2: FP32 24 lattices
 //    of 32 x 4096 50 / 54, 16-bit 54 / 49, 90 of them 170 / 178;
+//  - masks without ghosts: a few walls make whole strips slow that single steps take in
+//    their stride, so only out of L2: 1024^2 with a block 14.5 / 12.7, 1280^2 20.7 / 19.9,
+//    1536^2 22.1 / 37.1 (without G 512^2 4.8 / 5.1); where walls are everywhere single
+//    steps are slow too, and the line is that of open walls: 5 % of solid nodes, 768^2
+//    12.8 / 14.7, 40 lattices of 128^2 18.3 / 16.5;
 //  - Phi at the current level: launched one by one, single steps are bound by the
 //    host (64^2 3.7 / 6.1, 512^2 6.9 / 8.2); replayed, FP32 512^2 7.0 / 6.0, 640^2 8.4 /
 //    8.3, 16-bit 640^2 8.6 / 7.2, 768^2 9.3 / 10.9, and 40 lattices of 64^2, which take
@@ -40,8 +47,9 @@ inline bool two_steps_pay(const PairRun& r) {
     if (r.current) return !r.replayed || r.depth >= 2 || r.tiled >= (r.elem == 4 ? 400000 : 500000);
     if (!r.general) return r.vec || r.nodes >= 130000;
     if (r.ghosts) return true;
+    if (r.mask && !r.crowded && !r.off) return r.padded >= 1900000;
     const double share = (double)r.nodes / (double)r.columns;
-    const double least = share < 0.6 ? (r.elem == 4 ? 800e3 : 3e6) : (r.off ? 160e3 : 400e3);
+    const double least = share < 0.6 ? (r.elem == 4 ? 800e3 : 3e6) : (r.off && !r.mask ? 160e3 : 400e3);
     return (double)r.nodes * share * share >= least;
 }
 

@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -531,6 +532,7 @@ int trtrlb_create(const trtrlb_params* pp, const uint8_t* mask, void* stream, tr
             release(h);
             return rc;
         }
+        s.crowded = 2 * std::count(seg.begin(), seg.end(), (uint8_t)1) <= (long long)seg.size();
         s.seg = h->seg;
         s.segs = (p.nx + 31) / 32;
     }

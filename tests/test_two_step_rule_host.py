@@ -20,6 +20,8 @@ int main(int, char** v) {
     r.tiled = n * ((nx + 31) / 32 * 32) * ny;
     r.elem = atoi(v[5]); r.general = atoi(v[6]); r.ghosts = atoi(v[7]); r.vec = atoi(v[8]);
     r.depth = atoi(v[9]); r.replayed = atoi(v[10]);
+    r.mask = atoi(v[11]); r.crowded = atoi(v[12]);
+    r.padded = n * ((nx + 63) / 64 * 64) * ny;
     printf("%d", trt::two_steps_pay(r) ? 1 : 0);
 }
 """
@@ -33,8 +35,9 @@ def rule(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2312_10318_gb300", "csrc"),
                     str(d / "rule.cpp"), "-o", exe], check=True)
 
-    def call(nx, ny, n=1, mode="lagged", elem=4, general=0, ghosts=0, vec=0, depth=1, replayed=1):
-        return subprocess.run([exe, *(str(x) for x in (nx, ny, n, mode, elem, general, ghosts, vec, depth, replayed))],
+    def call(nx, ny, n=1, mode="lagged", elem=4, general=0, ghosts=0, vec=0, depth=1, replayed=1, mask=0, crowded=0):
+        return subprocess.run([exe, *(str(x) for x in (nx, ny, n, mode, elem, general, ghosts, vec, depth, replayed, mask,
+                                                       crowded))],
                               check=True, capture_output=True, text=True).stdout == "1"
     return call
 
@@ -53,6 +56,14 @@ def test_walls(rule):
     assert rule(512, 512, general=1, mode="off") and not rule(256, 256, general=1, mode="off")
     assert rule(32, 4096, 24, general=1, elem=4) and not rule(32, 4096, 24, general=1, elem=2)
     assert rule(32, 4096, 90, general=1, elem=2)
+
+
+def test_masks(rule):
+    kw = dict(general=1, mask=1)
+    assert not rule(1280, 1280, **kw) and rule(1536, 1536, **kw) and rule(100, 1024, 16, **kw)
+    assert rule(768, 768, mode="off", **kw) and not rule(128, 128, 40, mode="off", **kw)
+    assert rule(768, 768, crowded=1, **kw) and not rule(128, 128, 40, crowded=1, **kw)
+    assert rule(64, 64, ghosts=1, **kw)
 
 
 def test_current_phi(rule):
