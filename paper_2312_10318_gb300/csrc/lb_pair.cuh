@@ -24,7 +24,8 @@
 // pair_walk_general, which looks at one word per node.
 //
 // The same arithmetic in the same order as two single steps, each population
-// rounded to the storage type between them: the same bits.
+// rounded to the storage type between them: the same bits.  Which runs take it:
+// lb_pair_rule.h.
 //
 // Measured on GB300, us per step, single steps / this kernel: FP32 4096^2 227 /
 // 123, 1024^2 15.4 / 8.1; FP16 2048^2 42.1 / 27.4; whole solves, ms: creeping flow
