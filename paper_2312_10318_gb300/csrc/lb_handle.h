@@ -82,6 +82,7 @@ inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed
     r.current = s.g_mode == TRTRLB_G_CURRENT;
     r.off = s.g_mode == TRTRLB_G_OFF;
     const int width = r.current ? PAIR_AB_W : PAIR_W, together = shares_tma_launch(h) ? kTmaShare : kBatchStreams;
+    r.members = n;
     r.nodes += (long long)s.nx * s.ny;
     r.columns += (long long)pair_strips(s.nx, width) * width * s.ny;
     r.tiled += (long long)(s.nx + 31) / 32 * 32 * s.ny;
@@ -91,7 +92,6 @@ inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed
     r.crowded = (n == 1 || r.crowded) && s.crowded;
     r.mask = r.mask || s.mask != nullptr;
     r.padded += s.plane;
-    r.vec = s.vec;
     r.depth = (n + together - 1) / together;
     r.replayed = replayed;
 }

@@ -18,9 +18,10 @@ int main(int, char** v) {
     r.nodes = n * nx * ny;
     r.columns = n * ((nx + w - 1) / w * w) * ny;
     r.tiled = n * ((nx + 31) / 32 * 32) * ny;
-    r.elem = atoi(v[5]); r.general = atoi(v[6]); r.ghosts = atoi(v[7]); r.vec = atoi(v[8]);
-    r.depth = atoi(v[9]); r.replayed = atoi(v[10]);
-    r.mask = atoi(v[11]); r.crowded = atoi(v[12]);
+    r.elem = atoi(v[5]); r.general = atoi(v[6]); r.ghosts = atoi(v[7]);
+    r.depth = atoi(v[8]); r.replayed = atoi(v[9]);
+    r.mask = atoi(v[10]); r.crowded = atoi(v[11]);
+    r.members = (int)n;
     r.padded = n * ((nx + 63) / 64 * 64) * ny;
     printf("%d", trt::two_steps_pay(r) ? 1 : 0);
 }
@@ -35,16 +36,15 @@ def rule(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2312_10318_gb300", "csrc"),
                     str(d / "rule.cpp"), "-o", exe], check=True)
 
-    def call(nx, ny, n=1, mode="lagged", elem=4, general=0, ghosts=0, vec=0, depth=1, replayed=1, mask=0, crowded=0):
-        return subprocess.run([exe, *(str(x) for x in (nx, ny, n, mode, elem, general, ghosts, vec, depth, replayed, mask,
+    def call(nx, ny, n=1, mode="lagged", elem=4, general=0, ghosts=0, depth=1, replayed=1, mask=0, crowded=0):
+        return subprocess.run([exe, *(str(x) for x in (nx, ny, n, mode, elem, general, ghosts, depth, replayed, mask,
                                                        crowded))],
                               check=True, capture_output=True, text=True).stdout == "1"
     return call
 
 
 def test_periodic(rule):
-    assert rule(64, 64, vec=1) and rule(4096, 4096, 3)
-    assert not rule(250, 246) and not rule(33, 33, 40) and rule(250, 246, 8)
+    assert rule(64, 64) and rule(4096, 4096, 3) and rule(66, 64) and rule(66, 64, replayed=0)
 
 
 def test_walls(rule):
@@ -56,6 +56,12 @@ def test_walls(rule):
     assert rule(512, 512, general=1, mode="off") and not rule(256, 256, general=1, mode="off")
     assert rule(32, 4096, 24, general=1, elem=4) and not rule(32, 4096, 24, general=1, elem=2)
     assert rule(32, 4096, 90, general=1, elem=2)
+
+
+def test_several_lattices_launched_by_the_host(rule):
+    for kw in (dict(general=1), dict(general=1, mask=1), dict(general=1, mode="off")):
+        assert rule(130, 126, 8, replayed=0, **kw) and not rule(66, 64, 16, replayed=0, **kw)
+        assert not rule(130, 126, 4, replayed=0, **kw)
 
 
 def test_masks(rule):
