@@ -158,7 +158,7 @@ void choose_two_steps(const trtrlb_batch* b, std::vector<trt::State>& sim, bool 
             at.push_back(k);
             nodes += (long long)x.nx * x.ny;
         }
-        if (2 * nodes < all || trt::run_pays(m.data(), (int)m.size(), replayed)) continue;
+        if (2 * nodes < all || trt::run_pays(m.data(), (int)m.size(), replayed, true)) continue;
         for (size_t k : at) sim[k].pair = false;
     }
 }

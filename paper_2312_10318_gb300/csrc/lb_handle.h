@@ -77,7 +77,7 @@ constexpr int kBatchStreams = 6;  // a batch's own stream and those beside it
 
 // Adds lattice h, at state s, to the run r that it would share launches in (r of
 // n - 1 such lattices before: {} for n = 1).
-inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed) {
+inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed, bool batch) {
     const State& s = h->s;
     r.current = s.g_mode == TRTRLB_G_CURRENT;
     r.off = s.g_mode == TRTRLB_G_OFF;
@@ -94,6 +94,7 @@ inline void add_to_run(PairRun& r, const trtrlb_lattice* h, int n, bool replayed
     r.padded += s.plane;
     r.depth = (n + together - 1) / together;
     r.replayed = replayed;
+    r.batch = batch;
 }
 
 // Whether st is being captured into a caller's graph.
@@ -121,7 +122,7 @@ inline int64_t pair_launches(const State& s, int64_t n, bool even) {
 
 // Whether a run of the n lattices h, all of one format, flavour and G mode and all
 // able to, takes two steps per launch.
-bool run_pays(trtrlb_lattice* const* h, int n, bool replayed);
+bool run_pays(trtrlb_lattice* const* h, int n, bool replayed, bool batch);
 
 // Advances h by n time steps on st: two at a time from odd levels where the
 // two-step kernel runs the lattice.

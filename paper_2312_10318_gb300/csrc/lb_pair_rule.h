@@ -17,6 +17,7 @@ struct PairRun {
     long long padded;     // nodes with the rows' padding
     int depth;            // G_CURRENT: launches of a single step one after the other
     bool replayed;        // launches from a captured graph, not by the host one by one
+    bool batch;           // launches of a batch, not of one lattice's own steps
 };
 
 // Small launches of two steps last as long as one warp's walk: a band of two rows
@@ -45,9 +46,12 @@ struct PairRun {
 //    host (64^2 3.7 / 6.1, 512^2 6.9 / 8.2); replayed, FP32 512^2 7.0 / 6.0, 640^2 8.4 /
 //    8.3, 16-bit 640^2 8.6 / 7.2, 768^2 9.3 / 10.9, and 40 lattices of 64^2, which take
 //    three launches one after the other, 7.1 / 11.4.
-//  - several lattices whose launches the host makes one by one: their arguments (up to
-//    26 KB a launch) take it longer, more than 4 of them above all: with walls FP32 8
-//    lattices of 130 x 126 4.8 / 5.1, 16 of 66 x 64 4.7 / 3.7.
+//  - launches that the host makes one by one for a batch: its kernel of single steps,
+//    which looks the lattice up, takes 0.7 us longer than a lattice's own (one of 510 x
+//    512 with walls FP16 5.2 / 5.2, alone 5.2 / 4.4; a whole solve of 248 x 1518 BF16, 16
+//    steps, 71 / 86 us), and the arguments of more than 4 lattices (up to 26 KB a launch)
+//    longer still: with walls FP32 8 lattices of 130 x 126 4.8 / 5.1, 16 of 66 x 64 4.7 /
+//    3.7.
 inline bool two_steps_pay(const PairRun& r) {
     if (r.current) return !r.replayed || r.depth >= 2 || r.tiled >= (r.elem == 4 ? 400000 : 500000);
     if (!r.general) return true;
@@ -55,7 +59,7 @@ inline bool two_steps_pay(const PairRun& r) {
     const double share = (double)r.nodes / (double)r.columns;
     if (!r.replayed && r.members > 4) return (double)r.nodes * share * share >= 40e3;
     if (r.mask && !r.crowded && !r.off) return r.padded >= 1900000;
-    const double least = share < 0.6 ? (r.elem == 4 ? 800e3 : 3e6) : (r.off && !r.mask ? 160e3 : 400e3);
+    const double least = share < 0.6 ? (r.elem == 4 ? 800e3 : 3e6) : (r.off && !r.mask ? 160e3 : (r.batch && !r.replayed ? 230e3 : 400e3));
     return (double)r.nodes * share * share >= least;
 }
 

@@ -985,7 +985,7 @@ int trtrlb_two_step_run(const trtrlb_t* lattices, int32_t count, int32_t replaye
         std::lock_guard<std::mutex> lk(h->spare_mu);
         all = all && h->s.pair;
     }
-    *on = all && trt::run_pays(l.data(), count, replayed != 0) ? 1 : 0;
+    *on = all && trt::run_pays(l.data(), count, replayed != 0, count > 1 || replayed != 0) ? 1 : 0;
     return TRTRLB_OK;
 }
 
@@ -1038,11 +1038,11 @@ static T* at(T* const* a, int k) {
     return a ? a[k] : nullptr;
 }
 
-bool run_pays(trtrlb_lattice* const* h, int n, bool replayed) {
+bool run_pays(trtrlb_lattice* const* h, int n, bool replayed, bool batch) {
     PairRun r{};
     for (int k = 0; k < n; ++k) {
         if (h[k]->two_step == TwoStep::ALWAYS) return true;
-        add_to_run(r, h[k], k + 1, replayed);
+        add_to_run(r, h[k], k + 1, replayed, batch);
     }
     return two_steps_pay(r);
 }
@@ -1055,7 +1055,7 @@ cudaError_t advance(trtrlb_lattice* h, int64_t n, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         h->captured = h->captured || replayed;
     }
-    int64_t pairs = run_pays(&h, 1, replayed) ? pair_launches(h->s, n, h->captured) : 0;
+    int64_t pairs = run_pays(&h, 1, replayed, false) ? pair_launches(h->s, n, h->captured) : 0;
     while (n > 0) {
         cudaError_t e;
         int k = 1;

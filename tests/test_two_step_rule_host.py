@@ -20,7 +20,7 @@ int main(int, char** v) {
     r.tiled = n * ((nx + 31) / 32 * 32) * ny;
     r.elem = atoi(v[5]); r.general = atoi(v[6]); r.ghosts = atoi(v[7]);
     r.depth = atoi(v[8]); r.replayed = atoi(v[9]);
-    r.mask = atoi(v[10]); r.crowded = atoi(v[11]);
+    r.mask = atoi(v[10]); r.crowded = atoi(v[11]); r.batch = atoi(v[12]);
     r.members = (int)n;
     r.padded = n * ((nx + 63) / 64 * 64) * ny;
     printf("%d", trt::two_steps_pay(r) ? 1 : 0);
@@ -36,9 +36,10 @@ def rule(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "paper_2312_10318_gb300", "csrc"),
                     str(d / "rule.cpp"), "-o", exe], check=True)
 
-    def call(nx, ny, n=1, mode="lagged", elem=4, general=0, ghosts=0, depth=1, replayed=1, mask=0, crowded=0):
+    def call(nx, ny, n=1, mode="lagged", elem=4, general=0, ghosts=0, depth=1, replayed=1, mask=0, crowded=0,
+             batch=0):
         return subprocess.run([exe, *(str(x) for x in (nx, ny, n, mode, elem, general, ghosts, depth, replayed, mask,
-                                                       crowded))],
+                                                       crowded, batch))],
                               check=True, capture_output=True, text=True).stdout == "1"
     return call
 
@@ -62,6 +63,11 @@ def test_several_lattices_launched_by_the_host(rule):
     for kw in (dict(general=1), dict(general=1, mask=1), dict(general=1, mode="off")):
         assert rule(130, 126, 8, replayed=0, **kw) and not rule(66, 64, 16, replayed=0, **kw)
         assert not rule(130, 126, 4, replayed=0, **kw)
+
+
+def test_one_walled_lattice_launched_by_the_host(rule):
+    assert rule(248, 1518, elem=2, general=1, replayed=0, batch=1)
+    assert not rule(248, 1518, elem=2, general=1, replayed=0) and not rule(382, 380, general=1, replayed=0, batch=1)
 
 
 def test_masks(rule):
